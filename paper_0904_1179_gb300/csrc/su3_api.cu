@@ -39,6 +39,8 @@ int su3_sync(su3_lattice* h, const char* what) {
     SU3_CUDA(cudaMemcpy(h->h_pstatus, h->d_pstatus, sizeof(int), cudaMemcpyDeviceToHost), what);
     if (*h->h_pstatus != 0) {
       SU3_CUDA(cudaMemset(h->d_pstatus, 0, sizeof(int)), what);
+      // links that the sweep did not reach keep whatever they held
+      SU3_CUDA(cudaMemset(su3dev::sweep_far(h->d_sweep), 1, sizeof(int)), what);
       return su3_fail(SU3_ETIMEOUT,
                       "%s: a sweep gave up waiting for tiles of the previous half-sweep (bounded wait of %.3f s); "
                       "the configuration is incomplete",
@@ -350,13 +352,16 @@ int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pa
   if (rc != SU3_OK) return rc;
   const long long V = 2LL * g.Vh;
   double* stage[2] = {h->d_stage, h->d_stage2};
+  // the conversion into the store flags links far from SU(3); a batch's other replicas keep theirs
+  if (!get && !h->batch)
+    SU3_CUDA(cudaMemsetAsync(su3dev::sweep_far(h->d_sweep), 0, 2 * sizeof(int), h->stream), what);
   int i = 0;
   for (long long s0 = 0; s0 < V; s0 += kChunkSites, ++i) {
     const long long n = (V - s0) < kChunkSites ? (V - s0) : kChunkSites;
     const int b = i & 1;
     cudaStream_t cs = h->copy_stream;
     const size_t bytes = (size_t)n * 72 * sizeof(double);
-    ConvArgs a{g, h->precision, s0, n, stage[b], links, pairs ? 1 : 0};
+    ConvArgs a{g, h->precision, s0, n, stage[b], links, pairs ? 1 : 0, su3dev::sweep_far(h->d_sweep)};
     if (get) {
       // stage[b] is free once the copy-out of chunk i-2 has finished
       if (i >= 2) SU3_CUDA(cudaStreamWaitEvent(h->stream, h->ev_copied[b], 0), what);
@@ -439,7 +444,7 @@ int su3_create_ex(int L0, int L1, int L2, int L3, double beta, uint64_t seed, in
   const int nparts = su3k_plaquette_blocks(h->geom);
   const long long chunk = V < kChunkSites ? V : kChunkSites;
   if ((e = cudaMalloc(&h->links, h->link_bytes)) != cudaSuccess ||
-      (e = cudaMalloc(&h->d_sweep, sizeof(uint64_t))) != cudaSuccess ||
+      (e = cudaMalloc(&h->d_sweep, sizeof(su3dev::SweepState))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_stats, 2 * sizeof(unsigned long long))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_partials, (size_t)nparts * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_plaq, sizeof(double))) != cudaSuccess ||
@@ -452,7 +457,7 @@ int su3_create_ex(int L0, int L1, int L2, int L3, double beta, uint64_t seed, in
     return rc;
   }
   int rc = SU3_OK;
-  if ((e = cudaMemsetAsync(h->d_sweep, 0, sizeof(uint64_t), h->stream)) != cudaSuccess ||
+  if ((e = cudaMemsetAsync(h->d_sweep, 0, sizeof(su3dev::SweepState), h->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(h->d_stats, 0, 2 * sizeof(unsigned long long), h->stream)) != cudaSuccess) {
     rc = cuda_fail(e, "su3_create: memset");
   }
@@ -651,7 +656,7 @@ int su3_bounds_status(unsigned int* status, int clear) {
   if (!status) return fail(SU3_EINVAL, "su3_bounds_status: NULL status");
   *status = 0u;
 #ifdef SU3_BOUNDS_CHECK
-  cudaError_t (*const tus[4])(unsigned int*, bool) = {su3k_bounds_status_kernels, su3k_bounds_status_pair,
+  cudaError_t (*const tus[5])(unsigned int*, bool) = {su3k_bounds_status_kernels, su3k_bounds_status_f64, su3k_bounds_status_pair,
                                                         su3k_bounds_status_batch, su3k_bounds_status_decomp};
   for (auto f : tus) {
     unsigned int v = 0u;

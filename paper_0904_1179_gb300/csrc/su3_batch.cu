@@ -72,15 +72,17 @@ struct BatchArgs {
   long long wait_ns;
   int withhold_item;  // fault-injection hook: this item never signals completion (-1: none)
   int max_tries;      // SU(2) proposals per subgroup (1: one-hit heatbath)
+  int mu;             // direction of this launch (the FP64 kernels take it from here)
 };
 
 // The update of link (h, MU) of a replica: one direction per launch (the
 // sweep's four launches each run one direction's code).
 template <typename T, bool EFT, bool REPEAT, int MU>
-__device__ __forceinline__ void update_item(const ReplicaDesc& rd, void* links, int h, int p, uint64_t t, int max_tries) {
-  const UpdateConsts uc{rd.three_over_beta_f64, rd.three_over_beta, max_tries};
+__device__ __forceinline__ void update_item(const ReplicaDesc& rd, void* links, int h, int p, int mu, uint64_t t,
+                                            int max_tries, int* far) {
+  const UpdateConsts uc{rd.three_over_beta_f64, rd.three_over_beta, max_tries, far};
   if constexpr (std::is_same<T, double>::value)
-    update_link_f64<MU, true, REPEAT>(rd.g, (double2*)links + rd.offset, h, p, t, rd.key, uc);
+    update_link_f64<true, REPEAT>(rd.g, (double2*)links + rd.offset, h, p, mu, t, rd.key, uc);
   else
     update_link_f32<MU, true, EFT, REPEAT>(rd.g, (float4*)links + rd.offset, h, p, t, rd.key, uc);
 }
@@ -160,7 +162,7 @@ __device__ __forceinline__ void batch_item(const BatchArgs& a, const ReplicaDesc
   if (s_stop) return;
   const ReplicaDesc& rd = PARAM ? reps[it.x] : s_rep;
   const int h = it.z * (int)blockDim.x + (int)threadIdx.x;
-  if (h < rd.g.Vh) update_item<T, EFT, REPEAT, MU>(rd, a.links, h, it.y & 1, t, a.max_tries);
+  if (h < rd.g.Vh) update_item<T, EFT, REPEAT, MU>(rd, a.links, h, it.y & 1, a.mu, t, a.max_tries, sweep_far(a.sweep));
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -195,8 +197,11 @@ cudaError_t launch_mu(const BatchArgs& a, const ParamReplicas* pr, int threads, 
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = MU > 0 ? 1 : 0;
-  return pr ? cudaLaunchKernelEx(&cfg, k_batch_sweep_c<T, EFT, REPEAT, MU>, a, *pr)
-            : cudaLaunchKernelEx(&cfg, k_batch_sweep<T, EFT, REPEAT, MU>, a);
+  BatchArgs b = a;
+  b.mu = MU;
+  constexpr int kMu = std::is_same<T, double>::value ? 0 : MU;  // one FP64 kernel for the four directions
+  return pr ? cudaLaunchKernelEx(&cfg, k_batch_sweep_c<T, EFT, REPEAT, kMu>, b, *pr)
+            : cudaLaunchKernelEx(&cfg, k_batch_sweep<T, EFT, REPEAT, kMu>, b);
 }
 
 template <typename T, bool EFT, bool REPEAT>
@@ -421,6 +426,8 @@ int check_status(su3_lattice* h, const char* what) {
   SU3_CUDA(cudaMemcpy(b->h_status, b->d_status, sizeof(int), cudaMemcpyDeviceToHost), what);
   if (*b->h_status != 0) {
     SU3_CUDA(cudaMemset(b->d_status, 0, sizeof(int)), what);
+    // links that the sweep did not reach keep whatever they held
+    SU3_CUDA(cudaMemset(sweep_far(h->d_sweep), 1, sizeof(int)), what);
     return su3_fail(SU3_ETIMEOUT,
                     "%s: a batched sweep gave up waiting for a phase to complete (bounded wait of %.3f s); the "
                     "configuration of that sweep is incomplete",
@@ -511,7 +518,7 @@ int su3_batch_create(int n, const int (*dims)[4], const double* betas, const uin
   gmax.Vh = (int)(vmax / 2);
   const long long chunk = vmax < kChunkSites ? vmax : kChunkSites;
   if ((e = cudaMalloc(&h->links, h->link_bytes)) != cudaSuccess ||
-      (e = cudaMalloc(&h->d_sweep, sizeof(uint64_t))) != cudaSuccess ||
+      (e = cudaMalloc(&h->d_sweep, sizeof(SweepState))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_stats, 2 * sizeof(unsigned long long))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_partials, (size_t)su3k_plaquette_blocks(gmax) * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_stage, (size_t)chunk * 72 * sizeof(double))) != cudaSuccess ||
@@ -527,7 +534,7 @@ int su3_batch_create(int n, const int (*dims)[4], const double* betas, const uin
     return rc;
   }
   int rc = SU3_OK;
-  if ((e = cudaMemsetAsync(h->d_sweep, 0, sizeof(uint64_t), h->stream)) != cudaSuccess ||
+  if ((e = cudaMemsetAsync(h->d_sweep, 0, sizeof(SweepState), h->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(b->d_status, 0, sizeof(int), h->stream)) != cudaSuccess)
     rc = su3_cuda_fail(e, "su3_batch_create: memset");
   for (int r = 0; r < n && rc == SU3_OK; ++r) {
@@ -634,6 +641,8 @@ int su3_batch_autotune(su3_handle h, int* threads, int* blocks_per_sm, int* wind
   SU3_CUDA(cudaMalloc(&saved, h->link_bytes), "su3_batch_autotune: save buffer");
   cudaError_t e = cudaMemcpyAsync(saved, h->links, h->link_bytes, cudaMemcpyDeviceToDevice, h->stream);
   const uint64_t count = h->sweep_host;
+  int far[2] = {0, 0};
+  if (e == cudaSuccess) e = cudaMemcpyAsync(far, sweep_far(h->d_sweep), sizeof far, cudaMemcpyDeviceToHost, h->stream);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
@@ -682,6 +691,7 @@ int su3_batch_autotune(su3_handle h, int* threads, int* blocks_per_sm, int* wind
   if (rc == SU3_OK) {
     e = cudaMemcpyAsync(h->links, saved, h->link_bytes, cudaMemcpyDeviceToDevice, h->stream);
     if (e == cudaSuccess) e = su3k_launch_set_counter(h->d_sweep, count, h->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(sweep_far(h->d_sweep), far, sizeof far, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) rc = su3_cuda_fail(e, "su3_batch_autotune: restore");
     h->sweep_host = count;

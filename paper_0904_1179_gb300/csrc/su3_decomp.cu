@@ -102,17 +102,17 @@ __device__ __forceinline__ void block_partial_d(double v, double* out) {
 // MEAS: the fused plaquette of the odd-site phases of mu = 1, 2, 3, as in the
 // undivided kernels (every link of A_< is final; the ghosts were refreshed by
 // the exchanges after the phases before).
-template <int MU, bool REPEAT, bool MEAS>
-__global__ void __launch_bounds__(kMaxSweepThreads) k_decomp_half_sweep_f64(DecompArgs a) {
+template <bool REPEAT, bool MEAS>
+__global__ void __launch_bounds__(kMaxSweepThreads) k_decomp_half_sweep_f64(DecompArgs a, int mu) {
   const int k = blockIdx.y;
   const SubGeometry g = sub_geometry(a.g, a.nf, a.ndmpi, k);
   const int h = blockIdx.x * blockDim.x + threadIdx.x;
   UpdateCount c{0, 0};
   double m = 0.0;
   if (h < g.in.Vh) {
-    const UpdateConsts uc{a.three_over_beta_f64, a.three_over_beta, a.max_tries};
+    const UpdateConsts uc{a.three_over_beta_f64, a.three_over_beta, a.max_tries, sweep_far(a.sweep)};
     double2* U = (double2*)a.subs + (size_t)k * a.sub_elems;
-    c = update_link_f64<MU, false, REPEAT, MEAS>(g, U, h, a.parity, *a.sweep, a.key, uc, &m);
+    c = update_link_f64<false, REPEAT, MEAS>(g, U, h, a.parity, mu, *a.sweep, a.key, uc, &m);
   }
   if (a.count_stats) count_stats_d(c, a.stats);
   if (MEAS) block_partial_d(m, a.meas);
@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(kMaxSweepThreads, 4) k_decomp_half_sweep_f32(D
   UpdateCount c{0, 0};
   double m = 0.0;
   if (h < g.in.Vh) {
-    const UpdateConsts uc{a.three_over_beta_f64, a.three_over_beta, a.max_tries};
+    const UpdateConsts uc{a.three_over_beta_f64, a.three_over_beta, a.max_tries, sweep_far(a.sweep)};
     float4* U = (float4*)a.subs + (size_t)k * a.sub_elems;
     c = update_link_f32<MU, false, EFT, REPEAT, MEAS>(g, U, h, a.parity, *a.sweep, a.key, uc, &m);
   }
@@ -214,7 +214,7 @@ __global__ void k_decomp_move_f32_pairs(SubGeometry base, int nf, int ndmpi, flo
 template <int MU, bool REPEAT, bool MEAS>
 cudaError_t launch_update_form(const DecompArgs& a, int precision, const dim3& grid, int threads, cudaStream_t s) {
   if (precision == SU3_FP64)
-    k_decomp_half_sweep_f64<MU, REPEAT, MEAS><<<grid, threads, 0, s>>>(a);
+    k_decomp_half_sweep_f64<REPEAT, MEAS><<<grid, threads, 0, s>>>(a, MU);
   else if (precision == SU3_FP32_EFT)
     k_decomp_half_sweep_f32<MU, true, REPEAT, MEAS><<<grid, threads, 0, s>>>(a);
   else

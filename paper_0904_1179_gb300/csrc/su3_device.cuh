@@ -391,8 +391,8 @@ __host__ __device__ __forceinline__ int nb_half(const Geometry& g, const Site& s
 
 __device__ __forceinline__ int wrap_coord(int x, int L) { return x < 0 ? x + L : (x >= L ? x - L : x); }
 
-// nb_half and nb_half2 for a direction known only at run time (it differs
-// between the lanes that share one link update): selects, no indexed arrays.
+// nb_half and nb_half2 for a direction known only at run time: selects, no
+// indexed arrays.
 __device__ __forceinline__ int nb_half_rt(const Geometry& g, const Site& s, int nu, int d) {
   const int x0 = nu == 0 ? wrap_coord(s.x0 + d, g.L0) : s.x0;
   const int x1 = nu == 1 ? wrap_coord(s.x1 + d, g.L1) : s.x1;
@@ -488,6 +488,19 @@ __device__ __forceinline__ int nb_half2(const SubGeometry& g, const SubSite& s, 
   y[nu] = sub_step(g, y[nu], nu, +1);
   y[rho] = sub_step(g, y[rho], rho, -1);
   return sub_half(g, y[0], y[1], y[2], y[3]);
+}
+
+// The same for directions known only at run time (no indexed arrays).
+__device__ __forceinline__ int nb_half_rt(const SubGeometry& g, const SubSite& s, int nu, int d) {
+  return sub_half(g, nu == 0 ? sub_step(g, s.y0, 0, d) : s.y0, nu == 1 ? sub_step(g, s.y1, 1, d) : s.y1,
+                  nu == 2 ? sub_step(g, s.y2, 2, d) : s.y2, nu == 3 ? sub_step(g, s.y3, 3, d) : s.y3);
+}
+
+__device__ __forceinline__ int nb_half2_rt(const SubGeometry& g, const SubSite& s, int nu, int rho) {
+  const int d0 = (nu == 0) - (rho == 0), d1 = (nu == 1) - (rho == 1), d2 = (nu == 2) - (rho == 2),
+            d3 = (nu == 3) - (rho == 3);
+  return sub_half(g, d0 ? sub_step(g, s.y0, 0, d0) : s.y0, d1 ? sub_step(g, s.y1, 1, d1) : s.y1,
+                  d2 ? sub_step(g, s.y2, 2, d2) : s.y2, d3 ? sub_step(g, s.y3, 3, d3) : s.y3);
 }
 
 // ---------------------------------------------------------------------------
@@ -668,6 +681,39 @@ __device__ __forceinline__ void gram_schmidt_rows01(cx<double> r0[3], cx<double>
   const double i1 = rsqrt(n1);
 #pragma unroll
   for (int k = 0; k < 3; ++k) r1[k] = mk(r1[k].re * i1, r1[k].im * i1);
+}
+
+// Device words of a handle that its sweep kernels read: the sweep index (the
+// RNG position) and two flags of the FP64 store.  far: a link may be far from
+// SU(3) -- as links_set found it, or as an update left it (NaN) --, so updates
+// run in FP64 arithmetic throughout; otherwise they run in that of su3_fx.cuh,
+// whose range and reunitarisation assume near-unitary links.  far_next: an
+// FP64 update of this sweep left such a link.  Every link has been rewritten
+// by the end of a sweep, so the counter's increment moves far_next to far.
+struct SweepState {
+  uint64_t t;
+  int far, far_next;
+};
+__host__ __device__ __forceinline__ int* sweep_far(const uint64_t* sweep) {
+  return &((SweepState*)sweep)->far;
+}
+
+// Whether a link's rows 0, 1 are orthonormal and its row 2 is their completion
+// to 2^-10 (false for NaN and infinities).
+__device__ __forceinline__ bool far_from_su3(const mat3<double>& m) {
+  double n0 = 0.0, n1 = 0.0, off = 0.0;
+  cx<double> d = mk(0.0, 0.0);
+  mat3<double> c = m;
+  complete_row2(c);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    n0 = fma(m.e[0][k].re, m.e[0][k].re, fma(m.e[0][k].im, m.e[0][k].im, n0));
+    n1 = fma(m.e[1][k].re, m.e[1][k].re, fma(m.e[1][k].im, m.e[1][k].im, n1));
+    d = mac_ca(d, m.e[0][k], m.e[1][k]);
+    off += fabs(c.e[2][k].re - m.e[2][k].re) + fabs(c.e[2][k].im - m.e[2][k].im);
+  }
+  constexpr double tol = 0x1p-10;
+  return !(fabs(n0 - 1.0) < tol && fabs(n1 - 1.0) < tol && fabs(d.re) < tol && fabs(d.im) < tol && off < tol);
 }
 
 // ---------------------------------------------------------------------------

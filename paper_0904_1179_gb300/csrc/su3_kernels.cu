@@ -8,12 +8,13 @@
 // Abstract and Sec. 1 of Berg & Wu, arXiv:0904.1179), so threads are
 // independent; the counter-based Philox stream makes the result independent of
 // the launch configuration.  The work is a 4D stencil of 3x3 complex products,
-// not a dense contraction, so it runs on the FP32/FP64 CUDA cores.
+// not a dense contraction, so it runs on the CUDA cores.  The FP64 store's
+// half-sweeps are in su3_kernels_f64.cu.
 #include "su3_kernels.h"
 
 #include "su3_device.cuh"
+#include "su3_reduce.cuh"
 #include "su3_sitepair.cuh"
-#include "su3_sweepq.cuh"
 #include "su3_update.cuh"
 
 using namespace su3dev;
@@ -33,148 +34,6 @@ namespace {
 // ---------------------------------------------------------------------------
 // Single-lattice half-sweeps: one thread per link of (mu, parity).
 // ---------------------------------------------------------------------------
-template <bool STATS>
-__device__ __forceinline__ void count_stats(UpdateCount c, unsigned long long* stats) {
-  if (STATS) {
-    const int acc = __reduce_add_sync(0xffffffffu, c.accepted);
-    const int prop = __reduce_add_sync(0xffffffffu, c.proposed);
-    if ((threadIdx.x & 31) == 0) {
-      atomicAdd(&stats[0], (unsigned long long)acc);
-      atomicAdd(&stats[1], (unsigned long long)prop);
-    }
-  }
-}
-
-// Block sum of one value per thread into out[blockIdx.x] (fixed order).
-__device__ __forceinline__ void block_partial(double v, double* out) {
-  __shared__ double red[32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double w = threadIdx.x < (blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    if (threadIdx.x == 0) out[blockIdx.x] = w;
-  }
-}
-
-template <int MU, bool STATS, bool REPEAT, bool MEAS>
-__global__ void __launch_bounds__(kMaxSweepThreads) k_half_sweep_f64(HalfSweepArgs args) {
-  const int h = blockIdx.x * blockDim.x + threadIdx.x;
-  UpdateCount c{0, 0};
-  double m = 0.0;
-  if (h < args.geom.Vh) {
-    const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, args.max_tries};
-    c = update_link_f64<MU, false, REPEAT, MEAS>(args.geom, (double2*)args.links, h, args.parity, *args.sweep, args.key,
-                                                 uc, &m);
-  }
-  count_stats<STATS>(c, args.stats);
-  if (MEAS) block_partial(m, args.meas);
-}
-
-// The FP64 sweep as four persistent launches, one per direction MU with its
-// even and odd half-sweeps, chained by programmatic dependent launch
-// (su3_sweepq.cuh): a block takes a tile of `threads` sites of one parity in
-// one x3 layer of the lattice and waits only for the layers of the previous
-// half-sweep that its staples read, so one half-sweep's last wave overlaps
-// the next one's first and only one launch tail per sweep remains.  The
-// links change while the launch runs, so they are read through L2 (CG); the
-// update is that of k_half_sweep_f64, bit for bit.
-template <int MU, bool REPEAT>
-__global__ void __launch_bounds__(kMaxSweepThreads)
-    k_sweep_f64(HalfSweepArgs args, SweepQueue qa, int tiles_per_layer, int layers, int stats) {
-  __shared__ SweepItem s_item;
-  signal_dependents();
-  take_sweep_item<2, 2 * MU>(qa, MU, tiles_per_layer, layers, &s_item);
-  __syncthreads();
-  const SweepItem it = s_item;
-  if (it.phase < 0) return;
-  const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, args.max_tries};
-  const int h = it.tile * (int)blockDim.x + (int)threadIdx.x;  // layers are whole tiles: always a site of the lattice
-  const UpdateCount c =
-      update_link_f64<MU, true, REPEAT, false>(args.geom, (double2*)args.links, h, it.phase & 1, *args.sweep, args.key, uc);
-  if (stats) count_stats<true>(c, args.stats);
-  report_sweep_item(qa, layers, it);
-}
-
-// One FP64 half-sweep (phase 2 MU + parity) of the chained sweep: one block
-// per tile of sites of one x3 layer, the tile from the block's index
-// (su3_sweepq.cuh), waiting only for the layers of the previous launch's
-// half-sweep that its staples read.
-template <int MU, bool REPEAT>
-__global__ void __launch_bounds__(kMaxSweepThreads)
-    k_half_sweep_f64_chain(HalfSweepArgs args, SweepQueue qa, int tiles_per_layer, int layers, int stats, int parity) {
-  __shared__ SweepItem s_item;
-  signal_dependents();
-  own_sweep_item(qa, 2 * MU + parity, tiles_per_layer, layers, &s_item);
-  __syncthreads();
-  const SweepItem it = s_item;
-  if (it.phase < 0) return;
-  const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, args.max_tries};
-  const int h = it.tile * (int)blockDim.x + (int)threadIdx.x;  // layers are whole tiles: always a site of the lattice
-  const UpdateCount c =
-      update_link_f64<MU, true, REPEAT, false>(args.geom, (double2*)args.links, h, parity, *args.sweep, args.key, uc);
-  if (stats) count_stats<true>(c, args.stats);
-  report_sweep_item(qa, layers, it);
-}
-
-// A small lattice's half-sweep has too few links to fill the GPU, and each
-// link's FP64 update is a long dependent chain: the time is its latency.
-// Here four lanes share one link: lanes 0, 1, 2 compute rows 0,1 of the two
-// staple paths of the first, second and third direction nu != MU at the same
-// time, lane 0 gathers them and adds them up in the single-thread order
-// (forward then backward path, nu ascending, row 2 formed in the
-// accumulation), so the staple, and everything after it, is bit for bit that
-// of k_half_sweep_f64.  Lane 3 only idles.
-__device__ __forceinline__ mat3<double> shfl_rows01(const mat3<double>& m, int src) {
-  mat3<double> r;
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      r.e[i][k].re = __shfl_sync(0xffffffffu, m.e[i][k].re, src);
-      r.e[i][k].im = __shfl_sync(0xffffffffu, m.e[i][k].im, src);
-    }
-  return r;
-}
-
-template <int MU, bool STATS>
-__global__ void __launch_bounds__(kMaxSweepThreads) k_half_sweep_f64_split(HalfSweepArgs args) {
-  const Geometry& g = args.geom;
-  const int p = args.parity;
-  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int link = gid >> 2, part = gid & 3;
-  const bool active = link < g.Vh;
-  const int h = active ? link : 0;  // a group past the end works on site 0 and discards it (shuffles stay converged)
-  const Site st = site_of(g, h, p);
-  double2* U = (double2*)args.links;
-  mat3<double> F = zero3<double>(), B = zero3<double>();
-  if (part < 3) {
-    const int nu = part < MU ? part : part + 1;
-    const int h_pmu = nb_half(g, st, MU, +1);
-    F = forward_path<double, false>(g, U, st, h, p, MU, nu, h_pmu, nb_half_rt(g, st, nu, +1));
-    B = backward_path<double, false>(g, U, p, MU, nu, nb_half_rt(g, st, nu, -1), nb_half2_rt(g, st, MU, nu));
-  }
-  const int lane0 = (threadIdx.x & 31) & ~3;
-  mat3<double> A;
-  init_completed(A, F);
-  acc_completed(A, B);
-#pragma unroll
-  for (int k = 1; k < 3; ++k) {
-    acc_completed(A, shfl_rows01(F, lane0 + k));
-    acc_completed(A, shfl_rows01(B, lane0 + k));
-  }
-  UpdateCount c{0, 0};
-  if (part == 0 && active) {
-    const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, 1};
-    c = heatbath_f64<MU, false, false, false>(g, U, h, p, *args.sweep, (uint32_t)canon(g, st), args.key, uc, A, A,
-                                             nullptr);
-  }
-  count_stats<STATS>(c, args.stats);
-}
-
 // The same four-lane split for FP32 storage: rows 0,1 of the staple paths on
 // row pairs (12 floats each) are gathered into lane 0 and added in the
 // single-thread order; no register cap (small lattices leave the SMs nearly
@@ -219,7 +78,7 @@ __global__ void __launch_bounds__(kMaxSweepThreads) k_half_sweep_f32_split(HalfS
   }
   UpdateCount c{0, 0};
   if (part == 0 && active) {
-    const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, 1};
+    const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, 1, sweep_far(args.sweep)};
     c = heatbath_f32_on<MU, EFT, false, false, PAIRS>(g, U, h, p, *args.sweep, (uint32_t)canon(g, st), args.key, uc, A,
                                                        A, nullptr, load_pm3_l<false, PAIRS>(U, MU, p, h, g.Vh), true);
   }
@@ -232,7 +91,7 @@ __global__ void __launch_bounds__(SU3_F32_LB_THREADS, SU3_F32_MINBLOCKS) k_half_
   UpdateCount c{0, 0};
   double m = 0.0;
   if (h < args.geom.Vh) {
-    const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, args.max_tries};
+    const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, args.max_tries, sweep_far(args.sweep)};
     c = update_link_f32<MU, false, EFT, REPEAT, MEAS>(args.geom, (float4*)args.links, h, args.parity, *args.sweep,
                                                       args.key, uc, &m);
   }
@@ -240,7 +99,12 @@ __global__ void __launch_bounds__(SU3_F32_LB_THREADS, SU3_F32_MINBLOCKS) k_half_
   if (MEAS) block_partial(m, args.meas);
 }
 
-__global__ void k_increment(uint64_t* counter, uint64_t n) { *counter += n; }
+__global__ void k_increment(uint64_t* counter, uint64_t n) {
+  *counter += n;
+  int* far = sweep_far(counter);
+  far[0] = far[1];
+  far[1] = 0;
+}
 
 __global__ void __launch_bounds__(1024) k_meas_final(const double* parts, int n, double scale, const uint64_t* sweep,
                                                      double* out, int cap) {
@@ -444,6 +308,7 @@ __global__ void k_canon_to_store(ConvArgs args) {
     mat3<double> m;
 #pragma unroll
     for (int c = 0; c < 9; ++c) m.e[c / 3][c % 3] = mk(src[2 * c], src[2 * c + 1]);
+    if (far_from_su3(m)) *(volatile int*)args.far = 1;
     store_f64((double2*)args.links, mu, p, h, g.Vh, m);
   } else {
     float o[12];
@@ -508,56 +373,6 @@ __global__ void k_store_to_canon(ConvArgs args) {
 // ---------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------
-template <int MU, bool REPEAT>
-static cudaError_t launch_chain_f64_mu(const HalfSweepArgs& a, const SweepQueue& q, int tpl, int layers, int st,
-                                       int threads, cudaStream_t s) {
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(tpl * layers);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  for (int p = 0; p < 2; ++p) {
-    cfg.numAttrs = MU == 0 && p == 0 ? 0 : 1;
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, k_half_sweep_f64_chain<MU, REPEAT>, a, q, tpl, layers, st, p);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
-template <bool REPEAT>
-static cudaError_t launch_sweep_f64(const HalfSweepArgs& a, const SweepQueue& q, int tpl, int layers, bool stats,
-                                    int threads, bool chained, cudaStream_t s) {
-  const int blocks = 2 * tpl * layers, st = stats ? 1 : 0;
-  if (chained) {
-    cudaError_t e;
-    if ((e = launch_chain_f64_mu<0, REPEAT>(a, q, tpl, layers, st, threads, s)) != cudaSuccess) return e;
-    if ((e = launch_chain_f64_mu<1, REPEAT>(a, q, tpl, layers, st, threads, s)) != cudaSuccess) return e;
-    if ((e = launch_chain_f64_mu<2, REPEAT>(a, q, tpl, layers, st, threads, s)) != cudaSuccess) return e;
-    return launch_chain_f64_mu<3, REPEAT>(a, q, tpl, layers, st, threads, s);
-  }
-  k_sweep_f64<0, REPEAT><<<blocks, threads, 0, s>>>(a, q, tpl, layers, st);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // directions 1-3: programmatic dependent launches (su3_sweepq.cuh)
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = s;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  if ((e = cudaLaunchKernelEx(&cfg, k_sweep_f64<1, REPEAT>, a, q, tpl, layers, st)) != cudaSuccess) return e;
-  if ((e = cudaLaunchKernelEx(&cfg, k_sweep_f64<2, REPEAT>, a, q, tpl, layers, st)) != cudaSuccess) return e;
-  return cudaLaunchKernelEx(&cfg, k_sweep_f64<3, REPEAT>, a, q, tpl, layers, st);
-}
-
 template <int MU, bool STATS, bool EFT, bool REPEAT, bool MEAS>
 static cudaError_t launch_f32(const HalfSweepArgs& a, int blocks, int threads, cudaStream_t s) {
   k_half_sweep_f32<MU, STATS, EFT, REPEAT, MEAS><<<blocks, threads, 0, s>>>(a);
@@ -566,10 +381,6 @@ static cudaError_t launch_f32(const HalfSweepArgs& a, int blocks, int threads, c
 
 template <int MU, bool STATS, bool REPEAT, bool MEAS>
 static cudaError_t launch_prec(const HalfSweepArgs& a, int precision, int blocks, int threads, cudaStream_t s) {
-  if (precision == 0) {
-    k_half_sweep_f64<MU, STATS, REPEAT, MEAS><<<blocks, threads, 0, s>>>(a);
-    return cudaGetLastError();
-  }
   if (precision == 2) return launch_f32<MU, STATS, true, REPEAT, MEAS>(a, blocks, threads, s);
   return launch_f32<MU, STATS, false, REPEAT, MEAS>(a, blocks, threads, s);
 }
@@ -596,12 +407,7 @@ static cudaError_t launch_half_sweep_mu(const HalfSweepArgs& a, int precision, b
   }
   if (a.split && !repeat) {
     const int sblocks = (4 * a.geom.Vh + threads - 1) / threads;
-    if (precision == 0) {
-      if (stats)
-        k_half_sweep_f64_split<MU, true><<<sblocks, threads, 0, s>>>(a);
-      else
-        k_half_sweep_f64_split<MU, false><<<sblocks, threads, 0, s>>>(a);
-    } else if (precision == 2) {
+    if (precision == 2) {
       if (stats)
         launch_f32_split<MU, true, true>(a, sblocks, threads, s);
       else
@@ -621,23 +427,8 @@ static cudaError_t launch_half_sweep_mu(const HalfSweepArgs& a, int precision, b
                 : launch_prec<MU, false, false, false>(a, precision, blocks, threads, s);
 }
 
-int su3k_f64_sweep_layers(const Geometry& g, int threads, int* tiles_per_layer) {
-  const long long per_layer = (long long)g.hL0 * g.L1 * g.L2;  // sites of one parity in one x3 layer
-  if (threads <= 0 || threads > kMaxSweepThreads || per_layer % threads != 0 || g.L3 < 4) return 0;
-  *tiles_per_layer = (int)(per_layer / threads);
-  return g.L3;
-}
-
-cudaError_t su3k_launch_sweep_f64(const HalfSweepArgs& a, const SweepQueue& q, bool stats, int threads, bool chained,
-                                  cudaStream_t s) {
-  int tpl = 0;
-  const int layers = su3k_f64_sweep_layers(a.geom, threads, &tpl);
-  if (layers == 0 || a.meas || a.split) return cudaErrorInvalidValue;
-  return a.max_tries > 1 ? launch_sweep_f64<true>(a, q, tpl, layers, stats, threads, chained, s)
-                         : launch_sweep_f64<false>(a, q, tpl, layers, stats, threads, chained, s);
-}
-
 cudaError_t su3k_launch_half_sweep(const HalfSweepArgs& a, int mu, int precision, bool stats, int threads, cudaStream_t s) {
+  if (precision == 0) return su3k_launch_half_sweep_f64(a, mu, stats, threads, s);
   switch (mu) {
     case 0: return launch_half_sweep_mu<0>(a, precision, stats, threads, s);
     case 1: return launch_half_sweep_mu<1>(a, precision, stats, threads, s);

@@ -50,12 +50,15 @@ struct ConvArgs {
   double* canon;  // device staging buffer, canonical layout of the chunk
   void* links;
   int pairs;  // FP32 store in the site-paired layout
+  int* far;   // SweepState's flag, set where the FP64 store takes a link far from SU(3)
 };
 
 // Whether an FP32 store of an L0 x L1 x L2 x L3 lattice uses the site-paired
 // layout (su3_sitepair.cuh): L3 a multiple of 4.
 inline bool su3_fp32_pairs(int L3) { return L3 % 4 == 0; }
 
+// The same for the FP64 store (su3_kernels_f64.cu).
+cudaError_t su3k_launch_half_sweep_f64(const HalfSweepArgs& a, int mu, bool stats, int threads, cudaStream_t s);
 cudaError_t su3k_launch_half_sweep(const HalfSweepArgs& a, int mu, int precision, bool stats, int threads, cudaStream_t s);
 // Blocks of one half-sweep launch (the partial sums of the fused plaquette
 // come one per block).
@@ -77,7 +80,7 @@ cudaError_t su3k_prepare();
 // of phase q starts once phase q-1 has finished the x3 layers its staples
 // reach (its own layer and the two beside it).  Site-paired FP32
 // (su3_kernels_pair.cu): x3 layers of the pair lattice, tiles of `threads`
-// pairs; FP64 (su3_kernels.cu): x3 layers of the lattice, tiles of `threads`
+// pairs; FP64 (su3_kernels_f64.cu): x3 layers of the lattice, tiles of `threads`
 // sites of one parity.
 struct SweepQueue {
   unsigned int* counters;  // [0]: next work item of a one-launch sweep, [mu]: of direction mu's launch;
@@ -116,6 +119,7 @@ cudaError_t su3k_launch_sweep_f64(const HalfSweepArgs& a, const SweepQueue& q, b
 // Status words of the bounds-checked build, one per translation unit with
 // kernels (su3_device.cuh, link_ok); 0 in the product build.
 cudaError_t su3k_bounds_status_kernels(unsigned int* v, bool clear);
+cudaError_t su3k_bounds_status_f64(unsigned int* v, bool clear);
 cudaError_t su3k_bounds_status_pair(unsigned int* v, bool clear);
 cudaError_t su3k_bounds_status_batch(unsigned int* v, bool clear);
 cudaError_t su3k_bounds_status_decomp(unsigned int* v, bool clear);

@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(256, 2)
   __shared__ SweepItem s_item;
   constexpr int kPhases = MUSEL < 0 ? 8 : 2, kFirst = MUSEL < 0 ? 0 : 2 * MUSEL;
   if (MUSEL >= 0) signal_dependents();
-  take_sweep_item<kPhases, kFirst>(qa, MUSEL < 0 ? 0 : MUSEL, tiles_per_layer, layers, &s_item);
+  take_sweep_item<kPhases>(qa, kFirst, MUSEL < 0 ? 0 : MUSEL, tiles_per_layer, layers, &s_item);
   __syncthreads();
   const SweepItem it = s_item;
   if (it.phase < 0) return;

@@ -1,6 +1,6 @@
 // su3_sweepq.cuh -- the work queue of the persistent and chained sweeps
 // (k_sweep_f32_pair and k_half_sweep_f32_chain in su3_kernels_pair.cu,
-// k_sweep_f64 in su3_kernels.cu).
+// k_sweep_f64 in su3_kernels_f64.cu).
 //
 // A persistent sweep runs the half-sweeps (mu, parity) of a sweep, in the
 // order of the paper's sweep (mu = 0..3, even then odd sites; checkerboard
@@ -118,12 +118,12 @@ __device__ __forceinline__ bool wait_sweep_layers(const SweepQueue& qa, int phas
 }
 
 // Warp 0 takes the block's item from counter `ticket` of the queue (the
-// launch holds kPhases phases from kFirst on) and waits for the layers of
+// launch holds kPhases phases from `first` on) and waits for the layers of
 // phase q-1 it reads; the item lands in *item (shared memory), which the
 // block reads after a __syncthreads.
-template <int kPhases, int kFirst>
-__device__ __forceinline__ void take_sweep_item(const SweepQueue& qa, int ticket, int tiles_per_layer, int layers,
-                                                SweepItem* item) {
+template <int kPhases>
+__device__ __forceinline__ void take_sweep_item(const SweepQueue& qa, int first, int ticket, int tiles_per_layer,
+                                                int layers, SweepItem* item) {
   if (threadIdx.x >= 32) return;
   const int tiles_per_phase = tiles_per_layer * layers;
   const int lane = (int)threadIdx.x;
@@ -132,8 +132,8 @@ __device__ __forceinline__ void take_sweep_item(const SweepQueue& qa, int ticket
   idx = __shfl_sync(0xffffffffu, idx, 0);
   int phase = -1, tile = 0, layer = 0;
   if (idx < kPhases * tiles_per_phase) {
-    phase = kFirst + idx / tiles_per_phase;
-    sweep_tile_of(phase, idx - (phase - kFirst) * tiles_per_phase, tiles_per_layer, layers, &layer, &tile);
+    phase = first + idx / tiles_per_phase;
+    sweep_tile_of(phase, idx - (phase - first) * tiles_per_phase, tiles_per_layer, layers, &layer, &tile);
   }
   const bool ok = wait_sweep_layers(qa, phase, layer, tiles_per_layer, layers, phase >= 0);
   if (lane == 0) *item = SweepItem{ok ? phase : -1, tile, layer, idx};

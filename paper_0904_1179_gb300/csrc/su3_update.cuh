@@ -14,6 +14,7 @@
 #pragma once
 
 #include "su3_device.cuh"
+#include "su3_fx.cuh"
 #include "su3_pair.cuh"
 
 namespace su3dev {
@@ -117,9 +118,6 @@ __device__ __forceinline__ void store_pair_site(float4* U, int mu, int p, int h,
 // accumulation of A's row 2 (acc_completed).  The paths are added in the
 // order forward, backward for nu ascending; every kernel that forms a staple
 // keeps this order, so their results agree bit for bit.
-// Apart (optional): receives the sum of the terms with nu < MU.  After the
-// update, Re Tr(U_new Apart) is the sum of the plaquettes of the planes
-// (MU, nu < MU) at x and at x - nu-hat.
 // The two three-link paths of direction nu (nu != mu), rows 0,1:
 //   forward  F = U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+,
 //   backward B = U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu).
@@ -153,41 +151,6 @@ __device__ __forceinline__ mat3<T> backward_path(const G& g, const void* U, int 
   mul_dn_rows01(hm, f, b);
   return b;
 }
-
-// A = F (rows 0,1 given, row 2 completed): the first term of a staple.
-template <typename T>
-__device__ __forceinline__ void init_completed(mat3<T>& A, const mat3<T>& F) {
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    A.e[0][k] = F.e[0][k];
-    A.e[1][k] = F.e[1][k];
-  }
-  complete_row2(A);
-}
-
-template <typename T, int MU, bool CG, typename G, typename S>
-__device__ __forceinline__ mat3<T> staple(const G& g, const void* U, const S& st, int h, int p,
-                                          mat3<T>* Apart = nullptr) {
-  mat3<T> A;
-  const int h_pmu = nb_half(g, st, MU, +1);
-#pragma unroll
-  for (int nu = 0; nu < 4; ++nu) {
-    if (nu == MU) continue;
-    const int h_pnu = nb_half(g, st, nu, +1);
-    const int h_mnu = nb_half(g, st, nu, -1);
-    const int h_pmu_mnu = nb_half2(g, st, MU, nu);
-    const mat3<T> F = forward_path<T, CG>(g, U, st, h, p, MU, nu, h_pmu, h_pnu);
-    if (nu == (MU == 0 ? 1 : 0)) {
-      init_completed(A, F);
-    } else {
-      acc_completed(A, F);
-    }
-    acc_completed(A, backward_path<T, CG>(g, U, p, MU, nu, h_mnu, h_pmu_mnu));
-    if (Apart && nu == MU - 1) *Apart = A;
-  }
-  return A;
-}
-
 
 // 2x2 block of W = U A in rows/columns (i, j), projected on the SU(2) direction,
 // returned as 2r = (Re(W_ii+W_jj), Im(W_ij+W_ji), Re(W_ij-W_ji), Im(W_ii-W_jj)):
@@ -238,6 +201,7 @@ struct UpdateConsts {
   double three_over_beta_f64;  // 3 / beta: 1/alpha = 3 / (2 beta k) = three_over_beta / (2k)
   float three_over_beta;
   int max_tries;  // 1: one-hit heatbath; > 1: repeat until accepted, at most this many proposals
+  int* far;       // FP64 stores: the flags of SweepState (su3_device.cuh)
 };
 
 // Accepted and drawn SU(2) proposals of one link update (a degenerate
@@ -246,39 +210,72 @@ struct UpdateCount {
   int accepted, proposed;
 };
 
-// ---------------------------------------------------------------------------
-// One FP64 link update: staple, three one-hit SU(2) heatbath steps, FP64
-// Gram-Schmidt, store.  Returns the number of accepted SU(2) proposals.
-// ---------------------------------------------------------------------------
-// MEAS: also return in *meas (1/3) Re Tr(U_new A_<), A_< the staple terms of
-// the directions nu < MU (see staple()).
-// G: Geometry (periodic lattice) or SubGeometry (sublattice with ghost
-// layers); h enumerates the sites of parity p, hs is where the site is stored.
-template <int MU, bool CG, bool REPEAT, bool MEAS, typename KEY, typename G>
-__device__ __forceinline__ UpdateCount heatbath_f64(const G& g, double2* U, int h, int p, uint64_t t, uint32_t s,
-                                                    const KEY& key, const UpdateConsts& uc, const mat3<double>& A,
-                                                    const mat3<double>& Apart, double* meas);
+// Kennedy-Pendleton proposals of subgroup sub of link (s, mu) at sweep t in
+// FP64: a0..a3 of the accepted one into a; false if none of the ntries was.
+template <bool REPEAT, typename KEY>
+__device__ __forceinline__ bool propose_f64(uint32_t s, int mu, int sub, uint64_t t, const KEY& key, double inv_alpha,
+                                            int max_tries, double a[4], UpdateCount& cnt) {
+  const int ntries = REPEAT ? max_tries : 1;
+  for (int tr = 0; tr < ntries; ++tr) {
+    double uu[6];
+#pragma unroll
+    for (int call = 0; call < 3; ++call) {
+      const uint32_t w1 = (uint32_t)(mu | (sub << 2) | (call << 4)) | ((uint32_t)tr << 6);
+      const uint4 w = philox4x32_10(rng_counter(s, w1, t, kTagUpdate), key);
+      uu[2 * call] = u01_f64(w.x, w.y);
+      uu[2 * call + 1] = u01_f64(w.z, w.w);
+    }
+    ++cnt.proposed;
+    const double c = cospi(2.0 * uu[1]);  // cos(2 pi u1)
+    const double delta = -(log_u01(uu[0]) + c * c * log_u01(uu[2])) * inv_alpha;
+    if (uu[3] * uu[3] > 1.0 - 0.5 * delta) continue;
+    const double a0 = 1.0 - delta;
+    double rho = 1.0 - a0 * a0;
+    rho = rho > 0.0 ? sqrt(rho) : 0.0;
+    const double ct = 1.0 - 2.0 * uu[4];
+    double sn = 1.0 - ct * ct;
+    sn = sn > 0.0 ? sqrt(sn) : 0.0;
+    double sphi, cphi;
+    sincospi(2.0 * uu[5], &sphi, &cphi);  // angle 2 pi u5
+    a[0] = a0;
+    a[1] = rho * sn * cphi;
+    a[2] = rho * sn * sphi;
+    a[3] = rho * ct;
+    ++cnt.accepted;
+    return true;
+  }
+  return false;
+}
 
-template <int MU, bool CG, bool REPEAT, bool MEAS = false, typename KEY, typename G>
-__device__ __forceinline__ UpdateCount update_link_f64(const G& g, double2* U, int h, int p, uint64_t t,
-                                                       const KEY& key, const UpdateConsts& uc, double* meas = nullptr) {
+// ---------------------------------------------------------------------------
+// One FP64 link update in FP64 arithmetic: staple, three SU(2) heatbath steps,
+// Gram-Schmidt, store.  It serves configurations with links far from SU(3)
+// (SweepState::far), whose entries and products may leave the range of
+// su3_fx.cuh: one function for every direction and heatbath, not inlined and
+// its loops not unrolled, since no sweep of a proper configuration runs it.
+// meas (nullptr: off) receives (1/3) Re Tr(U_new A_<), A_< the staple terms of
+// the directions nu < mu.
+// G: Geometry (periodic lattice) or SubGeometry (sublattice with ghost
+// layers); h enumerates the sites of parity p.
+// ---------------------------------------------------------------------------
+template <bool CG, typename KEY, typename G>
+__device__ __noinline__ UpdateCount update_link_f64_far(const G& g, double2* U, int h, int p, int mu, uint64_t t,
+                                                        const KEY& key, const UpdateConsts& uc, double* meas) {
   const auto st = site_of(g, h, p);
   const uint32_t s = (uint32_t)canon(g, st);
   h = store_index(g, st, h);
-  mat3<double> Apart;
-  const mat3<double> A = staple<double, MU, CG>(g, U, st, h, p, MEAS ? &Apart : nullptr);
-  return heatbath_f64<MU, CG, REPEAT, MEAS>(g, U, h, p, t, s, key, uc, A, Apart, meas);
-}
-
-// Everything after the staple: three SU(2) heatbath steps, Gram-Schmidt and
-// the store of link (s, MU) at storage half index h.
-template <int MU, bool CG, bool REPEAT, bool MEAS, typename KEY, typename G>
-__device__ __forceinline__ UpdateCount heatbath_f64(const G& g, double2* U, int h, int p, uint64_t t, uint32_t s,
-                                                    const KEY& key, const UpdateConsts& uc, const mat3<double>& A,
-                                                    const mat3<double>& Apart, double* meas) {
+  mat3<double> A = zero3<double>(), Apart = A;
+  const int h_pmu = nb_half_rt(g, st, mu, +1);
+#pragma unroll 1
+  for (int nu = 0; nu < 4; ++nu) {
+    if (nu == mu) continue;
+    acc_completed(A, forward_path<double, CG>(g, U, st, h, p, mu, nu, h_pmu, nb_half_rt(g, st, nu, +1)));
+    acc_completed(A, backward_path<double, CG>(g, U, p, mu, nu, nb_half_rt(g, st, nu, -1), nb_half2_rt(g, st, mu, nu)));
+    if (nu == mu - 1) Apart = A;
+  }
   UpdateCount cnt{0, 0};
-  mat3<double> u = load_f64<CG>(U, MU, p, h, g.Vh);
-#pragma unroll
+  mat3<double> u = load_f64<CG>(U, mu, p, h, g.Vh);
+#pragma unroll 1
   for (int sub = 0; sub < 3; ++sub) {
     const int i = subrow_i(sub), j = subrow_j(sub);
     double r[4];  // 2r
@@ -290,35 +287,11 @@ __device__ __forceinline__ UpdateCount heatbath_f64(const G& g, double2* U, int 
     }
     const double ik = rsqrt(kk);                           // 1 / (2k)
     const double inv_alpha = uc.three_over_beta_f64 * ik;  // 1/alpha = 3 / (2 beta k)
-    const int ntries = REPEAT ? uc.max_tries : 1;
-    for (int tr = 0; tr < ntries; ++tr) {
-      double uu[6];
-#pragma unroll
-      for (int call = 0; call < 3; ++call) {
-        const uint32_t w1 = (uint32_t)(MU | (sub << 2) | (call << 4)) | ((uint32_t)tr << 6);
-        const uint4 w = philox4x32_10(rng_counter(s, w1, t, kTagUpdate), key);
-        uu[2 * call] = u01_f64(w.x, w.y);
-        uu[2 * call + 1] = u01_f64(w.z, w.w);
-      }
-      ++cnt.proposed;
-      const double c = cospi(2.0 * uu[1]);  // cos(2 pi u1)
-      const double delta = -(log_u01(uu[0]) + c * c * log_u01(uu[2])) * inv_alpha;
-      if (uu[3] * uu[3] > 1.0 - 0.5 * delta) continue;
-      const double a0 = 1.0 - delta;
-      double rho = 1.0 - a0 * a0;
-      rho = rho > 0.0 ? sqrt(rho) : 0.0;
-      const double ct = 1.0 - 2.0 * uu[4];
-      double sn = 1.0 - ct * ct;
-      sn = sn > 0.0 ? sqrt(sn) : 0.0;
-      double sphi, cphi;
-      sincospi(2.0 * uu[5], &sphi, &cphi);  // angle 2 pi u5
-      const double a[4] = {a0, rho * sn * cphi, rho * sn * sphi, rho * ct};
-      const double v[4] = {r[0] * ik, r[1] * ik, r[2] * ik, r[3] * ik};  // r / k
-      // Row 2 leaves the last subgroup unused: reunitarisation rebuilds it.
-      apply_su2(u, i, j, a, v, sub < 2);
-      ++cnt.accepted;
-      break;
-    }
+    double a[4];
+    if (!propose_f64<true>(s, mu, sub, t, key, inv_alpha, uc.max_tries, a, cnt)) continue;
+    const double v[4] = {r[0] * ik, r[1] * ik, r[2] * ik, r[3] * ik};  // r / k
+    // Row 2 leaves the last subgroup unused: reunitarisation rebuilds it.
+    apply_su2(u, i, j, a, v, sub < 2);
   }
   cx<double> r0[3] = {u.e[0][0], u.e[0][1], u.e[0][2]};
   cx<double> r1[3] = {u.e[1][0], u.e[1][1], u.e[1][2]};
@@ -330,8 +303,9 @@ __device__ __forceinline__ UpdateCount heatbath_f64(const G& g, double2* U, int 
     out.e[1][k] = r1[k];
   }
   complete_row2(out);
-  store_f64(U, MU, p, h, g.Vh, out);
-  if (MEAS) {
+  store_f64(U, mu, p, h, g.Vh, out);
+  if (far_from_su3(out)) atomicOr(uc.far + 1, 1);
+  if (meas) {
     double tr = 0.0;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -340,6 +314,241 @@ __device__ __forceinline__ UpdateCount heatbath_f64(const G& g, double2* U, int 
     *meas = tr * (1.0 / 3.0);
   }
   return cnt;
+}
+
+// ---------------------------------------------------------------------------
+// The FP64 link update on the integer and FP32 pipes (su3_fx.cuh): links are
+// read from the FP64 store, split into integer and FP32 parts, and multiplied
+// there; only the scalars of the Kennedy-Pendleton proposals are FP64 numbers.
+// Loads go entry by entry, in the order in which the products use them.
+// ---------------------------------------------------------------------------
+// A link of the store, or its adjoint.
+template <bool CG>
+struct FxLink {
+  const double2* b;
+  int si, sk;     // elements between rows and between columns
+  uint32_t flip;  // sign of the imaginary parts
+  bool ok;
+  __device__ __forceinline__ FxLink(const void* U, int mu, int p, int h, int Vh, bool dag = false)
+      : b((const double2*)U + link_base(mu, p, Vh, kEntriesF64) + h),
+        si(dag ? Vh : 3 * Vh),
+        sk(dag ? 3 * Vh : Vh),
+        flip(dag ? 0x80000000u : 0u),
+        ok(link_ok(mu, p, h, Vh)) {}
+  __device__ __forceinline__ cfx at(int i, int k) const {
+    if (!ok) return cfx{{0, 0.0f, 0.0f}, {0, 0.0f, 0.0f}};
+    const double2 v = ld_link<CG>(b + ((size_t)i * si + (size_t)k * sk));
+    return cfx{fx_from_double(v.x), fx_from_double(v.y, flip)};
+  }
+};
+
+// Rows 0,1 of X Y^+ Z.
+template <bool CG>
+__device__ __forceinline__ fx_rows01 path_fx(const FxLink<CG>& X, const FxLink<CG>& Y, const FxLink<CG>& Z) {
+  cfx x[2][3], t[2][3];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) x[i][k] = X.at(i, k);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    cfacc s[2] = {cfx_zero(), cfx_zero()};
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const cfx y = Y.at(k, j);
+      cfx_mac_cb(s[0], x[0][j], y);
+      cfx_mac_cb(s[1], x[1][j], y);
+    }
+    t[0][k] = cfx_norm(s[0]);
+    t[1][k] = cfx_norm(s[1]);
+  }
+  fx_rows01 f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    cfacc s[2] = {cfx_zero(), cfx_zero()};
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const cfx z = Z.at(j, k);
+      cfx_mac(s[0], t[0][j], z);
+      cfx_mac(s[1], t[1][j], z);
+    }
+    f.e[0][k] = cfx_norm(s[0]);
+    f.e[1][k] = cfx_norm(s[1]);
+  }
+  return f;
+}
+
+// The two paths of direction nu (forward_path, backward_path above): one piece
+// of code for both, so that the whole update stays within the instruction
+// caches.
+//   forward:  U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+,  backward: U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu);
+// hx, hy, hz: half indices of the three sites.
+template <bool CG>
+__device__ __forceinline__ fx_rows01 staple_path_fx(const void* U, int Vh, int p, int mu, int nu, bool backward, int hx,
+                                                    int hy, int hz) {
+  const int q = p ^ 1;
+  return path_fx(FxLink<CG>(U, nu, backward ? p : q, hx, Vh, backward), FxLink<CG>(U, mu, q, hy, Vh),
+                 FxLink<CG>(U, nu, backward ? q : p, hz, Vh, !backward));
+}
+
+// Six-staple sum of U_mu(x), x = st of parity p stored at h.
+// Apart (optional): receives the sum of the terms with nu < mu.  After the
+// update, Re Tr(U_new Apart) is the sum of the plaquettes of the planes
+// (mu, nu < mu) at x and at x - nu-hat.
+template <bool CG, typename G, typename S>
+__device__ __forceinline__ fx_mat staple_fx(const G& g, const void* U, const S& st, int h, int p, int mu,
+                                            fx_mat* Apart = nullptr) {
+  fx_staple A;
+  fx_staple_zero(A);
+  const int h_pmu = nb_half_rt(g, st, mu, +1);
+#pragma unroll 1
+  for (int path = 0; path < 6; ++path) {
+    const bool backward = path & 1;
+    const int nu = (path >> 1) + ((path >> 1) >= mu ? 1 : 0);
+    const int hy = nb_half_rt(g, st, nu, backward ? -1 : +1);
+    fx_staple_add(A, staple_path_fx<CG>(U, g.Vh, p, mu, nu, backward, backward ? nb_half2_rt(g, st, mu, nu) : h_pmu, hy,
+                                        backward ? hy : h));
+    if (Apart && backward && nu == mu - 1) *Apart = fx_staple_mat(A);
+  }
+  return fx_staple_mat(A);
+}
+
+// A sum of products of units 2^-30 and 2^-28 as FP64, times 2^58.  The cross
+// terms of the projection and of the measured trace (up to 2^65.4 in units of
+// 2^-90) are merged to 2^-54, 2^-3 of an FP64 unit of the sum's last place.
+__device__ __forceinline__ double fx_sum_to_double(const facc& s) {
+  const int ci = __float2int_rn(__fmul_rn(s.c, 0x1p-36f));
+  return __ll2double_rn(s.hh + 16LL * ci);
+}
+
+// Everything after the staple A (unit 2^-28): three SU(2) heatbath steps,
+// reunitarisation, the store of link (s, mu) at storage half index h.
+// MEAS: also (1/3) Re Tr(U_new Apart) into *meas.
+template <bool CG, bool REPEAT, bool MEAS, typename KEY, typename G>
+__device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h, int p, int mu, uint64_t t, uint32_t s,
+                                                   const KEY& key, const UpdateConsts& uc, const fx_mat& A,
+                                                   const fx_mat& Apart, double* meas) {
+  UpdateCount cnt{0, 0};
+  fx_mat u;
+  const FxLink<CG> own(U, mu, p, h, g.Vh);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u.e[i][k] = own.at(i, k);
+#pragma unroll
+  for (int sub = 0; sub < 3; ++sub) {
+    const int i = subrow_i(sub), j = subrow_j(sub);
+    // 2r as in su2_projection, each component one sum
+    facc w[4] = {{8, 0.0f}, {8, 0.0f}, {8, 0.0f}, {8, 0.0f}};  // half of what fx_sum_to_double's rounding drops
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const cfx &ui = u.e[i][c], &uj = u.e[j][c], &ai = A.e[c][i], &aj = A.e[c][j];
+      fx_mac(w[0], ui.re, ai.re);
+      fx_msub(w[0], ui.im, ai.im);
+      fx_mac(w[0], uj.re, aj.re);
+      fx_msub(w[0], uj.im, aj.im);
+      fx_mac(w[1], ui.re, aj.im);
+      fx_mac(w[1], ui.im, aj.re);
+      fx_mac(w[1], uj.re, ai.im);
+      fx_mac(w[1], uj.im, ai.re);
+      fx_mac(w[2], ui.re, aj.re);
+      fx_msub(w[2], ui.im, aj.im);
+      fx_msub(w[2], uj.re, ai.re);
+      fx_mac(w[2], uj.im, ai.im);
+      fx_mac(w[3], ui.re, ai.im);
+      fx_mac(w[3], ui.im, ai.re);
+      fx_msub(w[3], uj.re, aj.im);
+      fx_msub(w[3], uj.im, aj.re);
+    }
+    const double r[4] = {fx_sum_to_double(w[0]), fx_sum_to_double(w[1]), fx_sum_to_double(w[2]),
+                         fx_sum_to_double(w[3])};  // 2r 2^58
+    const double kk = r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + r[3] * r[3];
+    if (!(kk > 0.0)) {  // k = 0: degenerate staple (measure zero), leave the subgroup
+      ++cnt.proposed;
+      continue;
+    }
+    const double ik = rsqrt(kk);  // 2^-58 / (2k)
+    const double ik1 = __hiloint2double(__double2hiint(ik) + (58 << 20), __double2loint(ik));
+    double a[4];
+    if (!propose_f64<REPEAT>(s, mu, sub, t, key, uc.three_over_beta_f64 * ik1, uc.max_tries, a, cnt)) continue;
+    const double v[4] = {r[0] * ik, r[1] * ik, r[2] * ik, r[3] * ik};  // r / k
+    // R as in apply_su2
+    const cx<double> y00 = mk(a[0], a[3]), y01 = mk(a[2], a[1]);
+    const cx<double> v00 = mk(v[0], v[3]), v01 = mk(v[2], v[1]), v10 = mk(-v[2], v[1]), v11 = mk(v[0], -v[3]);
+    const cx<double> D00 = mac_cb(mac_cb(mk(0.0, 0.0), y00, v00), y01, v01);
+    const cx<double> D01 = mac_cb(mac_cb(mk(0.0, 0.0), y00, v10), y01, v11);
+    const cfx R00{fx_from_double(D00.re), fx_from_double(D00.im)}, R01{fx_from_double(D01.re), fx_from_double(D01.im)};
+    const cfx R10{fx_neg(R01.re), R01.im}, R11 = cfx_conj(R00);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const cfx ui = u.e[i][c], uj = u.e[j][c];
+      cfacc z = cfx_zero();
+      cfx_mac(z, R00, ui);
+      cfx_mac(z, R01, uj);
+      u.e[i][c] = cfx_norm(z);
+      if (sub < 2) {  // row 2 leaves the last subgroup unused: reunitarisation rebuilds it
+        z = cfx_zero();
+        cfx_mac(z, R10, ui);
+        cfx_mac(z, R11, uj);
+        u.e[j][c] = cfx_norm(z);
+      }
+    }
+  }
+  mat3<double> out;
+  if (fx_reunitarise(u)) {
+    fx_complete_row2(u);
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) out.e[i][k] = mk(fx_to_double(u.e[i][k].re), fx_to_double(u.e[i][k].im));
+  } else {  // a link of a configuration that was set with less than FP64 accuracy
+    cx<double> r0[3], r1[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      r0[k] = mk(fx_to_double(u.e[0][k].re), fx_to_double(u.e[0][k].im));
+      r1[k] = mk(fx_to_double(u.e[1][k].re), fx_to_double(u.e[1][k].im));
+    }
+    gram_schmidt_rows01(r0, r1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      out.e[0][k] = r0[k];
+      out.e[1][k] = r1[k];
+    }
+    complete_row2(out);
+    if (MEAS) {
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          u.e[i][k] = cfx{fx_from_double(out.e[i][k].re), fx_from_double(out.e[i][k].im)};
+    }
+  }
+  store_f64(U, mu, p, h, g.Vh, out);
+  if (MEAS) {
+    facc tr{8, 0.0f};
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        fx_mac(tr, u.e[i][k].re, Apart.e[k][i].re);
+        fx_msub(tr, u.e[i][k].im, Apart.e[k][i].im);
+      }
+    *meas = fx_sum_to_double(tr) * (0x1p-58 / 3.0);
+  }
+  return cnt;
+}
+
+// One update of an FP64 store's link U_mu(x) (h, parity p as in site_of).
+template <bool CG, bool REPEAT, bool MEAS = false, typename KEY, typename G>
+__device__ __forceinline__ UpdateCount update_link_f64(const G& g, double2* U, int h, int p, int mu, uint64_t t,
+                                                       const KEY& key, const UpdateConsts& uc, double* meas = nullptr) {
+  if (*(volatile const int*)uc.far) return update_link_f64_far<CG>(g, U, h, p, mu, t, key, uc, MEAS ? meas : nullptr);
+  const auto st = site_of(g, h, p);
+  const uint32_t s = (uint32_t)canon(g, st);
+  h = store_index(g, st, h);
+  fx_mat Apart;
+  const fx_mat A = staple_fx<CG>(g, U, st, h, p, mu, MEAS ? &Apart : nullptr);
+  return heatbath_fx<CG, REPEAT, MEAS>(g, U, h, p, mu, t, s, key, uc, A, Apart, meas);
 }
 
 // ---------------------------------------------------------------------------
