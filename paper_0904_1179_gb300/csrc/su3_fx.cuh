@@ -125,11 +125,11 @@ SU3_HD fx fx_norm_high(const facc& s) {
 // Where the accumulator of an fx_norm starts.
 SU3_HD facc fx_zero() { return facc{1LL << 29, 0.0f}; }
 
-// An FP64 number with |d| < 2 in the unit 2^-30: the mantissa as a 63-bit
+// An FP64 number with |d| < 2 in units of 2^-62: the mantissa as a 63-bit
 // fraction, shifted right by the exponent.  A bit of the value below 2^-62 is
 // dropped.  (Integer pipe only: a conversion on the FP64 pipe takes 16 cycles.)
 // flip: 0x80000000 negates d.
-SU3_HD fx fx_from_double(double d, uint32_t flip = 0u) {
+SU3_HD long long fx_i62_from_double(double d, uint32_t flip = 0u) {
   uint32_t hi, lo;
 #ifdef __CUDA_ARCH__
   hi = (uint32_t)__double2hiint(d);
@@ -155,8 +155,21 @@ SU3_HD fx fx_from_double(double d, uint32_t flip = 0u) {
 #else
   x = m >> (sh > 63 ? 63 : sh);
 #endif
+  return x;
+}
+SU3_HD fx fx_from_i62(long long x) {
   const int xl = (int)(uint32_t)x;
   return fx_make((int)(x >> 32) + (int)((uint32_t)xl >> 31), fx_i2f(xl));
+}
+SU3_HD fx fx_from_double(double d, uint32_t flip = 0u) { return fx_from_i62(fx_i62_from_double(d, flip)); }
+// The same by one conversion on the FP64 pipe, which is otherwise idle.
+SU3_HD fx fx_from_double_cvt(double d, uint32_t flip = 0u) {
+#ifdef __CUDA_ARCH__
+  const int hi = __double2hiint(d) + (62 << 20);
+  return fx_from_i62(__double2ll_rz(__hiloint2double((int)((uint32_t)hi ^ flip), __double2loint(d))));
+#else
+  return fx_from_double(d, flip);
+#endif
 }
 
 // The value in units of 2^-62 as a 64-bit integer (l rounded to two of them).

@@ -5,10 +5,12 @@
 //
 // The same update in FP64 arithmetic kept the FP64 pipe (two lanes per SM) busy
 // for 93 % of 13.2 ms per 32^4 sweep.  With the matrix products of the staple,
-// the rotations and the reunitarisation moved to the integer multiplier and FP32
-// (1.76 SM cycles per multiply-add and warp instead of 16) a sweep takes 5.15
-// ms; what is left on the FP64 pipe are the scalars of the proposals, about
-// 450 instructions per update.
+// the rotations and the reunitarisation on the integer multiplier and FP32 (1.76
+// SM cycles per multiply-add and warp instead of 16) a sweep took 5.15 ms; with
+// the scalars of the proposals there too (su3_fx_kp.cuh) and the subgroups in
+// one loop (instruction fetch had become the largest stall: 2.4 of 6.6 cycles
+// per instruction) 3.90 ms.  Now 20,000 instructions per warp at 0.51 issued
+// per cycle and scheduler; waits for instructions are still the first stall.
 #include "su3_kernels.h"
 
 #include "su3_device.cuh"
@@ -18,10 +20,9 @@
 
 using namespace su3dev;
 
-// Registers per thread.  GB300, 32^4, ms per sweep of eight launches (and of the
-// per-direction launches): 128 registers 5.28 (4.62), 144: 5.24 (4.79), 168:
-// 5.15 (4.69), 200: 6.27 (6.13), 255: 6.15 (6.18).  168 is the most that keeps
-// 12 warps on an SM (it spills 84 bytes); blocks of 256 threads stay legal.
+// Registers per thread.  GB300, 32^4, ms per sweep: 128 registers 4.52, 144: 4.44,
+// 168: 4.18, 200: 4.61.  168 is the most that keeps 12 warps on an SM; blocks of
+// 256 threads stay legal.
 #ifndef SU3_F64_REGS
 #define SU3_F64_REGS 168
 #endif

@@ -15,6 +15,7 @@
 
 #include "su3_device.cuh"
 #include "su3_fx.cuh"
+#include "su3_fx_kp.cuh"
 #include "su3_pair.cuh"
 
 namespace su3dev {
@@ -319,7 +320,8 @@ __device__ __noinline__ UpdateCount update_link_f64_far(const G& g, double2* U, 
 // ---------------------------------------------------------------------------
 // The FP64 link update on the integer and FP32 pipes (su3_fx.cuh): links are
 // read from the FP64 store, split into integer and FP32 parts, and multiplied
-// there; only the scalars of the Kennedy-Pendleton proposals are FP64 numbers.
+// there; the SU(2) steps (su3_fx_kp.cuh) use it too, but for the four FP64
+// operations that make delta from 1/alpha, whose range beta leaves open.
 // Loads go entry by entry, in the order in which the products use them.
 // ---------------------------------------------------------------------------
 // A link of the store, or its adjoint.
@@ -338,7 +340,11 @@ struct FxLink {
   __device__ __forceinline__ cfx at(int i, int k) const {
     if (!ok) return cfx{{0, 0.0f, 0.0f}, {0, 0.0f, 0.0f}};
     const double2 v = ld_link<CG>(b + ((size_t)i * si + (size_t)k * sk));
-    return cfx{fx_from_double(v.x), fx_from_double(v.y, flip)};
+    // Real parts on the integer pipe (14 instructions), imaginary parts by a
+    // conversion on the FP64 pipe (5, but 16 SM cycles of a pipe that is
+    // otherwise nearly idle): 32^4 3.90 ms per sweep, against 4.17 with both on
+    // the integer pipe and 4.26 with both converted.
+    return cfx{fx_from_double(v.x), fx_from_double_cvt(v.y, flip)};
   }
 };
 
@@ -413,20 +419,19 @@ __device__ __forceinline__ fx_mat staple_fx(const G& g, const void* U, const S& 
   return fx_staple_mat(A);
 }
 
-// A sum of products of units 2^-30 and 2^-28 as FP64, times 2^58.  The cross
-// terms of the projection and of the measured trace (up to 2^65.4 in units of
-// 2^-90) are merged to 2^-54, 2^-3 of an FP64 unit of the sum's last place.
-__device__ __forceinline__ double fx_sum_to_double(const facc& s) {
-  const int ci = __float2int_rn(__fmul_rn(s.c, 0x1p-36f));
-  return __ll2double_rn(s.hh + 16LL * ci);
+// A sum of products of units 2^-30 and 2^-28 merged (units of 2^-58).  The cross
+// terms of the projection and of the measured trace reach 2^65.4 in units of
+// 2^-90: they are taken to 2^-54.
+__device__ __forceinline__ long long fx_merge_wide(const facc& s) {
+  return s.hh + 16LL * __float2int_rn(__fmul_rn(s.c, 0x1p-36f));
 }
 
-// Everything after the staple A (unit 2^-28): three SU(2) heatbath steps,
+// Everything after the staple A0 (unit 2^-28): three SU(2) heatbath steps,
 // reunitarisation, the store of link (s, mu) at storage half index h.
 // MEAS: also (1/3) Re Tr(U_new Apart) into *meas.
 template <bool CG, bool REPEAT, bool MEAS, typename KEY, typename G>
 __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h, int p, int mu, uint64_t t, uint32_t s,
-                                                   const KEY& key, const UpdateConsts& uc, const fx_mat& A,
+                                                   const KEY& key, const UpdateConsts& uc, const fx_mat& A0,
                                                    const fx_mat& Apart, double* meas) {
   UpdateCount cnt{0, 0};
   fx_mat u;
@@ -435,14 +440,17 @@ __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int k = 0; k < 3; ++k) u.e[i][k] = own.at(i, k);
-#pragma unroll
+  // The subgroups (0,1), (0,2), (1,2) in one piece of code (instruction cache):
+  // the step always acts on rows 0, 1 of u and columns 0, 1 of A, and between the
+  // steps rows and columns change places: orders (0,1,2), (0,2,1), (1,2,0).
+  fx_mat A = A0;
+#pragma unroll 1
   for (int sub = 0; sub < 3; ++sub) {
-    const int i = subrow_i(sub), j = subrow_j(sub);
     // 2r as in su2_projection, each component one sum
-    facc w[4] = {{8, 0.0f}, {8, 0.0f}, {8, 0.0f}, {8, 0.0f}};  // half of what fx_sum_to_double's rounding drops
+    facc w[4] = {{0, 0.0f}, {0, 0.0f}, {0, 0.0f}, {0, 0.0f}};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const cfx &ui = u.e[i][c], &uj = u.e[j][c], &ai = A.e[c][i], &aj = A.e[c][j];
+      const cfx &ui = u.e[0][c], &uj = u.e[1][c], &ai = A.e[c][0], &aj = A.e[c][1];
       fx_mac(w[0], ui.re, ai.re);
       fx_msub(w[0], ui.im, ai.im);
       fx_mac(w[0], uj.re, aj.re);
@@ -460,40 +468,63 @@ __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h
       fx_msub(w[3], uj.re, aj.im);
       fx_msub(w[3], uj.im, aj.re);
     }
-    const double r[4] = {fx_sum_to_double(w[0]), fx_sum_to_double(w[1]), fx_sum_to_double(w[2]),
-                         fx_sum_to_double(w[3])};  // 2r 2^58
-    const double kk = r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + r[3] * r[3];
-    if (!(kk > 0.0)) {  // k = 0: degenerate staple (measure zero), leave the subgroup
-      ++cnt.proposed;
-      continue;
-    }
-    const double ik = rsqrt(kk);  // 2^-58 / (2k)
-    const double ik1 = __hiloint2double(__double2hiint(ik) + (58 << 20), __double2loint(ik));
-    double a[4];
-    if (!propose_f64<REPEAT>(s, mu, sub, t, key, uc.three_over_beta_f64 * ik1, uc.max_tries, a, cnt)) continue;
-    const double v[4] = {r[0] * ik, r[1] * ik, r[2] * ik, r[3] * ik};  // r / k
-    // R as in apply_su2
-    const cx<double> y00 = mk(a[0], a[3]), y01 = mk(a[2], a[1]);
-    const cx<double> v00 = mk(v[0], v[3]), v01 = mk(v[2], v[1]), v10 = mk(-v[2], v[1]), v11 = mk(v[0], -v[3]);
-    const cx<double> D00 = mac_cb(mac_cb(mk(0.0, 0.0), y00, v00), y01, v01);
-    const cx<double> D01 = mac_cb(mac_cb(mk(0.0, 0.0), y00, v10), y01, v11);
-    const cfx R00{fx_from_double(D00.re), fx_from_double(D00.im)}, R01{fx_from_double(D01.re), fx_from_double(D01.im)};
-    const cfx R10{fx_neg(R01.re), R01.im}, R11 = cfx_conj(R00);
+    const long long r[4] = {fx_merge_wide(w[0]), fx_merge_wide(w[1]), fx_merge_wide(w[2]), fx_merge_wide(w[3])};
+    fx v[4], a[4];
+    double ik;
+    bool accepted = false;
+    if (fx_direction(r, v, &ik)) {
+      const double inv_alpha = uc.three_over_beta_f64 * ik;  // 1/alpha = 3 / (2 beta k)
+      const int ntries = REPEAT ? uc.max_tries : 1;
+#pragma unroll 1
+      for (int tr = 0; tr < ntries && !accepted; ++tr) {
+        unsigned long long m[6];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const cfx ui = u.e[i][c], uj = u.e[j][c];
-      cfacc z = cfx_zero();
-      cfx_mac(z, R00, ui);
-      cfx_mac(z, R01, uj);
-      u.e[i][c] = cfx_norm(z);
-      if (sub < 2) {  // row 2 leaves the last subgroup unused: reunitarisation rebuilds it
+        for (int call = 0; call < 3; ++call) {
+          const uint32_t w1 = (uint32_t)(mu | (sub << 2) | (call << 4)) | ((uint32_t)tr << 6);
+          const uint4 b = philox4x32_10(rng_counter(s, w1, t, kTagUpdate), key);
+          m[2 * call] = fx_uniform(b.x, b.y);
+          m[2 * call + 1] = fx_uniform(b.z, b.w);
+        }
+        ++cnt.proposed;
+        accepted = fx_propose(m, inv_alpha, a);
+      }
+    } else {
+      ++cnt.proposed;  // k = 0: degenerate staple (measure zero), leave the subgroup
+    }
+    if (accepted) {
+      ++cnt.accepted;
+      cfx R00, R01;
+      fx_rotation(a, v, R00, R01);
+      const cfx R10{fx_neg(R01.re), R01.im}, R11 = cfx_conj(R00);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const cfx ui = u.e[0][c], uj = u.e[1][c];
+        cfacc z = cfx_zero();
+        cfx_mac(z, R00, ui);
+        cfx_mac(z, R01, uj);
+        u.e[0][c] = cfx_norm(z);
+        // (in the last subgroup row 2 is not used any more: reunitarisation rebuilds it)
         z = cfx_zero();
         cfx_mac(z, R10, ui);
         cfx_mac(z, R11, uj);
-        u.e[j][c] = cfx_norm(z);
+        u.e[1][c] = cfx_norm(z);
       }
     }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const bool first = sub == 0;
+      const cfx x[3] = {u.e[0][c], u.e[1][c], u.e[2][c]}, y[3] = {A.e[c][0], A.e[c][1], A.e[c][2]};
+      u.e[0][c] = first ? x[0] : x[2];
+      u.e[1][c] = first ? x[2] : x[1];
+      u.e[2][c] = first ? x[1] : x[0];
+      A.e[c][0] = first ? y[0] : y[2];
+      A.e[c][1] = first ? y[2] : y[1];
+      A.e[c][2] = first ? y[1] : y[0];
+    }
   }
+  // after the last change: (row 0, row 2, row 1)
+#pragma unroll
+  for (int c = 0; c < 3; ++c) u.e[1][c] = u.e[2][c];
   mat3<double> out;
   if (fx_reunitarise(u)) {
     fx_complete_row2(u);
@@ -525,7 +556,7 @@ __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h
   }
   store_f64(U, mu, p, h, g.Vh, out);
   if (MEAS) {
-    facc tr{8, 0.0f};
+    facc tr{0, 0.0f};
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -533,7 +564,7 @@ __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h
         fx_mac(tr, u.e[i][k].re, Apart.e[k][i].re);
         fx_msub(tr, u.e[i][k].im, Apart.e[k][i].im);
       }
-    *meas = fx_sum_to_double(tr) * (0x1p-58 / 3.0);
+    *meas = (double)fx_merge_wide(tr) * (0x1p-58 / 3.0);
   }
   return cnt;
 }

@@ -4,9 +4,11 @@
 // Prints the largest errors, in units of 2^-53.
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <random>
 
 #include "su3_fx.cuh"
+#include "su3_fx_kp.cuh"
 
 using namespace su3dev;
 typedef long double Q;
@@ -67,7 +69,99 @@ static M su3(int kind) {
 static cfx dec(const M& m, int i, int k) { return {fx_from_double(m.e[i][k][0]), fx_from_double(m.e[i][k][1])}; }
 static Q val(const fx& a, int unit) { return std::ldexp((Q)a.h, unit) + std::ldexp((Q)a.l, unit - 32); }
 
+// Errors of the fixed-point functions and of their FP64 form (root mean square
+// and largest), in units of 2^-53.
+struct Err {
+  Q most = 0, sum = 0;
+  long n = 0;
+  void add(Q e) {
+    e = std::fabs(e) * std::ldexp((Q)1, 53);
+    most = std::fmax(most, e);
+    sum += e * e;
+    ++n;
+  }
+  Q rms() const { return std::sqrt(sum / n); }
+};
+
+static void heatbath_scalars() {
+  const Q pi = std::acos((Q)-1);
+  std::normal_distribution<double> nd;
+  Err lg, trig, root, dir, dir64, a0, a0_64, ax, ax64, rot;
+  long other = 0;
+  for (int it = 0; it < 200000; ++it) {
+    // uniforms over the whole range, and near 0, 1/2 and 1
+    unsigned long long m = rng() >> 11;
+    const int cut = (int)(rng() % 52);
+    if (it % 5 == 1) m >>= cut;
+    if (it % 5 == 2) m = (1ull << 53) - 1 - (m >> cut);
+    if (it % 5 == 3) m = (1ull << 52) + (m >> (cut / 2 + 26));
+    m |= 1;
+    if (it == 0) m = 1;
+    if (it == 2) m = (1ull << 53) - 1;
+    const Q x = std::ldexp((Q)m, -53);
+    lg.add(std::ldexp((Q)fx_neg_log(m), -57) + std::log(x));
+    const fx_cs cs = fx_cossin<true>(m);
+    trig.add(val(cs.c, -30) - std::cos(2 * pi * x));
+    trig.add(val(cs.s, -30) - std::sin(2 * pi * x));
+    root.add(val(fx_two_root((long long)(m << 9)), -30) - 2 * std::sqrt(x * (1 - x)));
+
+    long long r[4];
+    const int scale = it % 3 == 0 ? 59 : 20 + (int)(rng() % 40);
+    for (long long& c : r) c = (long long)std::ldexp(nd(rng), scale);
+    if (it % 7 == 0) r[1] = r[2] = r[3] = 0;
+    if (it % 11 == 0) r[1] = -r[0];
+    Q k = 0;
+    double kd = 0;
+    for (long long c : r) {
+      k += (Q)c * c;
+      kd = std::fma((double)c, (double)c, kd);
+    }
+    if (k == 0) continue;
+    k = std::sqrt(k);
+    fx v[4], a[4];
+    double ik;
+    if (!fx_direction(r, v, &ik)) {
+      std::printf("a direction was refused\n");
+      std::exit(1);
+    }
+    for (int c = 0; c < 4; ++c) {
+      dir.add(val(v[c], -30) - r[c] / k);
+      dir64.add((Q)((double)r[c] * (1.0 / std::sqrt(kd))) - r[c] / k);
+    }
+    unsigned long long w[6];
+    for (unsigned long long& y : w) y = (rng() >> 11) | 1;
+    const double ia = std::pow(10.0, -2.5 + 3.0 * (double)(rng() % 1000) / 1000.0);
+    Q U[6];
+    double D[6];
+    for (int c = 0; c < 6; ++c) U[c] = D[c] = std::ldexp((double)w[c], -53);
+    const Q cq1 = std::cos(2 * pi * U[1]), delta = -(std::log(U[0]) + cq1 * cq1 * std::log(U[2])) * ia;
+    const bool take = U[3] * U[3] <= 1 - delta / 2, took = fx_propose(w, ia, a);
+    other += take != took;
+    if (!take || !took) continue;
+    const double cd = (double)cq1, dd = -std::fma(cd * cd, std::log(D[2]), std::log(D[0])) * ia;
+    const Q rho = std::sqrt(1 - (1 - delta) * (1 - delta)), ct = 1 - 2 * U[4], sn = std::sqrt(1 - ct * ct);
+    const double rhod = std::sqrt(std::fma(-(1 - dd), 1 - dd, 1.0)), ctd = 1 - 2 * D[4];
+    const double snd = std::sqrt(std::fma(-ctd, ctd, 1.0));
+    const Q e[4] = {1 - delta, rho * sn * std::cos(2 * pi * U[5]), rho * sn * std::sin(2 * pi * U[5]), rho * ct};
+    const double f[4] = {1 - dd, rhod * snd * (double)std::cos(2 * pi * U[5]),
+                         rhod * snd * (double)std::sin(2 * pi * U[5]), rhod * ctd};
+    for (int c = 0; c < 4; ++c) {
+      (c ? ax : a0).add(val(a[c], -30) - e[c]);
+      (c ? ax64 : a0_64).add((Q)f[c] - e[c]);
+    }
+    cfx R0, R1;
+    fx_rotation(a, v, R0, R1);
+    Q n = -1;
+    for (const fx& y : {R0.re, R0.im, R1.re, R1.im}) n += val(y, -30) * val(y, -30);
+    rot.add(n);
+  }
+  std::printf("log %.3Lf trig %.3Lf root %.3Lf dir %.3Lf dir_fp %.3Lf azero %.3Lf azero_fp %.3Lf avec %.3Lf avec_fp %.3Lf "
+              "unit %.3Lf flips %ld\n", lg.most, trig.most, root.most, dir.rms(), dir64.rms(), a0.rms(), a0_64.rms(), ax.rms(),
+              ax64.rms(), rot.most, other);
+}
+
 int main() {
+  heatbath_scalars();
   const Q u = std::ldexp((Q)1, -53);
   Q decode = 0, staple = 0, plain = 0, reunit = 0, round_trip = 0;
   for (int it = 0; it < 200000; ++it) {
