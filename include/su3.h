@@ -188,11 +188,12 @@ SU3_API int su3_set_block_size(su3_handle h, int threads);
  * choice; the paper has none): 0 = automatic (the default), 1 = one thread
  * per link (FP64 and single-site FP32 stores) or per pair of links (FP32
  * stores in the site-paired layout, L3 a multiple of 4), 4 = four lanes per
- * link, which share the staple's paths (for small lattices, whose half-sweep
- * leaves the GPU mostly idle).  Results do not depend on it: every form adds
- * the staple in the same order and rounds every step identically.  Phases
- * that measure the plaquette and the repeat-until-accepted heatbath always
- * take the one-thread form.  Not for batch or decomposed handles: SU3_EINVAL. */
+ * link, which share the staple's paths and, for FP64 stores, the columns of
+ * the link (for small lattices, whose half-sweep leaves the GPU mostly idle;
+ * the automatic choice for FP64 also takes eight lanes).  Results do not
+ * depend on it, bit for bit.  Phases that measure the plaquette and, for FP32
+ * stores, the repeat-until-accepted heatbath always take the one-thread form.
+ * Not for batch or decomposed handles: SU3_EINVAL. */
 SU3_API int su3_set_lanes(su3_handle h, int lanes);
 
 /* How a sweep is scheduled on the GPU (an implementation choice; the paper's

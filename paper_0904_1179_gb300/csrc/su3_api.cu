@@ -78,16 +78,29 @@ int sm_count() {
   return sms;
 }
 
-// Half-sweeps of small lattices run four lanes per link (k_half_sweep_*_split):
-// there the latency of one update is the bound.  FP64: when the split still
-// gives at most four warps per SM (GB300: 8^4 1.51x, 8^3x16 1.44x faster;
-// beyond that the FP64 pipe is loaded and the idle lanes during the heatbath
-// cost what the shorter staple chain saves: 10^4 1.04x, 12^4 0.61x).  FP32:
-// at most eight warps per SM (8^4 1.35x, 10^4 1.27x; 12^4 would lose: 0.92x).
+// Whether a lattice counts as small: its half-sweeps are bound by the latency of
+// one update and run several lanes per link, and the persistent and chained
+// schedules do not apply.  FP64: at most four warps per SM at four lanes per
+// link.  FP32 (k_half_sweep_f32_split): at most eight (8^4 1.35x, 10^4 1.27x;
+// 12^4 would lose: 0.92x).
 bool use_split(int Vh, int precision) {
   const int sms = sm_count();
   const long long warps_per_sm = precision == SU3_FP64 ? 4 : 8;
   return sms > 0 && 4LL * Vh <= 32LL * warps_per_sm * sms;
+}
+
+// Lanes per link of an FP64 half-sweep launched by itself
+// (k_half_sweep_f64_lanes), by the warps per SM they make.  GB300, ms per sweep
+// with 1 / 4 / 8 lanes: 4^4 0.234 / 0.103 / 0.082, 8^4 (3.4 warps per SM at 8
+// lanes) 0.238 / 0.109 / 0.090, 8^3 x 16 (6.7) 0.242 / 0.123 / 0.133, 10^4 0.246 /
+// 0.127 / 0.151, 12^4 (8.5 warps per SM at 4 lanes) 0.244 / 0.223 / 0.214, 14^4
+// (15.8) 0.246 / 0.250 / 0.332, 16^4 0.300 / 0.463 / 0.555: eight lanes up to four
+// warps per SM (one per scheduler), four up to ten.
+int f64_lanes_auto(int Vh) {
+  const int sms = sm_count();
+  if (sms <= 0) return 1;
+  if (8LL * Vh <= 4 * 32LL * sms) return 8;
+  return 4LL * Vh <= 10 * 32LL * sms ? 4 : 1;
 }
 
 int default_threads(int Vh) {
@@ -152,6 +165,7 @@ HalfSweepArgs half_sweep_args(const su3_lattice* h, int parity) {
   HalfSweepArgs a{};
   a.meas = nullptr;
   a.split = h->split;
+  a.lanes = h->precision == SU3_FP64 ? su3_f64_lanes(h) : 1;
   a.pairs = h->pairs;
   a.pgeom = h->pgeom;
   a.tile2 = h->pairs ? su3k_pair_tile2(h->pgeom, h->threads) : 0;
@@ -279,6 +293,7 @@ int enqueue_sweep_body(su3_lattice* h, bool measured) {
     for (int mu = 0; mu < 4; ++mu)
       for (int p = 0; p < 2; ++p) {
         HalfSweepArgs a = half_sweep_args(h, p);
+        a.chained = mu + p > 0;
         if (measured && p == 1 && mu >= 1) a.meas = h->d_meas_parts + (size_t)(mu - 1) * blocks;
         SU3_CUDA(su3k_launch_half_sweep(a, mu, h->precision, h->stats_on, h->threads, h->stream),
                  "half-sweep launch");
@@ -325,6 +340,8 @@ bool is_batch(const su3_lattice* h) { return h && h->batch; }
 }  // namespace
 
 void su3_release_handle(su3_lattice* h) { release(h); }
+
+int su3_f64_lanes(const su3_lattice* h) { return h->lanes ? h->lanes : f64_lanes_auto(h->geom.Vh); }
 
 int su3_internal_fail(int code, const char* msg) { return su3_fail(code, "%s", msg); }
 
@@ -676,10 +693,11 @@ int su3_set_lanes(su3_handle h, int lanes) {
     return fail(SU3_EINVAL, "su3_set_lanes: not for batch or decomposed handles");
   if (lanes != 0 && lanes != 1 && lanes != 4) return fail(SU3_EINVAL, "su3_set_lanes: lanes %d not 0, 1 or 4", lanes);
   const bool split = lanes == 0 ? use_split(h->geom.Vh, h->precision) : lanes == 4;
-  if (split != h->split) {
+  if (split != h->split || lanes != h->lanes) {
     SU3_CUDA(cudaStreamSynchronize(h->stream), "su3_set_lanes");
     drop_graphs(h);
     h->split = split;
+    h->lanes = lanes;
   }
   return SU3_OK;
 }

@@ -60,6 +60,7 @@ struct DecompArgs {
   int count_stats;   // accumulate acceptance statistics
   int max_tries;     // SU(2) proposals per subgroup (1: one-hit heatbath)
   double* meas;      // fused plaquette: one partial per block of this phase (nullptr: off)
+  int lanes;         // FP64 store: lanes per link
 };
 
 // Origin of sublattice k (index k = k0 + nf*(k1 + nf*...) over the cut directions).
@@ -116,6 +117,20 @@ __global__ void __launch_bounds__(kMaxSweepThreads) k_decomp_half_sweep_f64(Deco
   }
   if (a.count_stats) count_stats_d(c, a.stats);
   if (MEAS) block_partial_d(m, a.meas);
+}
+
+// The same with LPL lanes per link (small lattices; update_link_f64_lanes).
+template <int LPL, bool REPEAT>
+__global__ void __launch_bounds__(kMaxSweepThreads) k_decomp_half_sweep_f64_lanes(DecompArgs a, int mu) {
+  const int k = blockIdx.y;
+  const SubGeometry g = sub_geometry(a.g, a.nf, a.ndmpi, k);
+  const int link = (blockIdx.x * blockDim.x + threadIdx.x) / LPL;
+  const bool active = link < g.in.Vh;
+  const UpdateConsts uc{a.three_over_beta_f64, a.three_over_beta, a.max_tries, sweep_far(a.sweep)};
+  double2* U = (double2*)a.subs + (size_t)k * a.sub_elems;
+  const UpdateCount c =
+      update_link_f64_lanes<LPL, false, REPEAT>(g, U, active ? link : 0, a.parity, mu, a.sweep, a.key, uc, active);
+  if (a.count_stats) count_stats_d(c, a.stats);
 }
 
 template <int MU, bool EFT, bool REPEAT, bool MEAS>
@@ -213,7 +228,13 @@ __global__ void k_decomp_move_f32_pairs(SubGeometry base, int nf, int ndmpi, flo
 
 template <int MU, bool REPEAT, bool MEAS>
 cudaError_t launch_update_form(const DecompArgs& a, int precision, const dim3& grid, int threads, cudaStream_t s) {
-  if (precision == SU3_FP64)
+  if (precision == SU3_FP64 && !MEAS && a.lanes > 1) {
+    const dim3 lgrid((unsigned)(((long long)a.lanes * a.g.in.Vh + threads - 1) / threads), grid.y);
+    if (a.lanes == 8)
+      k_decomp_half_sweep_f64_lanes<8, REPEAT><<<lgrid, threads, 0, s>>>(a, MU);
+    else
+      k_decomp_half_sweep_f64_lanes<4, REPEAT><<<lgrid, threads, 0, s>>>(a, MU);
+  } else if (precision == SU3_FP64)
     k_decomp_half_sweep_f64<REPEAT, MEAS><<<grid, threads, 0, s>>>(a, MU);
   else if (precision == SU3_FP32_EFT)
     k_decomp_half_sweep_f32<MU, true, REPEAT, MEAS><<<grid, threads, 0, s>>>(a);
@@ -306,6 +327,7 @@ DecompArgs decomp_args(const su3_lattice* h, int parity) {
   a.stats = h->d_stats;
   a.max_tries = h->max_tries;
   a.meas = nullptr;
+  a.lanes = h->precision == SU3_FP64 ? su3_f64_lanes(h) : 1;
   return a;
 }
 

@@ -106,20 +106,15 @@ SU3_HD long long fx_merge(const facc& s) {
 #endif
   return s.hh + 4LL * ci;
 }
-SU3_HD fx fx_norm(const facc& s) {
-  const unsigned long long u = (unsigned long long)fx_merge(s);
+SU3_HD fx fx_norm_merged(long long m) {
+  const unsigned long long u = (unsigned long long)m;
   return fx_make((int)(uint32_t)(u >> 30), fx_i2f((int)(((uint32_t)u << 2) + 0x80000000u)));
 }
-// Sums of reals (not of products): h = round(hh / 4), for the unit 4 u.
-SU3_HD fx fx_norm_sum(const facc& s) {
-  const unsigned long long u = (unsigned long long)s.hh;
-  const int rem = (int)(((uint32_t)u << 30) + 0x80000000u);
-  return fx_make((int)(uint32_t)(u >> 2), fx_fma(s.c, 0.25f, fx_i2f(rem)));
-}
+SU3_HD fx fx_norm(const facc& s) { return fx_norm_merged(fx_merge(s)); }
 // A merged sum of unit 2^-60 in the unit 2^-28 (the high word; 2^31 added
 // before).
-SU3_HD fx fx_norm_high(const facc& s) {
-  const unsigned long long u = (unsigned long long)s.hh;
+SU3_HD fx fx_norm_high(long long m) {
+  const unsigned long long u = (unsigned long long)m;
   return fx_make((int)(uint32_t)(u >> 32), fx_i2f((int)((uint32_t)u ^ 0x80000000u)));
 }
 // Where the accumulator of an fx_norm starts.
@@ -235,31 +230,27 @@ SU3_HD void cfx_msub_cc(cfacc& s, const cfx& a, const cfx& b) {
 }
 SU3_HD cfacc cfx_zero() { return cfacc{fx_zero(), fx_zero()}; }
 SU3_HD cfx cfx_norm(const cfacc& s) { return cfx{fx_norm(s.re), fx_norm(s.im)}; }
-SU3_HD cfx cfx_norm_high(const cfacc& s) { return cfx{fx_norm_high(s.re), fx_norm_high(s.im)}; }
 
 // ---------------------------------------------------------------------------
-// Staple in this arithmetic.  A three-link path's rows 0,1 come out in the unit
-// 2^-30.  The staple's rows 0,1 are sums of at most six of them: the h summed
-// in 64 bits, the l in FP32; its row 2 is accumulated from the completions
-// conj(row0 x row1) in the unit 2^-60.
+// Staple in this arithmetic: the sum of three-link paths as 64-bit integers in
+// units of 2^-60 (at most six paths: 6 2^60 < 2^63).  Integer sums do not depend
+// on their order, so lanes that share a link's paths add them up to the same
+// bits as one thread does.  Rows 0,1 of a path are the merged sums of its last
+// product, row 2 is the merged completion conj(row0 x row1).
 // ---------------------------------------------------------------------------
 struct fx_rows01 {
   cfx e[2][3];
+  long long m[2][3][2];  // merged, with the 2^29 of fx_zero
 };
 struct fx_staple {
-  facc r01[2][3][2];  // sums of h and l (rows 0, 1; re, im)
-  cfacc r2[3];          // merged
+  long long r[3][3][2];
 };
 
 SU3_HD void fx_staple_zero(fx_staple& A) {
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int k = 0; k < 3; ++k)
-#pragma unroll
-      for (int c = 0; c < 2; ++c) A.r01[i][k][c] = facc{2, 0.0f};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) A.r2[k] = cfacc{{1LL << 31, 0.0f}, {1LL << 31, 0.0f}};
+    for (int k = 0; k < 3; ++k) A.r[i][k][0] = A.r[i][k][1] = 0;
 }
 
 // A += F (rows 0,1 given, row 2 completed).
@@ -268,51 +259,36 @@ SU3_HD void fx_staple_add(fx_staple& A, const fx_rows01& F) {
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-      A.r01[i][k][0].hh += F.e[i][k].re.h;
-      A.r01[i][k][1].hh += F.e[i][k].im.h;
-      A.r01[i][k][0].c = fx_add(A.r01[i][k][0].c, F.e[i][k].re.l);
-      A.r01[i][k][1].c = fx_add(A.r01[i][k][1].c, F.e[i][k].im.l);
+      A.r[i][k][0] += F.m[i][k][0];
+      A.r[i][k][1] += F.m[i][k][1];
     }
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const int a = (k + 1) % 3, b = (k + 2) % 3;
-    // the cross terms path by path: six paths' in one FP32 sum lose up to three bits
-    cfacc s{{A.r2[k].re.hh, 0.0f}, {A.r2[k].im.hh, 0.0f}};
+    cfacc s{{A.r[2][k][0], 0.0f}, {A.r[2][k][1], 0.0f}};
     cfx_mac_cc(s, F.e[0][a], F.e[1][b]);
     cfx_msub_cc(s, F.e[0][b], F.e[1][a]);
-    A.r2[k].re.hh = fx_merge(s.re);
-    A.r2[k].im.hh = fx_merge(s.im);
+    A.r[2][k][0] = fx_merge(s.re);
+    A.r[2][k][1] = fx_merge(s.im);
   }
 }
 
-// The staple as a matrix in the unit 2^-28 (entries up to 6).
+// One entry of row i of a staple of `paths` paths, in the unit 2^-28 (entries up
+// to 6).
+SU3_HD fx fx_staple_entry(long long m, int i, int paths) {
+  return fx_norm_high(m + ((1LL << 31) - (i < 2 ? (long long)paths << 29 : 0LL)));
+}
 struct fx_mat {
   cfx e[3][3];
 };
-SU3_HD fx_mat fx_staple_mat(const fx_staple& A) {
+SU3_HD fx_mat fx_staple_mat(const fx_staple& A, int paths) {
   fx_mat m;
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < 3; ++i)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      m.e[i][k].re = fx_norm_sum(A.r01[i][k][0]);
-      m.e[i][k].im = fx_norm_sum(A.r01[i][k][1]);
-    }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) m.e[2][k] = cfx_norm_high(A.r2[k]);
+    for (int k = 0; k < 3; ++k)
+      m.e[i][k] = cfx{fx_staple_entry(A.r[i][k][0], i, paths), fx_staple_entry(A.r[i][k][1], i, paths)};
   return m;
-}
-
-// Row 2 of an SU(3) matrix (unit 2^-30) from rows 0 and 1: conj(row0 x row1).
-SU3_HD void fx_complete_row2(fx_mat& m) {
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int a = (k + 1) % 3, b = (k + 2) % 3;
-    cfacc s = cfx_zero();
-    cfx_mac_cc(s, m.e[0][a], m.e[1][b]);
-    cfx_msub_cc(s, m.e[0][b], m.e[1][a]);
-    m.e[2][k] = cfx_norm(s);
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -324,43 +300,74 @@ SU3_HD void fx_complete_row2(fx_mat& m) {
 // rows unchanged, where a coefficient exceeds 2^-31: the caller takes the
 // FP64 Gram-Schmidt.
 // ---------------------------------------------------------------------------
-// A small sum in units of 2^-60 as FP32 (ok = false where it is not small):
-// its integer part reaches 2.5 2^30 (cancelled by the FP32 part, the cross
-// terms of h and l), so it is taken without its last four bits.
-SU3_HD float fx_small(const facc& s, bool& ok) {
-  const float v = fx_fma(fx_i2f((int)(s.hh >> 4)), 16.0f, fx_mul(s.c, 0x1p-32f));
-  ok = ok && s.hh < (1LL << 34) && s.hh > -(1LL << 34) && v < 0x1p29f && v > -0x1p29f;
-  return v;
+// One column's part of |r0|^2, |r1|^2, Re d and Im d, merged; the columns' parts
+// add up as integers.
+struct fx_gram {
+  long long n0, n1, dr, di;
+};
+SU3_HD fx_gram fx_gram_column(const cfx& a, const cfx& b) {
+  facc n0{0, 0.0f}, n1{0, 0.0f};
+  cfacc d{{0, 0.0f}, {0, 0.0f}};
+  fx_mac(n0, a.re, a.re);
+  fx_mac(n0, a.im, a.im);
+  fx_mac(n1, b.re, b.re);
+  fx_mac(n1, b.im, b.im);
+  cfx_mac_ca(d, a, b);
+  return fx_gram{fx_merge(n0), fx_merge(n1), fx_merge(d.re), fx_merge(d.im)};
+}
+// The coefficients of the correction from the whole sums; false where one is
+// 2^-31 or more.
+struct fx_gs {
+  float s0, s1, cr, ci;
+};
+SU3_HD bool fx_gs_coefficients(const fx_gram& g, fx_gs& c) {
+  const long long n0 = g.n0 - (1LL << 60), n1 = g.n1 - (1LL << 60), lim = 1LL << 29;
+  const bool ok = n0 < lim && n0 > -lim && n1 < lim && n1 > -lim && g.dr < lim && g.dr > -lim && g.di < lim && g.di > -lim;
+  // f is in units of 2^-30, l of 2^-62: a coefficient in units of 2^-60 gets the factor 2^-28
+  c.s0 = fx_mul(fx_i2f((int)n0), -0x1p-29f);
+  c.s1 = fx_mul(fx_i2f((int)n1), -0x1p-29f);
+  c.cr = fx_mul(fx_i2f((int)g.dr), -0x1p-28f);
+  c.ci = fx_mul(fx_i2f((int)g.di), -0x1p-28f);
+  return ok;
+}
+SU3_HD void fx_gs_column(const fx_gs& c, cfx& a, cfx& b) {
+  b.re.l = fx_fma(c.cr, a.re.f, fx_fma(-c.ci, a.im.f, fx_fma(c.s1, b.re.f, b.re.l)));
+  b.im.l = fx_fma(c.cr, a.im.f, fx_fma(c.ci, a.re.f, fx_fma(c.s1, b.im.f, b.im.l)));
+  a.re.l = fx_fma(c.s0, a.re.f, a.re.l);
+  a.im.l = fx_fma(c.s0, a.im.f, a.im.l);
 }
 
 SU3_HD bool fx_reunitarise(fx_mat& u) {
-  // half of the four bits that fx_small drops
-  facc n0{8 - (1LL << 60), 0.0f}, n1 = n0;
-  cfacc d{{8, 0.0f}, {8, 0.0f}};
+  fx_gram g{0, 0, 0, 0};
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    fx_mac(n0, u.e[0][k].re, u.e[0][k].re);
-    fx_mac(n0, u.e[0][k].im, u.e[0][k].im);
-    fx_mac(n1, u.e[1][k].re, u.e[1][k].re);
-    fx_mac(n1, u.e[1][k].im, u.e[1][k].im);
-    cfx_mac_ca(d, u.e[0][k], u.e[1][k]);
+    const fx_gram q = fx_gram_column(u.e[0][k], u.e[1][k]);
+    g.n0 += q.n0;
+    g.n1 += q.n1;
+    g.dr += q.dr;
+    g.di += q.di;
   }
-  bool ok = true;
-  const float e0 = fx_small(n0, ok), e1 = fx_small(n1, ok), dr = fx_small(d.re, ok), di = fx_small(d.im, ok);
-  if (!ok) return false;
-  // f is in units of 2^-30, l of 2^-62: a coefficient in units of 2^-60 gets the factor 2^-28
-  const float s0 = fx_mul(e0, -0x1p-29f), s1 = fx_mul(e1, -0x1p-29f);
-  const float cr = fx_mul(dr, -0x1p-28f), ci = fx_mul(di, -0x1p-28f);
+  fx_gs c;
+  if (!fx_gs_coefficients(g, c)) return false;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    cfx& a = u.e[0][k];
-    cfx& b = u.e[1][k];
-    b.re.l = fx_fma(cr, a.re.f, fx_fma(-ci, a.im.f, fx_fma(s1, b.re.f, b.re.l)));
-    b.im.l = fx_fma(cr, a.im.f, fx_fma(ci, a.re.f, fx_fma(s1, b.im.f, b.im.l)));
-    a.re.l = fx_fma(s0, a.re.f, a.re.l);
-    a.im.l = fx_fma(s0, a.im.f, a.im.l);
-  }
+  for (int k = 0; k < 3; ++k) fx_gs_column(c, u.e[0][k], u.e[1][k]);
   return true;
+}
+
+// Entry k of row 2 of an SU(3) matrix from entries a = k + 1, b = k + 2 (mod 3) of
+// rows 0 and 1: conj(x0a x1b - x0b x1a).
+SU3_HD cfx fx_row2_entry(const cfx& x0a, const cfx& x0b, const cfx& x1a, const cfx& x1b) {
+  cfacc s = cfx_zero();
+  cfx_mac_cc(s, x0a, x1b);
+  cfx_msub_cc(s, x0b, x1a);
+  return cfx_norm(s);
+}
+SU3_HD void fx_complete_row2(fx_mat& m) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int a = (k + 1) % 3, b = (k + 2) % 3;
+    m.e[2][k] = fx_row2_entry(m.e[0][a], m.e[0][b], m.e[1][a], m.e[1][b]);
+  }
 }
 
 }  // namespace su3dev

@@ -124,7 +124,6 @@ SU3_HD long long fx_neg_log(unsigned long long m) {
 struct fx_cs {
   fx c, s;
 };
-template <bool SIN>
 SU3_HD fx_cs fx_cossin(unsigned long long m) {
   const uint32_t o = (uint32_t)(m >> 50);  // octant; odd ones are mirrored
   unsigned long long w = m & ((1ull << 50) - 1);
@@ -153,17 +152,10 @@ SU3_HD fx_cs fx_cossin(unsigned long long m) {
   fx_mac(b, s0, ct);
   fx_mac(b, c0, st);
   const bool swap = (o + 1) & 2, negc = (o + 2) & 4, negs = o & 4;
-  fx_cs r;
-  if (SIN) {
-    const fx x = fx_norm(a), y = fx_norm(b);
-    r.c = swap ? y : x;
-    r.s = swap ? x : y;
-    r.s = negs ? fx_neg(r.s) : r.s;
-  } else {
-    r.c = fx_norm(swap ? b : a);
-    r.s = r.c;
-  }
+  const fx x = fx_norm(a), y = fx_norm(b);
+  fx_cs r{swap ? y : x, swap ? x : y};
   r.c = negc ? fx_neg(r.c) : r.c;
+  r.s = negs ? fx_neg(r.s) : r.s;
   return r;
 }
 
@@ -245,42 +237,62 @@ SU3_HD bool fx_direction(const long long rI[4], fx v[4], double* ik) {
   return true;
 }
 
-// One Kennedy-Pendleton proposal from the uniforms m[0..5] (odd integers,
-// u = m 2^-53) at 1/alpha = inv_alpha: delta = -(ln u0 + cos^2(2 pi u1) ln u2) /
-// alpha; accepted if u3^2 <= 1 - delta/2, then a0 = 1 - delta and a1..a3 on the
-// sphere of radius sqrt(1 - a0^2) in the direction of u4, u5.
-SU3_HD bool fx_propose(const unsigned long long m[6], double inv_alpha, fx a[4]) {
-  // cos^2 = (1 + cos(4 pi u1)) / 2
-  const fx c2 = fx_cossin<false>((m[1] << 1) & ((1ull << 53) - 1)).c;
-  const fx cc = fx_from_i62((fx_to_i62(c2) + (1LL << 62)) >> 1);
-  // S = -ln u0 - cos^2 ln u2 (at most 74) in units of 2^-56; cos^2's integer part
-  // times both words of the second logarithm (up to 37: its low word is too
-  // large for an FP32 part)
-  const long long l0 = fx_neg_log(m[0]), l2 = fx_neg_log(m[2]);
-  const int l2l = (int)(uint32_t)l2, l2h = (int)(l2 >> 32) + (int)((uint32_t)l2l >> 31);
-  const long long S = (l0 >> 1) + (((long long)cc.h * l2h) << 1) + (((long long)cc.h * l2l) >> 31) +
-                      fx_f2i(fx_mul(fx_mul(cc.l, 0x1p-31f), fx_i2f(l2h)));
+// A Kennedy-Pendleton proposal from the uniforms m[0..5] (odd integers, u = m
+// 2^-53): delta = -(ln u0 + cos^2(2 pi u1) ln u2) / alpha; accepted if u3^2 <= 1 -
+// delta/2, then a0 = 1 - delta and a1..a3 on the sphere of radius sqrt(1 -
+// a0^2) in the direction of u4, u5.  fx_draw is the part that does not depend
+// on the staple, fx_propose the rest.
+struct fx_drawn {
+  long long S;   // -ln u0 - cos^2 ln u2 in units of 2^-56
+  long long u3;  // u3 in units of 2^-62
+  fx d[3];       // direction: sin(theta) cos(phi), sin(theta) sin(phi), cos(theta)
+};
+SU3_HD fx_drawn fx_draw(const unsigned long long m[6]) {
+  fx_drawn r;
+  // cos^2 = (1 + cos(4 pi u1)) / 2; the two logarithms and the two angles in one
+  // piece of code (instruction cache)
+  long long l0 = 0, l2 = 0;
+  fx_cs c2{}, phi{};
 #ifdef __CUDA_ARCH__
-  const double Sd = __ll2double_rn(S);
+#pragma unroll 1
+#endif
+  for (int n = 0; n < 2; ++n) {
+    l0 = l2;
+    c2 = phi;
+    l2 = fx_neg_log(n == 0 ? m[0] : m[2]);
+    phi = fx_cossin(n == 0 ? (m[1] << 1) & ((1ull << 53) - 1) : m[5]);
+  }
+  const fx cc = fx_from_i62((fx_to_i62(c2.c) + (1LL << 62)) >> 1);
+  // S is at most 74; cos^2's integer part times both words of the second logarithm
+  // (up to 37: its low word is too large for an FP32 part)
+  const int l2l = (int)(uint32_t)l2, l2h = (int)(l2 >> 32) + (int)((uint32_t)l2l >> 31);
+  r.S = (l0 >> 1) + (((long long)cc.h * l2h) << 1) + (((long long)cc.h * l2l) >> 31) +
+        fx_f2i(fx_mul(fx_mul(cc.l, 0x1p-31f), fx_i2f(l2h)));
+  r.u3 = (long long)(m[3] << 9);
+  const long long u4 = (long long)(m[4] << 9);
+  const fx sn = fx_two_root(u4);
+  r.d[0] = fx_mulv(sn, phi.c);
+  r.d[1] = fx_mulv(sn, phi.s);
+  r.d[2] = fx_from_i62((1LL << 62) - 2 * u4);
+  return r;
+}
+SU3_HD bool fx_propose(const fx_drawn& w, double inv_alpha, fx a[4]) {
+#ifdef __CUDA_ARCH__
+  const double Sd = __ll2double_rn(w.S);
 #else
-  const double Sd = (double)S;
+  const double Sd = (double)w.S;
 #endif
   const double delta = Sd * 0x1p-56 * inv_alpha;
   if (!(delta < 2.0)) return false;
   const long long p62 = fx_i62_from_double(delta) >> 1;  // delta / 2
-  const fx u3 = fx_from_i62((long long)(m[3] << 9));
+  const fx u3 = fx_from_i62(w.u3);
   facc t{0, 0.0f};
   fx_mac(t, u3, u3);
   if (fx_merge(t) > (1LL << 60) - (p62 >> 2)) return false;
-  const long long u4 = (long long)(m[4] << 9);
-  const fx rho = fx_two_root(p62), sn = fx_two_root(u4);
-  const fx ct = fx_from_i62((1LL << 62) - 2 * u4);
-  const fx_cs phi = fx_cossin<true>(m[5]);
-  const fx rs = fx_mulv(rho, sn);
+  const fx rho = fx_two_root(p62);
   a[0] = fx_from_i62((1LL << 62) - 2 * p62);
-  a[1] = fx_mulv(rs, phi.c);
-  a[2] = fx_mulv(rs, phi.s);
-  a[3] = fx_mulv(rho, ct);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) a[c + 1] = fx_mulv(rho, w.d[c]);
   return true;
 }
 

@@ -1,5 +1,5 @@
 // su3_kernels_f64.cu -- the half-sweeps of the FP64 store (see su3_kernels.cu):
-// one thread per link, or four lanes per link on small lattices.  The update
+// one thread per link, or four or eight lanes per link on small lattices.  The update
 // runs on the integer and FP32 pipes (su3_fx.cuh); the direction mu is a run-time
 // argument, so that one copy of its code serves the four directions.
 //
@@ -92,64 +92,18 @@ __global__ void SU3_F64_BOUNDS
   report_sweep_item(qa, layers, it);
 }
 
-// A small lattice's half-sweep has too few links to fill the GPU, and each
-// link's update is a long dependent chain: the time is its latency.  Here four
-// lanes share one link: lanes 0, 1, 2 compute rows 0,1 of the two staple paths
-// of the first, second and third direction nu != mu at the same time, lane 0
-// gathers them and adds them up in the single-thread order (forward then
-// backward path, nu ascending, row 2 formed in the accumulation), so the
-// staple, and everything after it, is bit for bit that of k_half_sweep_f64.
-// Lane 3 only idles.
-__device__ __forceinline__ fx_rows01 shfl_rows01(const fx_rows01& m, int src) {
-  fx_rows01 r;
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const fx &a = m.e[i][k].re, &b = m.e[i][k].im;
-      r.e[i][k].re = fx_make(__shfl_sync(0xffffffffu, a.h, src), __shfl_sync(0xffffffffu, a.l, src));
-      r.e[i][k].im = fx_make(__shfl_sync(0xffffffffu, b.h, src), __shfl_sync(0xffffffffu, b.l, src));
-    }
-  return r;
-}
-
-__global__ void __launch_bounds__(kMaxSweepThreads) k_half_sweep_f64_split(HalfSweepArgs args, int mu, int stats) {
-  const Geometry& g = args.geom;
-  const int p = args.parity;
+// A small lattice's half-sweep: LPL lanes per link (update_link_f64_lanes).
+// Launched as a programmatic dependent of the half-sweep before it, a block
+// draws its random numbers while that one drains.
+template <int LPL, bool REPEAT>
+__global__ void __launch_bounds__(kMaxSweepThreads) k_half_sweep_f64_lanes(HalfSweepArgs args, int mu, int stats) {
+  signal_dependents();
   const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  const int link = gid >> 2, part = gid & 3;
-  const bool active = link < g.Vh;
-  const int h = active ? link : 0;  // a group past the end works on site 0 and discards it (shuffles stay converged)
-  double2* U = (double2*)args.links;
-  const UpdateConsts uc = update_consts(args);
-  UpdateCount c{0, 0};
-  if (*(volatile const int*)uc.far) {  // links far from SU(3): one lane per link
-    if (part == 0 && active) c = update_link_f64_far<false>(g, U, h, p, mu, *args.sweep, args.key, uc, nullptr);
-  } else {
-    const Site st = site_of(g, h, p);
-    fx_rows01 F{}, B{};
-    if (part < 3) {
-      const int nu = part < mu ? part : part + 1;
-      const int h_mnu = nb_half_rt(g, st, nu, -1);
-      F = staple_path_fx<false>(U, g.Vh, p, mu, nu, false, nb_half_rt(g, st, mu, +1), nb_half_rt(g, st, nu, +1), h);
-      B = staple_path_fx<false>(U, g.Vh, p, mu, nu, true, nb_half2_rt(g, st, mu, nu), h_mnu, h_mnu);
-    }
-    const int lane0 = (threadIdx.x & 31) & ~3;
-    fx_staple A;
-    fx_staple_zero(A);
-    fx_staple_add(A, F);
-    fx_staple_add(A, B);
-#pragma unroll 1
-    for (int k = 1; k < 3; ++k) {
-      fx_staple_add(A, shfl_rows01(F, lane0 + k));
-      fx_staple_add(A, shfl_rows01(B, lane0 + k));
-    }
-    if (part == 0 && active) {
-      const fx_mat m = fx_staple_mat(A);
-      c = heatbath_fx<false, false, false>(g, U, h, p, mu, *args.sweep, (uint32_t)canon(g, st), args.key, uc, m, m,
-                                           nullptr);
-    }
-  }
+  const int link = gid / LPL;
+  const bool active = link < args.geom.Vh;  // a group past the end works on site 0 (shuffles stay converged)
+  const UpdateCount c = update_link_f64_lanes<LPL, false, REPEAT>(args.geom, (double2*)args.links, active ? link : 0,
+                                                                 args.parity, mu, args.sweep, args.key,
+                                                                 update_consts(args), active);
   if (stats) count_stats<true>(c, args.stats);
 }
 
@@ -193,8 +147,21 @@ cudaError_t su3k_launch_half_sweep_f64(const HalfSweepArgs& a, int mu, bool stat
       k_half_sweep_f64<true, true><<<blocks, threads, 0, s>>>(a, mu, 0);
     else
       k_half_sweep_f64<false, true><<<blocks, threads, 0, s>>>(a, mu, 0);
-  } else if (a.split && !repeat) {
-    k_half_sweep_f64_split<<<(4 * a.geom.Vh + threads - 1) / threads, threads, 0, s>>>(a, mu, st);
+  } else if (a.lanes > 1) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(((long long)a.lanes * a.geom.Vh + threads - 1) / threads));
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.chained ? 1 : 0;
+    if (a.lanes == 8)
+      return repeat ? cudaLaunchKernelEx(&cfg, k_half_sweep_f64_lanes<8, true>, a, mu, st)
+                    : cudaLaunchKernelEx(&cfg, k_half_sweep_f64_lanes<8, false>, a, mu, st);
+    return repeat ? cudaLaunchKernelEx(&cfg, k_half_sweep_f64_lanes<4, true>, a, mu, st)
+                  : cudaLaunchKernelEx(&cfg, k_half_sweep_f64_lanes<4, false>, a, mu, st);
   } else if (repeat) {
     k_half_sweep_f64<true, false><<<blocks, threads, 0, s>>>(a, mu, st);
   } else {

@@ -48,7 +48,8 @@ struct su3_lattice {
   int meas_cap = 0;
   int threads = kSu3DefaultThreads;
   int max_tries = 1;  // SU(2) proposals per subgroup (1: one-hit heatbath)
-  bool split = false;  // small FP64 lattice: four lanes per link update
+  bool split = false;  // small lattice: several lanes per link update
+  int lanes = 0;       // as set by su3_set_lanes (0: automatic)
   bool pairs = false;  // FP32 store in the site-paired layout (L3 a multiple of 4)
   su3dev::Geometry geom{};
   su3dev::Geometry pgeom{};  // pair lattice L0 x L1 x L2 x L3/2 (pairs only)
@@ -75,6 +76,8 @@ int su3_sync(su3_lattice* h, const char* what);
 // Synchronises.
 int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pairs, double* host, bool get,
                  const char* what);
+// Lanes per link of an FP64 half-sweep of this lattice (1, 4 or 8).
+int su3_f64_lanes(const su3_lattice* h);
 // Free a handle and everything it owns (batch part included).
 void su3_release_handle(su3_lattice* h);
 // Free the batch part of a handle (defined in su3_batch.cu).

@@ -348,38 +348,40 @@ struct FxLink {
   }
 };
 
-// Rows 0,1 of X Y^+ Z.
+// Rows 0,1 of X Y^+ Z: the two products in one piece of code, run twice
+// (instruction cache; see staple_path_fx).  Yd: the link Y^+.
 template <bool CG>
-__device__ __forceinline__ fx_rows01 path_fx(const FxLink<CG>& X, const FxLink<CG>& Y, const FxLink<CG>& Z) {
-  cfx x[2][3], t[2][3];
+__device__ __forceinline__ fx_rows01 path_fx(const FxLink<CG>& X, const FxLink<CG>& Yd, const FxLink<CG>& Z) {
+  fx_rows01 f;
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) x[i][k] = X.at(i, k);
+    for (int k = 0; k < 3; ++k) f.e[i][k] = X.at(i, k);
+  FxLink<CG> L = Yd;
+#pragma unroll 1
+  for (int n = 0; n < 2; ++n) {
+    cfx t[2][3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    cfacc s[2] = {cfx_zero(), cfx_zero()};
+    for (int k = 0; k < 3; ++k) {
+      cfacc s[2] = {cfx_zero(), cfx_zero()};
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const cfx y = Y.at(k, j);
-      cfx_mac_cb(s[0], x[0][j], y);
-      cfx_mac_cb(s[1], x[1][j], y);
+      for (int j = 0; j < 3; ++j) {
+        const cfx z = L.at(j, k);
+        cfx_mac(s[0], f.e[0][j], z);
+        cfx_mac(s[1], f.e[1][j], z);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        f.m[i][k][0] = fx_merge(s[i].re);
+        f.m[i][k][1] = fx_merge(s[i].im);
+        t[i][k] = cfx{fx_norm_merged(f.m[i][k][0]), fx_norm_merged(f.m[i][k][1])};
+      }
     }
-    t[0][k] = cfx_norm(s[0]);
-    t[1][k] = cfx_norm(s[1]);
-  }
-  fx_rows01 f;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    cfacc s[2] = {cfx_zero(), cfx_zero()};
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const cfx z = Z.at(j, k);
-      cfx_mac(s[0], t[0][j], z);
-      cfx_mac(s[1], t[1][j], z);
-    }
-    f.e[0][k] = cfx_norm(s[0]);
-    f.e[1][k] = cfx_norm(s[1]);
+      for (int k = 0; k < 3; ++k) f.e[i][k] = t[i][k];
+    L = Z;
   }
   return f;
 }
@@ -393,7 +395,7 @@ template <bool CG>
 __device__ __forceinline__ fx_rows01 staple_path_fx(const void* U, int Vh, int p, int mu, int nu, bool backward, int hx,
                                                     int hy, int hz) {
   const int q = p ^ 1;
-  return path_fx(FxLink<CG>(U, nu, backward ? p : q, hx, Vh, backward), FxLink<CG>(U, mu, q, hy, Vh),
+  return path_fx(FxLink<CG>(U, nu, backward ? p : q, hx, Vh, backward), FxLink<CG>(U, mu, q, hy, Vh, true),
                  FxLink<CG>(U, nu, backward ? q : p, hz, Vh, !backward));
 }
 
@@ -414,9 +416,9 @@ __device__ __forceinline__ fx_mat staple_fx(const G& g, const void* U, const S& 
     const int hy = nb_half_rt(g, st, nu, backward ? -1 : +1);
     fx_staple_add(A, staple_path_fx<CG>(U, g.Vh, p, mu, nu, backward, backward ? nb_half2_rt(g, st, mu, nu) : h_pmu, hy,
                                         backward ? hy : h));
-    if (Apart && backward && nu == mu - 1) *Apart = fx_staple_mat(A);
+    if (Apart && backward && nu == mu - 1) *Apart = fx_staple_mat(A, path + 1);
   }
-  return fx_staple_mat(A);
+  return fx_staple_mat(A, 6);
 }
 
 // A sum of products of units 2^-30 and 2^-28 merged (units of 2^-58).  The cross
@@ -424,6 +426,61 @@ __device__ __forceinline__ fx_mat staple_fx(const G& g, const void* U, const S& 
 // 2^-90: they are taken to 2^-54.
 __device__ __forceinline__ long long fx_merge_wide(const facc& s) {
   return s.hh + 16LL * __float2int_rn(__fmul_rn(s.c, 0x1p-36f));
+}
+
+// Column c's part of 2r (su2_projection), merged (units of 2^-58): u_ic, u_jc and
+// A_ci, A_cj.
+__device__ __forceinline__ void fx_projection_column(const cfx& ui, const cfx& uj, const cfx& ai, const cfx& aj,
+                                                     long long r[4]) {
+  facc w[4] = {{0, 0.0f}, {0, 0.0f}, {0, 0.0f}, {0, 0.0f}};
+  fx_mac(w[0], ui.re, ai.re);
+  fx_msub(w[0], ui.im, ai.im);
+  fx_mac(w[0], uj.re, aj.re);
+  fx_msub(w[0], uj.im, aj.im);
+  fx_mac(w[1], ui.re, aj.im);
+  fx_mac(w[1], ui.im, aj.re);
+  fx_mac(w[1], uj.re, ai.im);
+  fx_mac(w[1], uj.im, ai.re);
+  fx_mac(w[2], ui.re, aj.re);
+  fx_msub(w[2], ui.im, aj.im);
+  fx_msub(w[2], uj.re, ai.re);
+  fx_mac(w[2], uj.im, ai.im);
+  fx_mac(w[3], ui.re, ai.im);
+  fx_mac(w[3], ui.im, ai.re);
+  fx_msub(w[3], uj.re, aj.im);
+  fx_msub(w[3], uj.im, aj.re);
+#pragma unroll
+  for (int n = 0; n < 4; ++n) r[n] = fx_merge_wide(w[n]);
+}
+
+// Entries of one column of the two rows that R turns (R10 = -conj(R01), R11 =
+// conj(R00)).
+__device__ __forceinline__ void fx_rotate_column(const cfx& R00, const cfx& R01, cfx& ui, cfx& uj) {
+  const cfx R10{fx_neg(R01.re), R01.im}, R11 = cfx_conj(R00);
+  cfacc z = cfx_zero();
+  cfx_mac(z, R00, ui);
+  cfx_mac(z, R01, uj);
+  cfacc w = cfx_zero();
+  cfx_mac(w, R10, ui);
+  cfx_mac(w, R11, uj);
+  ui = cfx_norm(z);
+  uj = cfx_norm(w);
+}
+
+// The uniforms of proposal tr of subgroup sub.
+template <typename KEY>
+__device__ __forceinline__ fx_drawn fx_draw_at(uint32_t s, int mu, int sub, int tr, uint64_t t, const KEY& key) {
+  unsigned long long m[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll 1
+  for (int call = 0; call < 3; ++call) {
+    const uint32_t w1 = (uint32_t)(mu | (sub << 2) | (call << 4)) | ((uint32_t)tr << 6);
+    const uint4 b = philox4x32_10(rng_counter(s, w1, t, kTagUpdate), key);
+#pragma unroll
+    for (int n = 0; n < 4; ++n) m[n] = m[n + 2];
+    m[4] = fx_uniform(b.x, b.y);
+    m[5] = fx_uniform(b.z, b.w);
+  }
+  return fx_draw(m);
 }
 
 // Everything after the staple A0 (unit 2^-28): three SU(2) heatbath steps,
@@ -446,29 +503,14 @@ __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h
   fx_mat A = A0;
 #pragma unroll 1
   for (int sub = 0; sub < 3; ++sub) {
-    // 2r as in su2_projection, each component one sum
-    facc w[4] = {{0, 0.0f}, {0, 0.0f}, {0, 0.0f}, {0, 0.0f}};
+    long long r[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const cfx &ui = u.e[0][c], &uj = u.e[1][c], &ai = A.e[c][0], &aj = A.e[c][1];
-      fx_mac(w[0], ui.re, ai.re);
-      fx_msub(w[0], ui.im, ai.im);
-      fx_mac(w[0], uj.re, aj.re);
-      fx_msub(w[0], uj.im, aj.im);
-      fx_mac(w[1], ui.re, aj.im);
-      fx_mac(w[1], ui.im, aj.re);
-      fx_mac(w[1], uj.re, ai.im);
-      fx_mac(w[1], uj.im, ai.re);
-      fx_mac(w[2], ui.re, aj.re);
-      fx_msub(w[2], ui.im, aj.im);
-      fx_msub(w[2], uj.re, ai.re);
-      fx_mac(w[2], uj.im, ai.im);
-      fx_mac(w[3], ui.re, ai.im);
-      fx_mac(w[3], ui.im, ai.re);
-      fx_msub(w[3], uj.re, aj.im);
-      fx_msub(w[3], uj.im, aj.re);
+      long long q[4];
+      fx_projection_column(u.e[0][c], u.e[1][c], A.e[c][0], A.e[c][1], q);
+#pragma unroll
+      for (int n = 0; n < 4; ++n) r[n] += q[n];
     }
-    const long long r[4] = {fx_merge_wide(w[0]), fx_merge_wide(w[1]), fx_merge_wide(w[2]), fx_merge_wide(w[3])};
     fx v[4], a[4];
     double ik;
     bool accepted = false;
@@ -477,16 +519,8 @@ __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h
       const int ntries = REPEAT ? uc.max_tries : 1;
 #pragma unroll 1
       for (int tr = 0; tr < ntries && !accepted; ++tr) {
-        unsigned long long m[6];
-#pragma unroll
-        for (int call = 0; call < 3; ++call) {
-          const uint32_t w1 = (uint32_t)(mu | (sub << 2) | (call << 4)) | ((uint32_t)tr << 6);
-          const uint4 b = philox4x32_10(rng_counter(s, w1, t, kTagUpdate), key);
-          m[2 * call] = fx_uniform(b.x, b.y);
-          m[2 * call + 1] = fx_uniform(b.z, b.w);
-        }
         ++cnt.proposed;
-        accepted = fx_propose(m, inv_alpha, a);
+        accepted = fx_propose(fx_draw_at(s, mu, sub, tr, t, key), inv_alpha, a);
       }
     } else {
       ++cnt.proposed;  // k = 0: degenerate staple (measure zero), leave the subgroup
@@ -495,20 +529,8 @@ __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h
       ++cnt.accepted;
       cfx R00, R01;
       fx_rotation(a, v, R00, R01);
-      const cfx R10{fx_neg(R01.re), R01.im}, R11 = cfx_conj(R00);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const cfx ui = u.e[0][c], uj = u.e[1][c];
-        cfacc z = cfx_zero();
-        cfx_mac(z, R00, ui);
-        cfx_mac(z, R01, uj);
-        u.e[0][c] = cfx_norm(z);
-        // (in the last subgroup row 2 is not used any more: reunitarisation rebuilds it)
-        z = cfx_zero();
-        cfx_mac(z, R10, ui);
-        cfx_mac(z, R11, uj);
-        u.e[1][c] = cfx_norm(z);
-      }
+      for (int c = 0; c < 3; ++c) fx_rotate_column(R00, R01, u.e[0][c], u.e[1][c]);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -566,6 +588,189 @@ __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h
       }
     *meas = (double)fx_merge_wide(tr) * (0x1p-58 / 3.0);
   }
+  return cnt;
+}
+
+// ---------------------------------------------------------------------------
+// The same update shared by LPL = 4 or 8 neighbouring lanes of a warp, for
+// lattices whose half-sweep leaves the GPU mostly idle: there the time is the
+// latency of one update.
+//   staple: 4 lanes: lanes 0-2 take the two paths of one direction each; 8 lanes:
+//     lanes 0-5 take one path each.  The paths are added as integers.
+//   heatbath: lane c < 3 holds column c of the link and row c of the staple; the
+//     projections and the Gram-Schmidt sums add up over the lanes as integers,
+//     the scalars of a subgroup are computed by every lane.
+//   draws: lane n < 3 draws the numbers of subgroup n, before it waits for the
+//     half-sweep before this one (grid_wait), on which they do not depend.
+// Integer sums make every link bit for bit that of update_link_f64.  All lanes
+// of the warp call (shuffles); a group with active = false discards its
+// result.
+// ---------------------------------------------------------------------------
+template <int LPL>
+struct LaneGroup {
+  int part, c, base;
+  __device__ __forceinline__ LaneGroup() {
+    const int lane = (int)threadIdx.x & 31;
+    part = lane & (LPL - 1);
+    c = part < 3 ? part : 0;
+    base = lane & ~(LPL - 1);
+  }
+  // column c + s (mod 3)
+  __device__ __forceinline__ int col(int s) const {
+    const int k = c + s;
+    return k >= 3 ? k - 3 : k;
+  }
+  template <typename T>
+  __device__ __forceinline__ T from(T v, int k) const {
+    return __shfl_sync(0xffffffffu, v, base + k);
+  }
+  __device__ __forceinline__ fx from(const fx& v, int k) const { return fx_make(from(v.h, k), from(v.l, k)); }
+  __device__ __forceinline__ cfx from(const cfx& v, int k) const { return cfx{from(v.re, k), from(v.im, k)}; }
+  // sum over the columns
+  __device__ __forceinline__ long long sum(long long v) const { return v + from(v, col(1)) + from(v, col(2)); }
+};
+
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <int LPL, bool CG, bool REPEAT, typename KEY, typename G>
+__device__ __forceinline__ UpdateCount update_link_f64_lanes(const G& g, double2* U, int h, int p, int mu,
+                                                             const uint64_t* sweep, const KEY& key,
+                                                             const UpdateConsts& uc, bool active) {
+  const LaneGroup<LPL> lg;
+  const uint64_t t = *sweep;
+  const auto st = site_of(g, h, p);
+  const uint32_t s = (uint32_t)canon(g, st);
+  const fx_drawn mine = fx_draw_at(s, mu, lg.c, 0, t, key);
+  UpdateCount cnt{0, 0};
+  grid_wait();
+  if (*(volatile const int*)uc.far) {  // links far from SU(3): one lane per link
+    if (lg.part == 0 && active) cnt = update_link_f64_far<CG>(g, U, h, p, mu, t, key, uc, nullptr);
+    return cnt;
+  }
+  h = store_index(g, st, h);
+  fx_staple A;
+  fx_staple_zero(A);
+  constexpr int kPaths = LPL == 8 ? 1 : 2;  // per lane
+  if (lg.part * kPaths < 6) {
+    const int h_pmu = nb_half_rt(g, st, mu, +1);
+#pragma unroll 1
+    for (int n = 0; n < kPaths; ++n) {
+      const int path = lg.part * kPaths + n;
+      const bool backward = path & 1;
+      const int nu = (path >> 1) + ((path >> 1) >= mu ? 1 : 0);
+      const int hy = nb_half_rt(g, st, nu, backward ? -1 : +1);
+      fx_staple_add(A, staple_path_fx<CG>(U, g.Vh, p, mu, nu, backward, backward ? nb_half2_rt(g, st, mu, nu) : h_pmu,
+                                          hy, backward ? hy : h));
+    }
+  }
+  if constexpr (LPL == 8) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) A.r[i][k][q] += __shfl_down_sync(0xffffffffu, A.r[i][k][q], 3, LPL);
+  }
+  // row c of the sum: lane c + n (mod 3) sends its row c
+  cfx a[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    long long m[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const long long x0 = A.r[0][k][q], x1 = A.r[1][k][q], x2 = A.r[2][k][q];
+      m[q] = lg.c == 0 ? x0 : (lg.c == 1 ? x1 : x2);
+      m[q] += lg.from(lg.c == 0 ? x2 : (lg.c == 1 ? x0 : x1), lg.col(1));  // row c - 1 goes to lane c - 1
+      m[q] += lg.from(lg.c == 0 ? x1 : (lg.c == 1 ? x2 : x0), lg.col(2));
+    }
+    a[k] = cfx{fx_staple_entry(m[0], lg.c, 6), fx_staple_entry(m[1], lg.c, 6)};
+  }
+  const FxLink<CG> own(U, mu, p, h, g.Vh);
+  cfx u[3] = {own.at(0, lg.c), own.at(1, lg.c), own.at(2, lg.c)};
+#pragma unroll 1
+  for (int sub = 0; sub < 3; ++sub) {
+    long long r[4];
+    fx_projection_column(u[0], u[1], a[0], a[1], r);
+#pragma unroll
+    for (int n = 0; n < 4; ++n) r[n] = lg.sum(r[n]);
+    fx_drawn w;
+    w.S = lg.from(mine.S, sub);
+    w.u3 = lg.from(mine.u3, sub);
+#pragma unroll
+    for (int n = 0; n < 3; ++n) w.d[n] = lg.from(mine.d[n], sub);
+    fx v[4], q[4];
+    double ik;
+    bool accepted = false;
+    if (fx_direction(r, v, &ik)) {
+      const double inv_alpha = uc.three_over_beta_f64 * ik;
+      ++cnt.proposed;
+      accepted = fx_propose(w, inv_alpha, q);
+      if (REPEAT) {
+#pragma unroll 1
+        for (int tr = 1; tr < uc.max_tries && !accepted; ++tr) {
+          ++cnt.proposed;
+          accepted = fx_propose(fx_draw_at(s, mu, sub, tr, t, key), inv_alpha, q);
+        }
+      }
+    } else {
+      ++cnt.proposed;
+    }
+    if (accepted) {
+      ++cnt.accepted;
+      cfx R00, R01;
+      fx_rotation(q, v, R00, R01);
+      fx_rotate_column(R00, R01, u[0], u[1]);
+    }
+    const bool first = sub == 0;
+    const cfx x[3] = {u[0], u[1], u[2]}, y[3] = {a[0], a[1], a[2]};
+    u[0] = first ? x[0] : x[2];
+    u[1] = first ? x[2] : x[1];
+    u[2] = first ? x[1] : x[0];
+    a[0] = first ? y[0] : y[2];
+    a[1] = first ? y[2] : y[1];
+    a[2] = first ? y[1] : y[0];
+  }
+  cfx r0 = u[0], r1 = u[2];
+  fx_gram gr = fx_gram_column(r0, r1);
+  gr.n0 = lg.sum(gr.n0);
+  gr.n1 = lg.sum(gr.n1);
+  gr.dr = lg.sum(gr.dr);
+  gr.di = lg.sum(gr.di);
+  fx_gs co;
+  const bool ok = fx_gs_coefficients(gr, co);
+  cx<double> o[3];
+  if (__any_sync(0xffffffffu, lg.part < 3 && !ok)) {  // as in heatbath_fx
+    const double d[4] = {fx_to_double(r0.re), fx_to_double(r0.im), fx_to_double(r1.re), fx_to_double(r1.im)};
+    cx<double> b0[3], b1[3];
+    mat3<double> m;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      b0[k] = mk(lg.from(d[0], k), lg.from(d[1], k));
+      b1[k] = mk(lg.from(d[2], k), lg.from(d[3], k));
+    }
+    gram_schmidt_rows01(b0, b1);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      m.e[0][k] = b0[k];
+      m.e[1][k] = b1[k];
+    }
+    complete_row2(m);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) o[i] = lg.c == 0 ? m.e[i][0] : (lg.c == 1 ? m.e[i][1] : m.e[i][2]);
+  }
+  fx_gs_column(co, r0, r1);
+  const cfx row2 = fx_row2_entry(lg.from(r0, lg.col(1)), lg.from(r0, lg.col(2)), lg.from(r1, lg.col(1)), lg.from(r1, lg.col(2)));
+  if (ok) {
+    o[0] = mk(fx_to_double(r0.re), fx_to_double(r0.im));
+    o[1] = mk(fx_to_double(r1.re), fx_to_double(r1.im));
+    o[2] = mk(fx_to_double(row2.re), fx_to_double(row2.im));
+  }
+  if (active && lg.part < 3 && link_ok(mu, p, h, g.Vh)) {
+    double2* b = U + link_base(mu, p, g.Vh, kEntriesF64) + h + (size_t)lg.c * g.Vh;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) b[(size_t)(3 * i) * g.Vh] = make_double2(o[i].re, o[i].im);
+  }
+  if (lg.part != 0 || !active) cnt = UpdateCount{0, 0};
   return cnt;
 }
 

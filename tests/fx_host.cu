@@ -100,7 +100,7 @@ static void heatbath_scalars() {
     if (it == 2) m = (1ull << 53) - 1;
     const Q x = std::ldexp((Q)m, -53);
     lg.add(std::ldexp((Q)fx_neg_log(m), -57) + std::log(x));
-    const fx_cs cs = fx_cossin<true>(m);
+    const fx_cs cs = fx_cossin(m);
     trig.add(val(cs.c, -30) - std::cos(2 * pi * x));
     trig.add(val(cs.s, -30) - std::sin(2 * pi * x));
     root.add(val(fx_two_root((long long)(m << 9)), -30) - 2 * std::sqrt(x * (1 - x)));
@@ -135,7 +135,7 @@ static void heatbath_scalars() {
     double D[6];
     for (int c = 0; c < 6; ++c) U[c] = D[c] = std::ldexp((double)w[c], -53);
     const Q cq1 = std::cos(2 * pi * U[1]), delta = -(std::log(U[0]) + cq1 * cq1 * std::log(U[2])) * ia;
-    const bool take = U[3] * U[3] <= 1 - delta / 2, took = fx_propose(w, ia, a);
+    const bool take = U[3] * U[3] <= 1 - delta / 2, took = fx_propose(fx_draw(w), ia, a);
     other += take != took;
     if (!take || !took) continue;
     const double cd = (double)cq1, dd = -std::fma(cd * cd, std::log(D[2]), std::log(D[0])) * ia;
@@ -217,7 +217,9 @@ int main() {
           }
           Fd[i][k][0] = re;
           Fd[i][k][1] = im;
-          f.e[i][k] = cfx_norm(s);
+          f.m[i][k][0] = fx_merge(s.re);
+          f.m[i][k][1] = fx_merge(s.im);
+          f.e[i][k] = cfx{fx_norm_merged(f.m[i][k][0]), fx_norm_merged(f.m[i][k][1])};
           ref[i][k] = {ref[i][k].re + F[i][k].re, ref[i][k].im + F[i][k].im};
           f64[i][k][0] += re;
           f64[i][k][1] += im;
@@ -232,7 +234,7 @@ int main() {
       }
       fx_staple_add(A, f);
     }
-    const fx_mat m = fx_staple_mat(A);
+    const fx_mat m = fx_staple_mat(A, 6);
     for (int i = 0; i < 3; ++i)
       for (int k = 0; k < 3; ++k) {
         staple = std::fmax(staple, std::fabs(val(m.e[i][k].re, -28) - ref[i][k].re) / u);
