@@ -437,7 +437,7 @@ int su3_create_ex(int L0, int L1, int L2, int L3, double beta, uint64_t seed, in
   h->threads = default_threads(h->pairs ? h->pgeom.Vh : h->geom.Vh);
   h->split = use_split(h->geom.Vh, precision);
   {
-    const cudaError_t ep = su3k_prepare();
+    const cudaError_t ep = precision == SU3_FP64 ? su3k_prepare_f64() : su3k_prepare();
     if (ep != cudaSuccess) {
       delete h;
       return cuda_fail(ep, "su3_create: kernel attributes");

@@ -193,7 +193,7 @@ cudaError_t launch_mu(const BatchArgs& a, const ParamReplicas* pr, int threads, 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.n_items);
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = std::is_same<T, double>::value ? (size_t)threads * kFxRingBytes : 0;
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = MU > 0 ? 1 : 0;
@@ -229,7 +229,8 @@ int max_blocks_per_sm(int precision, int threads) {
   int n = 0;
   cudaError_t e =
       precision == SU3_FP64
-          ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_c<double, false, false, 0>, threads, 0)
+          ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_c<double, false, false, 0>, threads,
+                                                          (size_t)threads * kFxRingBytes)
           : precision == SU3_FP32_EFT
                 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_c<float, true, false, 0>, threads, 0)
                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_c<float, false, false, 0>, threads, 0);
@@ -240,6 +241,17 @@ std::mutex g_tune_mutex;
 std::map<std::string, std::vector<int>> g_tune_cache;  // key -> {threads, blocks per SM, window}
 
 }  // namespace
+
+cudaError_t su3k_prepare_batch_f64() {
+  const void* const k[] = {(const void*)k_batch_sweep_c<double, false, false, 0>, (const void*)k_batch_sweep_c<double, false, true, 0>,
+                           (const void*)k_batch_sweep<double, false, false, 0>, (const void*)k_batch_sweep<double, false, true, 0>};
+  for (const void* f : k) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SU3_BATCH_LB_THREADS * kFxRingBytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
 
 SU3_BOUNDS_STATUS_FN(su3k_bounds_status_batch)
 
@@ -460,6 +472,10 @@ int su3_batch_create(int n, const int (*dims)[4], const double* betas, const uin
   if (start != SU3_COLD && start != SU3_HOT) return fail(SU3_EINVAL, "su3_batch_create: bad start");
   if (precision != SU3_FP64 && precision != SU3_FP32_MIXED && precision != SU3_FP32_EFT)
     return fail(SU3_EINVAL, "su3_batch_create: bad precision");
+  if (precision == SU3_FP64) {
+    const cudaError_t ep = su3k_prepare_batch_f64();
+    if (ep != cudaSuccess) return su3_cuda_fail(ep, "su3_batch_create: kernel attributes");
+  }
   su3_batch* b = new (std::nothrow) su3_batch;
   su3_lattice* h = b ? new (std::nothrow) su3_lattice : nullptr;
   if (!b || !h) {

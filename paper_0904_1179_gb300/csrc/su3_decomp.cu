@@ -231,11 +231,11 @@ cudaError_t launch_update_form(const DecompArgs& a, int precision, const dim3& g
   if (precision == SU3_FP64 && !MEAS && a.lanes > 1) {
     const dim3 lgrid((unsigned)(((long long)a.lanes * a.g.in.Vh + threads - 1) / threads), grid.y);
     if (a.lanes == 8)
-      k_decomp_half_sweep_f64_lanes<8, REPEAT><<<lgrid, threads, 0, s>>>(a, MU);
+      k_decomp_half_sweep_f64_lanes<8, REPEAT><<<lgrid, threads, (size_t)threads * kFxRingBytes, s>>>(a, MU);
     else
-      k_decomp_half_sweep_f64_lanes<4, REPEAT><<<lgrid, threads, 0, s>>>(a, MU);
+      k_decomp_half_sweep_f64_lanes<4, REPEAT><<<lgrid, threads, (size_t)threads * kFxRingBytes, s>>>(a, MU);
   } else if (precision == SU3_FP64)
-    k_decomp_half_sweep_f64<REPEAT, MEAS><<<grid, threads, 0, s>>>(a, MU);
+    k_decomp_half_sweep_f64<REPEAT, MEAS><<<grid, threads, (size_t)threads * kFxRingBytes, s>>>(a, MU);
   else if (precision == SU3_FP32_EFT)
     k_decomp_half_sweep_f32<MU, true, REPEAT, MEAS><<<grid, threads, 0, s>>>(a);
   else
@@ -487,6 +487,20 @@ void host_sub_geometry(const int L[4], int ndmpi, int mpifactor, SubGeometry& g)
 // ---------------------------------------------------------------------------
 bool su3_decomp_active(const su3_lattice* h) { return h && h->decomp && h->decomp->active; }
 
+cudaError_t su3k_prepare_decomp_f64() {
+  const void* const k[] = {
+      (const void*)k_decomp_half_sweep_f64<false, false>,   (const void*)k_decomp_half_sweep_f64<true, false>,
+      (const void*)k_decomp_half_sweep_f64<false, true>,    (const void*)k_decomp_half_sweep_f64<true, true>,
+      (const void*)k_decomp_half_sweep_f64_lanes<4, false>, (const void*)k_decomp_half_sweep_f64_lanes<4, true>,
+      (const void*)k_decomp_half_sweep_f64_lanes<8, false>, (const void*)k_decomp_half_sweep_f64_lanes<8, true>};
+  for (const void* f : k) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSweepThreads * kFxRingBytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
 SU3_BOUNDS_STATUS_FN(su3k_bounds_status_decomp)
 
 void su3_decomp_invalidate(su3_decomp* d) {
@@ -572,6 +586,13 @@ int su3_decomp_create(int L0, int L1, int L2, int L3, double beta, uint64_t seed
   su3_handle h = nullptr;
   rc = su3_create_ex(L0, L1, L2, L3, beta, seed, start, precision, cuda_stream, &h);
   if (rc != SU3_OK) return rc;
+  if (precision == SU3_FP64) {
+    const cudaError_t ep = su3k_prepare_decomp_f64();
+    if (ep != cudaSuccess) {
+      su3_release_handle(h);
+      return su3_cuda_fail(ep, "su3_decomp_create: kernel attributes");
+    }
+  }
   su3_decomp* d = new (std::nothrow) su3_decomp;
   if (!d) {
     su3_release_handle(h);

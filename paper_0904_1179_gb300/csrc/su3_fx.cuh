@@ -69,8 +69,15 @@ struct fx {
 struct cfx {
   fx re, im;
 };
+// The same without f (two registers a real, for numbers kept over long code).
+struct cfxs {
+  int hr, hi;
+  float lr, li;
+};
 
 SU3_HD fx fx_make(int h, float l) { return fx{h, l, fx_i2f(h)}; }
+SU3_HD cfx cfx_of(const cfxs& a) { return cfx{fx_make(a.hr, a.lr), fx_make(a.hi, a.li)}; }
+SU3_HD cfxs cfx_short(const cfx& a) { return cfxs{a.re.h, a.im.h, a.re.l, a.im.l}; }
 SU3_HD fx fx_neg(fx a) { return fx{-a.h, -a.l, -a.f}; }
 SU3_HD cfx cfx_conj(cfx a) { return cfx{a.re, fx_neg(a.im)}; }
 
@@ -240,7 +247,6 @@ SU3_HD cfx cfx_norm(const cfacc& s) { return cfx{fx_norm(s.re), fx_norm(s.im)}; 
 // ---------------------------------------------------------------------------
 struct fx_rows01 {
   cfx e[2][3];
-  long long m[2][3][2];  // merged, with the 2^29 of fx_zero
 };
 struct fx_staple {
   long long r[3][3][2];
@@ -253,15 +259,9 @@ SU3_HD void fx_staple_zero(fx_staple& A) {
     for (int k = 0; k < 3; ++k) A.r[i][k][0] = A.r[i][k][1] = 0;
 }
 
-// A += F (rows 0,1 given, row 2 completed).
-SU3_HD void fx_staple_add(fx_staple& A, const fx_rows01& F) {
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      A.r[i][k][0] += F.m[i][k][0];
-      A.r[i][k][1] += F.m[i][k][1];
-    }
+// Row 2 of A += F (rows 0,1 given, row 2 completed).  The merged sums of F's rows
+// 0,1 (with the 2^29 of fx_zero) are added to A's by who forms them.
+SU3_HD void fx_staple_add_row2(fx_staple& A, const fx_rows01& F) {
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const int a = (k + 1) % 3, b = (k + 2) % 3;

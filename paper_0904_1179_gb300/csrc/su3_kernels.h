@@ -76,6 +76,10 @@ int su3k_pair_tile2(const su3dev::Geometry& gp, int threads);
 // kernel attributes it needs (set once, before any stream capture).
 constexpr int kPairRingBytesPerThread = 3 * 7 * 16;
 cudaError_t su3k_prepare();
+// The same for the FP64 kernels: single lattices, batches, sublattices.
+cudaError_t su3k_prepare_f64();
+cudaError_t su3k_prepare_batch_f64();
+cudaError_t su3k_prepare_decomp_f64();
 
 // The persistent sweeps (su3_sweepq.cuh): the half-sweeps of one sweep as
 // tiles of one block each, handed out in order from a device counter; a tile

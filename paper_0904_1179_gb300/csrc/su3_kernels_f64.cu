@@ -96,7 +96,7 @@ __global__ void SU3_F64_BOUNDS
 // Launched as a programmatic dependent of the half-sweep before it, a block
 // draws its random numbers while that one drains.
 template <int LPL, bool REPEAT>
-__global__ void __launch_bounds__(kMaxSweepThreads) k_half_sweep_f64_lanes(HalfSweepArgs args, int mu, int stats) {
+__global__ void SU3_F64_BOUNDS k_half_sweep_f64_lanes(HalfSweepArgs args, int mu, int stats) {
   signal_dependents();
   const int gid = blockIdx.x * blockDim.x + threadIdx.x;
   const int link = gid / LPL;
@@ -122,7 +122,7 @@ cudaError_t launch_sweep_f64(const HalfSweepArgs& a, const SweepQueue& q, int tp
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chained ? tpl * layers : 2 * tpl * layers);
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = (size_t)threads * kFxRingBytes;
   cfg.stream = s;
   cfg.attrs = attr;
   for (int mu = 0; mu < 4; ++mu)
@@ -142,11 +142,12 @@ cudaError_t su3k_launch_half_sweep_f64(const HalfSweepArgs& a, int mu, bool stat
   const int blocks = (a.geom.Vh + threads - 1) / threads;
   const bool repeat = a.max_tries > 1;
   const int st = stats ? 1 : 0;
+  const size_t smem = (size_t)threads * kFxRingBytes;
   if (mu > 0 && a.meas) {  // fused plaquette (statistics are not counted in these phases)
     if (repeat)
-      k_half_sweep_f64<true, true><<<blocks, threads, 0, s>>>(a, mu, 0);
+      k_half_sweep_f64<true, true><<<blocks, threads, smem, s>>>(a, mu, 0);
     else
-      k_half_sweep_f64<false, true><<<blocks, threads, 0, s>>>(a, mu, 0);
+      k_half_sweep_f64<false, true><<<blocks, threads, smem, s>>>(a, mu, 0);
   } else if (a.lanes > 1) {
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -154,6 +155,7 @@ cudaError_t su3k_launch_half_sweep_f64(const HalfSweepArgs& a, int mu, bool stat
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(((long long)a.lanes * a.geom.Vh + threads - 1) / threads));
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = a.chained ? 1 : 0;
@@ -163,9 +165,9 @@ cudaError_t su3k_launch_half_sweep_f64(const HalfSweepArgs& a, int mu, bool stat
     return repeat ? cudaLaunchKernelEx(&cfg, k_half_sweep_f64_lanes<4, true>, a, mu, st)
                   : cudaLaunchKernelEx(&cfg, k_half_sweep_f64_lanes<4, false>, a, mu, st);
   } else if (repeat) {
-    k_half_sweep_f64<true, false><<<blocks, threads, 0, s>>>(a, mu, st);
+    k_half_sweep_f64<true, false><<<blocks, threads, smem, s>>>(a, mu, st);
   } else {
-    k_half_sweep_f64<false, false><<<blocks, threads, 0, s>>>(a, mu, st);
+    k_half_sweep_f64<false, false><<<blocks, threads, smem, s>>>(a, mu, st);
   }
   return cudaGetLastError();
 }
@@ -184,6 +186,22 @@ cudaError_t su3k_launch_sweep_f64(const HalfSweepArgs& a, const SweepQueue& q, b
   if (layers == 0 || a.meas || a.split) return cudaErrorInvalidValue;
   return a.max_tries > 1 ? launch_sweep_f64<true>(a, q, tpl, layers, stats, threads, chained, s)
                          : launch_sweep_f64<false>(a, q, tpl, layers, stats, threads, chained, s);
+}
+
+// The ring takes up to 100 KB of dynamic shared memory (256 threads).
+cudaError_t su3k_prepare_f64() {
+  const void* const k[] = {(const void*)k_half_sweep_f64<false, false>, (const void*)k_half_sweep_f64<true, false>,
+                           (const void*)k_half_sweep_f64<false, true>,  (const void*)k_half_sweep_f64<true, true>,
+                           (const void*)k_sweep_f64<false>,             (const void*)k_sweep_f64<true>,
+                           (const void*)k_half_sweep_f64_chain<false>,  (const void*)k_half_sweep_f64_chain<true>,
+                           (const void*)k_half_sweep_f64_lanes<4, false>, (const void*)k_half_sweep_f64_lanes<4, true>,
+                           (const void*)k_half_sweep_f64_lanes<8, false>, (const void*)k_half_sweep_f64_lanes<8, true>};
+  for (const void* f : k) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSweepThreads * kFxRingBytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 SU3_BOUNDS_STATUS_FN(su3k_bounds_status_f64)

@@ -318,107 +318,175 @@ __device__ __noinline__ UpdateCount update_link_f64_far(const G& g, double2* U, 
 }
 
 // ---------------------------------------------------------------------------
+// cp.async: 16-byte copies from global to shared memory that do not pass
+// through registers, tracked in commit groups per thread.
+// ---------------------------------------------------------------------------
+// Both forms copy through L1 (.ca): cache operators are performance hints
+// and do not change the memory-consistency behaviour, so links written by
+// other blocks of a persistent launch are seen once the block has acquired
+// their completion counts; and on GB300 the L1-bypassing cp.async.cg made the
+// site-paired sweep 1.7 times slower.
+template <bool CG>
+__device__ __forceinline__ void cp_async16(uint32_t saddr, const float4* gsrc) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(gsrc) : "memory");
+}
+__device__ __forceinline__ void cp_async16(double2* dst, const double2* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// ---------------------------------------------------------------------------
 // The FP64 link update on the integer and FP32 pipes (su3_fx.cuh): links are
 // read from the FP64 store, split into integer and FP32 parts, and multiplied
 // there; the SU(2) steps (su3_fx_kp.cuh) use it too, but for the four FP64
 // operations that make delta from 1/alpha, whose range beta leaves open.
-// Loads go entry by entry, in the order in which the products use them.
 // ---------------------------------------------------------------------------
-// A link of the store, or its adjoint.
-template <bool CG>
+// A link entry of the store, split.  Real parts on the integer pipe (14
+// instructions), imaginary parts by a conversion on the FP64 pipe (5, but 16 SM
+// cycles of a pipe that is otherwise nearly idle): 32^4 3.90 ms per sweep,
+// against 4.17 with both on the integer pipe and 4.26 with both converted.
+__device__ __forceinline__ cfx fx_entry(double2 v, uint32_t flip) {
+  return cfx{fx_from_double(v.x), fx_from_double_cvt(v.y, flip)};
+}
+
+// A link of the store, or its adjoint, entry by entry.
 struct FxLink {
   const double2* b;
-  int si, sk;     // elements between rows and between columns
-  uint32_t flip;  // sign of the imaginary parts
-  bool ok;
+  uint32_t si, sk;  // elements between rows and between columns
+  // (an access that the bounds-checked build finds out of range reads link 0)
   __device__ __forceinline__ FxLink(const void* U, int mu, int p, int h, int Vh, bool dag = false)
-      : b((const double2*)U + link_base(mu, p, Vh, kEntriesF64) + h),
-        si(dag ? Vh : 3 * Vh),
-        sk(dag ? 3 * Vh : Vh),
-        flip(dag ? 0x80000000u : 0u),
-        ok(link_ok(mu, p, h, Vh)) {}
-  __device__ __forceinline__ cfx at(int i, int k) const {
-    if (!ok) return cfx{{0, 0.0f, 0.0f}, {0, 0.0f, 0.0f}};
-    const double2 v = ld_link<CG>(b + ((size_t)i * si + (size_t)k * sk));
-    // Real parts on the integer pipe (14 instructions), imaginary parts by a
-    // conversion on the FP64 pipe (5, but 16 SM cycles of a pipe that is
-    // otherwise nearly idle): 32^4 3.90 ms per sweep, against 4.17 with both on
-    // the integer pipe and 4.26 with both converted.
-    return cfx{fx_from_double(v.x), fx_from_double_cvt(v.y, flip)};
+      : b((const double2*)U + link_base(mu, p, Vh, kEntriesF64) + (link_ok(mu, p, h, Vh) ? h : 0)),
+        si(dag ? (uint32_t)Vh : 3u * (uint32_t)Vh),
+        sk(dag ? 3u * (uint32_t)Vh : (uint32_t)Vh) {}
+  // 9 Vh < 2^32
+  __device__ __forceinline__ const double2* at(int i, int k) const { return b + (size_t)((uint32_t)i * si + (uint32_t)k * sk); }
+};
+
+// The links of a path pass through shared memory: each thread owns three slots,
+// for rows 0,1 of X and for Y and Z, and requests the next path's link with 16-byte
+// cp.async copies once it has read the slot, so that three links are in flight
+// behind the arithmetic (the code of a path is rolled up for the instruction
+// caches and loads nothing ahead by itself).  Strides of 7 and 9 double2: eight
+// lanes' 16-byte reads touch every bank once.  Dynamic shared memory,
+// kFxRingBytes per thread.
+constexpr int kFxRingBytes = (7 + 9 + 9) * 16;
+
+struct FxRing {
+  double2 *x, *yz;  // this thread's slot of X, and of Y; Z is `step` further
+  int step;
+  __device__ __forceinline__ FxRing() {
+    extern __shared__ double2 fx_ring[];
+    const int n = blockDim.x, t = threadIdx.x;
+    x = fx_ring + 7 * t;
+    yz = fx_ring + 7 * n + 9 * t;
+    step = 9 * n;
+  }
+  __device__ __forceinline__ void fetch_rows01(const FxLink& l) const {
+#pragma unroll
+    for (int e = 0; e < 6; ++e) cp_async16(x + e, l.at(e / 3, e % 3));
+  }
+  __device__ __forceinline__ void fetch(int slot, const FxLink& l) const {
+#pragma unroll
+    for (int e = 0; e < 9; ++e) cp_async16(yz + slot * step + e, l.at(e / 3, e % 3));
   }
 };
 
-// Rows 0,1 of X Y^+ Z: the two products in one piece of code, run twice
-// (instruction cache; see staple_path_fx).  Yd: the link Y^+.
-template <bool CG>
-__device__ __forceinline__ fx_rows01 path_fx(const FxLink<CG>& X, const FxLink<CG>& Yd, const FxLink<CG>& Z) {
-  fx_rows01 f;
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) f.e[i][k] = X.at(i, k);
-  FxLink<CG> L = Yd;
-#pragma unroll 1
-  for (int n = 0; n < 2; ++n) {
-    cfx t[2][3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      cfacc s[2] = {cfx_zero(), cfx_zero()};
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const cfx z = L.at(j, k);
-        cfx_mac(s[0], f.e[0][j], z);
-        cfx_mac(s[1], f.e[1][j], z);
-      }
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        f.m[i][k][0] = fx_merge(s[i].re);
-        f.m[i][k][1] = fx_merge(s[i].im);
-        t[i][k] = cfx{fx_norm_merged(f.m[i][k][0]), fx_norm_merged(f.m[i][k][1])};
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) f.e[i][k] = t[i][k];
-    L = Z;
+// The two paths of direction nu (forward_path, backward_path above) have one
+// form, X Y^+ Z:
+//   forward:  U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+,  backward: U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu),
+// number 2 n and 2 n + 1 for the n-th direction nu != mu.  hx, hy, hz: half indices.
+struct FxPath {
+  int nu, hx, hy, hz;
+  bool backward;
+  template <typename G, typename S>
+  __device__ __forceinline__ FxPath(const G& g, const S& st, int h, int mu, int path) {
+    backward = path & 1;
+    nu = (path >> 1) + ((path >> 1) >= mu ? 1 : 0);
+    hy = nb_half_rt(g, st, nu, backward ? -1 : +1);
+    hx = backward ? nb_half2_rt(g, st, mu, nu) : nb_half_rt(g, st, mu, +1);
+    hz = backward ? hy : h;
   }
-  return f;
-}
+  __device__ __forceinline__ FxLink X(const void* U, int p, int Vh) const {
+    return FxLink(U, nu, backward ? p : p ^ 1, hx, Vh, backward);
+  }
+  __device__ __forceinline__ FxLink Yd(const void* U, int p, int mu, int Vh) const {
+    return FxLink(U, mu, p ^ 1, hy, Vh, true);
+  }
+  __device__ __forceinline__ FxLink Z(const void* U, int p, int Vh) const {
+    return FxLink(U, nu, backward ? p ^ 1 : p, hz, Vh, !backward);
+  }
+};
 
-// The two paths of direction nu (forward_path, backward_path above): one piece
-// of code for both, so that the whole update stays within the instruction
-// caches.
-//   forward:  U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+,  backward: U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu);
-// hx, hy, hz: half indices of the three sites.
-template <bool CG>
-__device__ __forceinline__ fx_rows01 staple_path_fx(const void* U, int Vh, int p, int mu, int nu, bool backward, int hx,
-                                                    int hy, int hz) {
-  const int q = p ^ 1;
-  return path_fx(FxLink<CG>(U, nu, backward ? p : q, hx, Vh, backward), FxLink<CG>(U, mu, q, hy, Vh, true),
-                 FxLink<CG>(U, nu, backward ? q : p, hz, Vh, !backward));
-}
-
-// Six-staple sum of U_mu(x), x = st of parity p stored at h.
+// Adds the paths first .. last - 1 of U_mu(x), x = st of parity p stored at h, to A;
+// own (optional): a link that ends up in the ring's slot of Y (cp_async_wait<0>).
 // Apart (optional): receives the sum of the terms with nu < mu.  After the
 // update, Re Tr(U_new Apart) is the sum of the plaquettes of the planes
 // (mu, nu < mu) at x and at x - nu-hat.
 template <bool CG, typename G, typename S>
-__device__ __forceinline__ fx_mat staple_fx(const G& g, const void* U, const S& st, int h, int p, int mu,
-                                            fx_mat* Apart = nullptr) {
-  fx_staple A;
-  fx_staple_zero(A);
-  const int h_pmu = nb_half_rt(g, st, mu, +1);
-#pragma unroll 1
-  for (int path = 0; path < 6; ++path) {
-    const bool backward = path & 1;
-    const int nu = (path >> 1) + ((path >> 1) >= mu ? 1 : 0);
-    const int hy = nb_half_rt(g, st, nu, backward ? -1 : +1);
-    fx_staple_add(A, staple_path_fx<CG>(U, g.Vh, p, mu, nu, backward, backward ? nb_half2_rt(g, st, mu, nu) : h_pmu, hy,
-                                        backward ? hy : h));
-    if (Apart && backward && nu == mu - 1) *Apart = fx_staple_mat(A, path + 1);
+__device__ __forceinline__ void staple_paths_fx(fx_staple& A, const G& g, const void* U, const S& st, int h, int p,
+                                                int mu, int first, int last, const FxRing& ring, const FxLink* own,
+                                                fx_mat* Apart = nullptr) {
+  {
+    const FxPath t(g, st, h, mu, first);
+    ring.fetch_rows01(t.X(U, p, g.Vh));
+    cp_async_commit();
+    ring.fetch(0, t.Yd(U, p, mu, g.Vh));
+    cp_async_commit();
+    ring.fetch(1, t.Z(U, p, g.Vh));
+    cp_async_commit();
   }
-  return fx_staple_mat(A, 6);
+#pragma unroll 1
+  for (int path = first; path < last; ++path) {
+    const bool backward = path & 1, more = path + 1 < last;
+    const FxPath t(g, st, h, mu, more ? path + 1 : path);
+    fx_rows01 f;
+    cp_async_wait<2>();
+#pragma unroll
+    for (int e = 0; e < 6; ++e) f.e[e / 3][e % 3] = fx_entry(ring.x[e], backward ? 0x80000000u : 0u);
+    if (more) ring.fetch_rows01(t.X(U, p, g.Vh));
+    cp_async_commit();
+    // the two products in one piece of code
+#pragma unroll 1
+    for (int n = 0; n < 2; ++n) {
+      const double2* z = ring.yz + n * ring.step;
+      const uint32_t flip = n == 0 || !backward ? 0x80000000u : 0u;
+      cfx q[2][3];
+      cp_async_wait<2>();
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        cfacc s[2] = {cfx_zero(), cfx_zero()};
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+          const cfx y = fx_entry(z[3 * j + k], flip);
+          cfx_mac(s[0], f.e[0][j], y);
+          cfx_mac(s[1], f.e[1][j], y);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          const long long re = fx_merge(s[i].re), im = fx_merge(s[i].im);
+          q[i][k] = cfx{fx_norm_merged(re), fx_norm_merged(im)};
+          A.r[i][k][0] += n ? re : 0;  // the path's rows 0,1
+          A.r[i][k][1] += n ? im : 0;
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) f.e[i][k] = q[i][k];
+      if (more)
+        ring.fetch(n, n == 0 ? t.Yd(U, p, mu, g.Vh) : t.Z(U, p, g.Vh));
+      else if (own && n == 0)
+        ring.fetch(0, *own);
+      cp_async_commit();
+    }
+    fx_staple_add_row2(A, f);
+    if (Apart && backward && (path >> 1) == mu - 1) *Apart = fx_staple_mat(A, path + 1);
+  }
 }
 
 // A sum of products of units 2^-30 and 2^-28 merged (units of 2^-58).  The cross
@@ -483,31 +551,33 @@ __device__ __forceinline__ fx_drawn fx_draw_at(uint32_t s, int mu, int sub, int 
   return fx_draw(m);
 }
 
-// Everything after the staple A0 (unit 2^-28): three SU(2) heatbath steps,
+// Everything after the staple A0 (unit 2^-28) of the link u: three SU(2) heatbath steps,
 // reunitarisation, the store of link (s, mu) at storage half index h.
 // MEAS: also (1/3) Re Tr(U_new Apart) into *meas.
 template <bool CG, bool REPEAT, bool MEAS, typename KEY, typename G>
 __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h, int p, int mu, uint64_t t, uint32_t s,
-                                                   const KEY& key, const UpdateConsts& uc, const fx_mat& A0,
+                                                   const KEY& key, const UpdateConsts& uc, fx_mat u, const fx_mat& A0,
                                                    const fx_mat& Apart, double* meas) {
   UpdateCount cnt{0, 0};
-  fx_mat u;
-  const FxLink<CG> own(U, mu, p, h, g.Vh);
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) u.e[i][k] = own.at(i, k);
   // The subgroups (0,1), (0,2), (1,2) in one piece of code (instruction cache):
   // the step always acts on rows 0, 1 of u and columns 0, 1 of A, and between the
   // steps rows and columns change places: orders (0,1,2), (0,2,1), (1,2,0).
-  fx_mat A = A0;
+  // They are kept without f, which the uses convert again: 36 registers.
+  cfxs us[3][3], A[3][3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      us[i][k] = cfx_short(u.e[i][k]);
+      A[i][k] = cfx_short(A0.e[i][k]);
+    }
 #pragma unroll 1
   for (int sub = 0; sub < 3; ++sub) {
     long long r[4] = {0, 0, 0, 0};
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       long long q[4];
-      fx_projection_column(u.e[0][c], u.e[1][c], A.e[c][0], A.e[c][1], q);
+      fx_projection_column(cfx_of(us[0][c]), cfx_of(us[1][c]), cfx_of(A[c][0]), cfx_of(A[c][1]), q);
 #pragma unroll
       for (int n = 0; n < 4; ++n) r[n] += q[n];
     }
@@ -530,23 +600,31 @@ __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h
       cfx R00, R01;
       fx_rotation(a, v, R00, R01);
 #pragma unroll
-      for (int c = 0; c < 3; ++c) fx_rotate_column(R00, R01, u.e[0][c], u.e[1][c]);
+      for (int c = 0; c < 3; ++c) {
+        cfx x = cfx_of(us[0][c]), y = cfx_of(us[1][c]);
+        fx_rotate_column(R00, R01, x, y);
+        us[0][c] = cfx_short(x);
+        us[1][c] = cfx_short(y);
+      }
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const bool first = sub == 0;
-      const cfx x[3] = {u.e[0][c], u.e[1][c], u.e[2][c]}, y[3] = {A.e[c][0], A.e[c][1], A.e[c][2]};
-      u.e[0][c] = first ? x[0] : x[2];
-      u.e[1][c] = first ? x[2] : x[1];
-      u.e[2][c] = first ? x[1] : x[0];
-      A.e[c][0] = first ? y[0] : y[2];
-      A.e[c][1] = first ? y[2] : y[1];
-      A.e[c][2] = first ? y[1] : y[0];
+      const cfxs x[3] = {us[0][c], us[1][c], us[2][c]}, y[3] = {A[c][0], A[c][1], A[c][2]};
+      us[0][c] = first ? x[0] : x[2];
+      us[1][c] = first ? x[2] : x[1];
+      us[2][c] = first ? x[1] : x[0];
+      A[c][0] = first ? y[0] : y[2];
+      A[c][1] = first ? y[2] : y[1];
+      A[c][2] = first ? y[1] : y[0];
     }
   }
   // after the last change: (row 0, row 2, row 1)
 #pragma unroll
-  for (int c = 0; c < 3; ++c) u.e[1][c] = u.e[2][c];
+  for (int c = 0; c < 3; ++c) {
+    u.e[0][c] = cfx_of(us[0][c]);
+    u.e[1][c] = cfx_of(us[2][c]);
+  }
   mat3<double> out;
   if (fx_reunitarise(u)) {
     fx_complete_row2(u);
@@ -648,21 +726,13 @@ __device__ __forceinline__ UpdateCount update_link_f64_lanes(const G& g, double2
     return cnt;
   }
   h = store_index(g, st, h);
+  const FxLink own(U, mu, p, h, g.Vh);
+  const double2 mine_u[3] = {ld_link<CG>(own.at(0, lg.c)), ld_link<CG>(own.at(1, lg.c)), ld_link<CG>(own.at(2, lg.c))};
   fx_staple A;
   fx_staple_zero(A);
   constexpr int kPaths = LPL == 8 ? 1 : 2;  // per lane
-  if (lg.part * kPaths < 6) {
-    const int h_pmu = nb_half_rt(g, st, mu, +1);
-#pragma unroll 1
-    for (int n = 0; n < kPaths; ++n) {
-      const int path = lg.part * kPaths + n;
-      const bool backward = path & 1;
-      const int nu = (path >> 1) + ((path >> 1) >= mu ? 1 : 0);
-      const int hy = nb_half_rt(g, st, nu, backward ? -1 : +1);
-      fx_staple_add(A, staple_path_fx<CG>(U, g.Vh, p, mu, nu, backward, backward ? nb_half2_rt(g, st, mu, nu) : h_pmu,
-                                          hy, backward ? hy : h));
-    }
-  }
+  if (lg.part * kPaths < 6)
+    staple_paths_fx<CG>(A, g, U, st, h, p, mu, lg.part * kPaths, (lg.part + 1) * kPaths, FxRing(), nullptr);
   if constexpr (LPL == 8) {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -685,8 +755,7 @@ __device__ __forceinline__ UpdateCount update_link_f64_lanes(const G& g, double2
     }
     a[k] = cfx{fx_staple_entry(m[0], lg.c, 6), fx_staple_entry(m[1], lg.c, 6)};
   }
-  const FxLink<CG> own(U, mu, p, h, g.Vh);
-  cfx u[3] = {own.at(0, lg.c), own.at(1, lg.c), own.at(2, lg.c)};
+  cfx u[3] = {fx_entry(mine_u[0], 0u), fx_entry(mine_u[1], 0u), fx_entry(mine_u[2], 0u)};
 #pragma unroll 1
   for (int sub = 0; sub < 3; ++sub) {
     long long r[4];
@@ -783,8 +852,18 @@ __device__ __forceinline__ UpdateCount update_link_f64(const G& g, double2* U, i
   const uint32_t s = (uint32_t)canon(g, st);
   h = store_index(g, st, h);
   fx_mat Apart;
-  const fx_mat A = staple_fx<CG>(g, U, st, h, p, mu, MEAS ? &Apart : nullptr);
-  return heatbath_fx<CG, REPEAT, MEAS>(g, U, h, p, mu, t, s, key, uc, A, Apart, meas);
+  fx_staple A;
+  fx_staple_zero(A);
+  const FxRing ring;
+  const FxLink own(U, mu, p, h, g.Vh);
+  staple_paths_fx<CG>(A, g, U, st, h, p, mu, 0, 6, ring, &own, MEAS ? &Apart : nullptr);
+  cp_async_wait<0>();
+  fx_mat u;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) u.e[i][k] = fx_entry(ring.yz[3 * i + k], 0u);
+  return heatbath_fx<CG, REPEAT, MEAS>(g, U, h, p, mu, t, s, key, uc, u, fx_staple_mat(A, 6), Apart, meas);
 }
 
 // ---------------------------------------------------------------------------
@@ -858,25 +937,6 @@ __device__ __forceinline__ pm3 staple_p(const G& g, const float4* U, const S& st
     if (Apart && nu == MU - 1) *Apart = A;
   }
   return A;
-}
-
-// ---------------------------------------------------------------------------
-// cp.async: 16-byte copies from global to shared memory that do not pass
-// through registers, tracked in commit groups per thread.
-// ---------------------------------------------------------------------------
-// Both forms copy through L1 (.ca): cache operators are performance hints
-// and do not change the memory-consistency behaviour, so links written by
-// other blocks of a persistent launch are seen once the block has acquired
-// their completion counts; and on GB300 the L1-bypassing cp.async.cg made the
-// site-paired sweep 1.7 times slower.
-template <bool CG>
-__device__ __forceinline__ void cp_async16(uint32_t saddr, const float4* gsrc) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(saddr), "l"(gsrc) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 // The hardware square root (about 1 ulp): the FP32 heatbath needs no

@@ -217,9 +217,10 @@ int main() {
           }
           Fd[i][k][0] = re;
           Fd[i][k][1] = im;
-          f.m[i][k][0] = fx_merge(s.re);
-          f.m[i][k][1] = fx_merge(s.im);
-          f.e[i][k] = cfx{fx_norm_merged(f.m[i][k][0]), fx_norm_merged(f.m[i][k][1])};
+          const long long mr = fx_merge(s.re), mi = fx_merge(s.im);
+          f.e[i][k] = cfx{fx_norm_merged(mr), fx_norm_merged(mi)};
+          A.r[i][k][0] += mr;
+          A.r[i][k][1] += mi;
           ref[i][k] = {ref[i][k].re + F[i][k].re, ref[i][k].im + F[i][k].im};
           f64[i][k][0] += re;
           f64[i][k][1] += im;
@@ -232,7 +233,7 @@ int main() {
         f64[2][k][0] += std::fma(p[0], q[0], std::fma(-p[1], q[1], std::fma(-v[0], w[0], v[1] * w[1])));
         f64[2][k][1] -= std::fma(p[0], q[1], std::fma(p[1], q[0], std::fma(-v[0], w[1], -v[1] * w[0])));
       }
-      fx_staple_add(A, f);
+      fx_staple_add_row2(A, f);
     }
     const fx_mat m = fx_staple_mat(A, 6);
     for (int i = 0; i < 3; ++i)
