@@ -82,7 +82,7 @@ __device__ __forceinline__ void update_item(const ReplicaDesc& rd, void* links, 
                                             int max_tries, int* far) {
   const UpdateConsts uc{rd.three_over_beta_f64, rd.three_over_beta, max_tries, far};
   if constexpr (std::is_same<T, double>::value)
-    update_link_f64<true, REPEAT>(rd.g, (double2*)links + rd.offset, h, p, mu, t, rd.key, uc);
+    update_link_f64<REPEAT>(rd.g, (double2*)links + rd.offset, h, p, mu, t, rd.key, uc);
   else
     update_link_f32<MU, true, EFT, REPEAT>(rd.g, (float4*)links + rd.offset, h, p, t, rd.key, uc);
 }

@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kMaxSweepThreads) k_decomp_half_sweep_f64(Deco
   if (h < g.in.Vh) {
     const UpdateConsts uc{a.three_over_beta_f64, a.three_over_beta, a.max_tries, sweep_far(a.sweep)};
     double2* U = (double2*)a.subs + (size_t)k * a.sub_elems;
-    c = update_link_f64<false, REPEAT, MEAS>(g, U, h, a.parity, mu, *a.sweep, a.key, uc, &m);
+    c = update_link_f64<REPEAT, MEAS>(g, U, h, a.parity, mu, *a.sweep, a.key, uc, &m);
   }
   if (a.count_stats) count_stats_d(c, a.stats);
   if (MEAS) block_partial_d(m, a.meas);
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kMaxSweepThreads) k_decomp_half_sweep_f64_lane
   const UpdateConsts uc{a.three_over_beta_f64, a.three_over_beta, a.max_tries, sweep_far(a.sweep)};
   double2* U = (double2*)a.subs + (size_t)k * a.sub_elems;
   const UpdateCount c =
-      update_link_f64_lanes<LPL, false, REPEAT>(g, U, active ? link : 0, a.parity, mu, a.sweep, a.key, uc, active);
+      update_link_f64_lanes<LPL, REPEAT>(g, U, active ? link : 0, a.parity, mu, a.sweep, a.key, uc, active);
   if (a.count_stats) count_stats_d(c, a.stats);
 }
 

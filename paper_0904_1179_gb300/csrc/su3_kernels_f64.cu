@@ -41,7 +41,7 @@ __global__ void SU3_F64_BOUNDS k_half_sweep_f64(HalfSweepArgs args, int mu, int 
   UpdateCount c{0, 0};
   double m = 0.0;
   if (h < args.geom.Vh)
-    c = update_link_f64<false, REPEAT, MEAS>(args.geom, (double2*)args.links, h, args.parity, mu, *args.sweep, args.key,
+    c = update_link_f64<REPEAT, MEAS>(args.geom, (double2*)args.links, h, args.parity, mu, *args.sweep, args.key,
                                              update_consts(args), &m);
   if (!MEAS && stats) count_stats<true>(c, args.stats);
   if (MEAS) block_partial(m, args.meas);
@@ -53,8 +53,10 @@ __global__ void SU3_F64_BOUNDS k_half_sweep_f64(HalfSweepArgs args, int mu, int 
 // one x3 layer of the lattice and waits only for the layers of the previous
 // half-sweep that its staples read, so one half-sweep's last wave overlaps
 // the next one's first and only one launch tail per sweep remains.  The
-// links change while the launch runs, so they are read through L2 (CG); the
-// update is that of k_half_sweep_f64, bit for bit.
+// links change while the launch runs: the waiting block's acquire drops the SM's
+// L1 lines before its cp.async copies go through L1 (copies past L1, .cg, took
+// 1.50 ms per 24^4 sweep instead of 1.05); the update is that of k_half_sweep_f64,
+// bit for bit.
 template <bool REPEAT>
 __global__ void SU3_F64_BOUNDS
     k_sweep_f64(HalfSweepArgs args, SweepQueue qa, int tiles_per_layer, int layers, int stats, int mu) {
@@ -65,7 +67,7 @@ __global__ void SU3_F64_BOUNDS
   const SweepItem it = s_item;
   if (it.phase < 0) return;
   const int h = it.tile * (int)blockDim.x + (int)threadIdx.x;  // layers are whole tiles: always a site of the lattice
-  const UpdateCount c = update_link_f64<true, REPEAT>(args.geom, (double2*)args.links, h, it.phase & 1, mu, *args.sweep,
+  const UpdateCount c = update_link_f64<REPEAT>(args.geom, (double2*)args.links, h, it.phase & 1, mu, *args.sweep,
                                                       args.key, update_consts(args));
   if (stats) count_stats<true>(c, args.stats);
   report_sweep_item(qa, layers, it);
@@ -86,7 +88,7 @@ __global__ void SU3_F64_BOUNDS
   const SweepItem it = s_item;
   if (it.phase < 0) return;
   const int h = it.tile * (int)blockDim.x + (int)threadIdx.x;  // layers are whole tiles: always a site of the lattice
-  const UpdateCount c = update_link_f64<true, REPEAT>(args.geom, (double2*)args.links, h, parity, mu, *args.sweep,
+  const UpdateCount c = update_link_f64<REPEAT>(args.geom, (double2*)args.links, h, parity, mu, *args.sweep,
                                                       args.key, update_consts(args));
   if (stats) count_stats<true>(c, args.stats);
   report_sweep_item(qa, layers, it);
@@ -101,7 +103,7 @@ __global__ void SU3_F64_BOUNDS k_half_sweep_f64_lanes(HalfSweepArgs args, int mu
   const int gid = blockIdx.x * blockDim.x + threadIdx.x;
   const int link = gid / LPL;
   const bool active = link < args.geom.Vh;  // a group past the end works on site 0 (shuffles stay converged)
-  const UpdateCount c = update_link_f64_lanes<LPL, false, REPEAT>(args.geom, (double2*)args.links, active ? link : 0,
+  const UpdateCount c = update_link_f64_lanes<LPL, REPEAT>(args.geom, (double2*)args.links, active ? link : 0,
                                                                  args.parity, mu, args.sweep, args.key,
                                                                  update_consts(args), active);
   if (stats) count_stats<true>(c, args.stats);

@@ -254,12 +254,13 @@ __device__ __forceinline__ bool propose_f64(uint32_t s, int mu, int sub, uint64_
 // (SweepState::far), whose entries and products may leave the range of
 // su3_fx.cuh: one function for every direction and heatbath, not inlined and
 // its loops not unrolled, since no sweep of a proper configuration runs it.
+// Links are read through L2: blocks of the same launch may have written them.
 // meas (nullptr: off) receives (1/3) Re Tr(U_new A_<), A_< the staple terms of
 // the directions nu < mu.
 // G: Geometry (periodic lattice) or SubGeometry (sublattice with ghost
 // layers); h enumerates the sites of parity p.
 // ---------------------------------------------------------------------------
-template <bool CG, typename KEY, typename G>
+template <typename KEY, typename G>
 __device__ __noinline__ UpdateCount update_link_f64_far(const G& g, double2* U, int h, int p, int mu, uint64_t t,
                                                         const KEY& key, const UpdateConsts& uc, double* meas) {
   const auto st = site_of(g, h, p);
@@ -270,12 +271,12 @@ __device__ __noinline__ UpdateCount update_link_f64_far(const G& g, double2* U, 
 #pragma unroll 1
   for (int nu = 0; nu < 4; ++nu) {
     if (nu == mu) continue;
-    acc_completed(A, forward_path<double, CG>(g, U, st, h, p, mu, nu, h_pmu, nb_half_rt(g, st, nu, +1)));
-    acc_completed(A, backward_path<double, CG>(g, U, p, mu, nu, nb_half_rt(g, st, nu, -1), nb_half2_rt(g, st, mu, nu)));
+    acc_completed(A, forward_path<double, true>(g, U, st, h, p, mu, nu, h_pmu, nb_half_rt(g, st, nu, +1)));
+    acc_completed(A, backward_path<double, true>(g, U, p, mu, nu, nb_half_rt(g, st, nu, -1), nb_half2_rt(g, st, mu, nu)));
     if (nu == mu - 1) Apart = A;
   }
   UpdateCount cnt{0, 0};
-  mat3<double> u = load_f64<CG>(U, mu, p, h, g.Vh);
+  mat3<double> u = load_f64<true>(U, mu, p, h, g.Vh);
 #pragma unroll 1
   for (int sub = 0; sub < 3; ++sub) {
     const int i = subrow_i(sub), j = subrow_j(sub);
@@ -427,7 +428,7 @@ struct FxPath {
 // Apart (optional): receives the sum of the terms with nu < mu.  After the
 // update, Re Tr(U_new Apart) is the sum of the plaquettes of the planes
 // (mu, nu < mu) at x and at x - nu-hat.
-template <bool CG, typename G, typename S>
+template <typename G, typename S>
 __device__ __forceinline__ void staple_paths_fx(fx_staple& A, const G& g, const void* U, const S& st, int h, int p,
                                                 int mu, int first, int last, const FxRing& ring, const FxLink* own,
                                                 fx_mat* Apart = nullptr) {
@@ -554,7 +555,7 @@ __device__ __forceinline__ fx_drawn fx_draw_at(uint32_t s, int mu, int sub, int 
 // Everything after the staple A0 (unit 2^-28) of the link u: three SU(2) heatbath steps,
 // reunitarisation, the store of link (s, mu) at storage half index h.
 // MEAS: also (1/3) Re Tr(U_new Apart) into *meas.
-template <bool CG, bool REPEAT, bool MEAS, typename KEY, typename G>
+template <bool REPEAT, bool MEAS, typename KEY, typename G>
 __device__ __forceinline__ UpdateCount heatbath_fx(const G& g, double2* U, int h, int p, int mu, uint64_t t, uint32_t s,
                                                    const KEY& key, const UpdateConsts& uc, fx_mat u, const fx_mat& A0,
                                                    const fx_mat& Apart, double* meas) {
@@ -710,7 +711,7 @@ struct LaneGroup {
 
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-template <int LPL, bool CG, bool REPEAT, typename KEY, typename G>
+template <int LPL, bool REPEAT, typename KEY, typename G>
 __device__ __forceinline__ UpdateCount update_link_f64_lanes(const G& g, double2* U, int h, int p, int mu,
                                                              const uint64_t* sweep, const KEY& key,
                                                              const UpdateConsts& uc, bool active) {
@@ -722,17 +723,17 @@ __device__ __forceinline__ UpdateCount update_link_f64_lanes(const G& g, double2
   UpdateCount cnt{0, 0};
   grid_wait();
   if (*(volatile const int*)uc.far) {  // links far from SU(3): one lane per link
-    if (lg.part == 0 && active) cnt = update_link_f64_far<CG>(g, U, h, p, mu, t, key, uc, nullptr);
+    if (lg.part == 0 && active) cnt = update_link_f64_far(g, U, h, p, mu, t, key, uc, nullptr);
     return cnt;
   }
   h = store_index(g, st, h);
   const FxLink own(U, mu, p, h, g.Vh);
-  const double2 mine_u[3] = {ld_link<CG>(own.at(0, lg.c)), ld_link<CG>(own.at(1, lg.c)), ld_link<CG>(own.at(2, lg.c))};
+  const double2 mine_u[3] = {__ldcg(own.at(0, lg.c)), __ldcg(own.at(1, lg.c)), __ldcg(own.at(2, lg.c))};
   fx_staple A;
   fx_staple_zero(A);
   constexpr int kPaths = LPL == 8 ? 1 : 2;  // per lane
   if (lg.part * kPaths < 6)
-    staple_paths_fx<CG>(A, g, U, st, h, p, mu, lg.part * kPaths, (lg.part + 1) * kPaths, FxRing(), nullptr);
+    staple_paths_fx(A, g, U, st, h, p, mu, lg.part * kPaths, (lg.part + 1) * kPaths, FxRing(), nullptr);
   if constexpr (LPL == 8) {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
@@ -844,10 +845,10 @@ __device__ __forceinline__ UpdateCount update_link_f64_lanes(const G& g, double2
 }
 
 // One update of an FP64 store's link U_mu(x) (h, parity p as in site_of).
-template <bool CG, bool REPEAT, bool MEAS = false, typename KEY, typename G>
+template <bool REPEAT, bool MEAS = false, typename KEY, typename G>
 __device__ __forceinline__ UpdateCount update_link_f64(const G& g, double2* U, int h, int p, int mu, uint64_t t,
                                                        const KEY& key, const UpdateConsts& uc, double* meas = nullptr) {
-  if (*(volatile const int*)uc.far) return update_link_f64_far<CG>(g, U, h, p, mu, t, key, uc, MEAS ? meas : nullptr);
+  if (*(volatile const int*)uc.far) return update_link_f64_far(g, U, h, p, mu, t, key, uc, MEAS ? meas : nullptr);
   const auto st = site_of(g, h, p);
   const uint32_t s = (uint32_t)canon(g, st);
   h = store_index(g, st, h);
@@ -856,14 +857,14 @@ __device__ __forceinline__ UpdateCount update_link_f64(const G& g, double2* U, i
   fx_staple_zero(A);
   const FxRing ring;
   const FxLink own(U, mu, p, h, g.Vh);
-  staple_paths_fx<CG>(A, g, U, st, h, p, mu, 0, 6, ring, &own, MEAS ? &Apart : nullptr);
+  staple_paths_fx(A, g, U, st, h, p, mu, 0, 6, ring, &own, MEAS ? &Apart : nullptr);
   cp_async_wait<0>();
   fx_mat u;
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int k = 0; k < 3; ++k) u.e[i][k] = fx_entry(ring.yz[3 * i + k], 0u);
-  return heatbath_fx<CG, REPEAT, MEAS>(g, U, h, p, mu, t, s, key, uc, u, fx_staple_mat(A, 6), Apart, meas);
+  return heatbath_fx<REPEAT, MEAS>(g, U, h, p, mu, t, s, key, uc, u, fx_staple_mat(A, 6), Apart, meas);
 }
 
 // ---------------------------------------------------------------------------
