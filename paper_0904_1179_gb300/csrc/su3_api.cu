@@ -161,6 +161,20 @@ void release(su3_lattice* h) {
   delete h;
 }
 
+// Whether the FP64 half-sweeps with several lanes per link are programmatic
+// dependents of each other: their draws then run while the half-sweep before
+// drains, but a programmatic launch costs about 1 us more than a plain one, and
+// the early warps take issue slots from the last.  GB300, ms per sweep, plain /
+// programmatic: 4^4 (0.2 warps per SM) 0.084 / 0.076, 6^4 (1.1) 0.088 / 0.080,
+// 8^4 (3.4) 0.090 / 0.095, 8^3 x 16 (3.4 at four lanes) 0.111 / 0.118, 10^4 (4.1)
+// 0.131 / 0.140, 12^4 (8.5) 0.178 / 0.168.  (Without draws to overlap it only
+// costs: the FP32 half-sweeps of 8^4 to 24^3 x 16 took 8 to 25 % longer.)
+bool f64_lanes_chained(const su3_lattice* h) {
+  const int sms = sm_count(), lanes = su3_f64_lanes(h);
+  const long long threads = (long long)lanes * h->geom.Vh;
+  return sms > 0 && lanes > 1 && (threads <= 2 * 32LL * sms || threads >= 8 * 32LL * sms);
+}
+
 HalfSweepArgs half_sweep_args(const su3_lattice* h, int parity) {
   HalfSweepArgs a{};
   a.meas = nullptr;
@@ -293,7 +307,7 @@ int enqueue_sweep_body(su3_lattice* h, bool measured) {
     for (int mu = 0; mu < 4; ++mu)
       for (int p = 0; p < 2; ++p) {
         HalfSweepArgs a = half_sweep_args(h, p);
-        a.chained = mu + p > 0;
+        a.chained = mu + p > 0 && h->precision == SU3_FP64 && f64_lanes_chained(h);
         if (measured && p == 1 && mu >= 1) a.meas = h->d_meas_parts + (size_t)(mu - 1) * blocks;
         SU3_CUDA(su3k_launch_half_sweep(a, mu, h->precision, h->stats_on, h->threads, h->stream),
                  "half-sweep launch");
@@ -458,7 +472,7 @@ int su3_create_ex(int L0, int L1, int L2, int L3, double beta, uint64_t seed, in
   // the site-paired FP32 store pads each (mu, parity) array to whole tiles of pairs
   h->link_bytes = h->pairs ? (size_t)8 * 6 * su3dev::pair_padded(V / 4) * sizeof(float4)
                            : (size_t)V * 4 * (precision == SU3_FP64 ? 18 * sizeof(double) : 12 * sizeof(float));
-  const int nparts = su3k_plaquette_blocks(h->geom);
+  const int nparts = precision == SU3_FP64 ? su3k_plaquette_f64_blocks(h->geom) : su3k_plaquette_blocks(h->geom);
   const long long chunk = V < kChunkSites ? V : kChunkSites;
   if ((e = cudaMalloc(&h->links, h->link_bytes)) != cudaSuccess ||
       (e = cudaMalloc(&h->d_sweep, sizeof(su3dev::SweepState))) != cudaSuccess ||
@@ -584,7 +598,9 @@ double su3_plaquette(su3_handle h) {
   }
   if (su3_decomp_sync_global(h) != SU3_OK) return NAN;
   PlaqArgs a{h->geom, h->links, h->d_partials, h->pairs ? 1 : 0};
-  cudaError_t e = su3k_launch_plaquette(a, h->precision, h->d_plaq, h->stream);
+  cudaError_t e = h->precision == SU3_FP64
+                      ? su3k_launch_plaquette_f64(a, su3dev::sweep_far(h->d_sweep), h->d_plaq, h->stream)
+                      : su3k_launch_plaquette(a, h->precision, h->d_plaq, h->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_plaq, h->d_plaq, sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {

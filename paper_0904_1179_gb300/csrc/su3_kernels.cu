@@ -13,6 +13,7 @@
 #include "su3_kernels.h"
 
 #include "su3_device.cuh"
+#include "su3_plaquette.cuh"
 #include "su3_reduce.cuh"
 #include "su3_sitepair.cuh"
 #include "su3_update.cuh"
@@ -194,91 +195,16 @@ __global__ void k_hot_start(InitArgs args) {
 }
 
 // ---------------------------------------------------------------------------
-// Plaquette: one thread per site, six planes, FP64 accumulation, fixed-order
+// Plaquette: one thread per site, six planes (su3_plaquette.cuh), fixed-order
 // block reduction into partials[blockIdx.x], then one block sums the partials.
 // ---------------------------------------------------------------------------
 template <typename T>
-__device__ __forceinline__ mat3<T> load_any(const void* U, int mu, int p, int h, int Vh, bool pairs);
-template <>
-__device__ __forceinline__ mat3<double> load_any<double>(const void* U, int mu, int p, int h, int Vh, bool) {
-  return load_f64((const double2*)U, mu, p, h, Vh);
-}
-template <>
-__device__ __forceinline__ mat3<float> load_any<float>(const void* U, int mu, int p, int h, int Vh, bool pairs) {
-  return load_f32_any((const float4*)U, mu, p, h, Vh, pairs);
-}
-
-// Re Tr(X Y^+) with X = U_mu(x) U_nu(x+mu), Y = U_nu(x) U_mu(x+nu).
-template <typename T>
-__device__ __forceinline__ double plaq_site(const Geometry& g, const void* U, const Site& st, int h, int p, bool pairs) {
-  const int q = p ^ 1;
-  double sum = 0.0;
-#pragma unroll
-  for (int mu = 0; mu < 4; ++mu)
-#pragma unroll
-    for (int nu = mu + 1; nu < 4; ++nu) {
-      const mat3<T> a = load_any<T>(U, mu, p, h, g.Vh, pairs);
-      const mat3<T> b = load_any<T>(U, nu, q, nb_half(g, st, mu, +1), g.Vh, pairs);
-      const mat3<T> c = load_any<T>(U, nu, p, h, g.Vh, pairs);
-      const mat3<T> d = load_any<T>(U, mu, q, nb_half(g, st, nu, +1), g.Vh, pairs);
-      T tr = T(0);
-#pragma unroll
-      for (int i = 0; i < 3; ++i)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          cx<T> x = mk(T(0), T(0)), y = x;
-#pragma unroll
-          for (int j = 0; j < 3; ++j) {
-            x = mac(x, a.e[i][j], b.e[j][k]);
-            y = mac(y, c.e[i][j], d.e[j][k]);
-          }
-          tr = fma(x.re, y.re, tr);
-          tr = fma(x.im, y.im, tr);
-        }
-      sum += (double)tr;
-    }
-  return sum;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_plaquette_partial(PlaqArgs args) {
-  const Geometry g = args.geom;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;  // over 2 * Vh: (parity, h)
-  double v = 0.0;
-  if (idx < 2 * g.Vh) {
-    const int p = idx >= g.Vh ? 1 : 0;
-    const int h = idx - p * g.Vh;
-    const Site st = site_of(g, h, p);
-    v = plaq_site<T>(g, args.links, st, h, p, args.pairs != 0);
-  }
-  __shared__ double red[32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const int nw = blockDim.x >> 5;
-    double w = threadIdx.x < nw ? red[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    if (threadIdx.x == 0) args.partials[blockIdx.x] = w;
-  }
+__global__ void __launch_bounds__(kPlaqThreads) k_plaquette_partial(PlaqArgs args) {
+  plaq_block<T>(args.geom, args.links, args.pairs != 0, (int)blockIdx.x, args.partials + blockIdx.x);
 }
 
 __global__ void __launch_bounds__(1024) k_plaquette_final(const double* partials, int n, double scale, double* out) {
-  __shared__ double red[32];
-  double v = 0.0;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) v += partials[i];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double w = threadIdx.x < (int)(blockDim.x >> 5) ? red[threadIdx.x] : 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-    if (threadIdx.x == 0) *out = w * scale;
-  }
+  sum_partials(partials, n, scale, out);
 }
 
 // ---------------------------------------------------------------------------
@@ -471,14 +397,14 @@ cudaError_t su3k_launch_init(const InitArgs& a, bool hot, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-int su3k_plaquette_blocks(const Geometry& g) { return (2 * g.Vh + 255) / 256; }
+int su3k_plaquette_blocks(const Geometry& g) { return plaq_blocks(g); }
 
 cudaError_t su3k_launch_plaquette(const PlaqArgs& a, int precision, double* out, cudaStream_t s) {
   const int blocks = su3k_plaquette_blocks(a.geom);
   if (precision == 0)
-    k_plaquette_partial<double><<<blocks, 256, 0, s>>>(a);
+    k_plaquette_partial<double><<<blocks, kPlaqThreads, 0, s>>>(a);
   else
-    k_plaquette_partial<float><<<blocks, 256, 0, s>>>(a);
+    k_plaquette_partial<float><<<blocks, kPlaqThreads, 0, s>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const double V = 2.0 * (double)a.geom.Vh;

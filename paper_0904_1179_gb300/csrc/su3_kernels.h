@@ -138,6 +138,10 @@ cudaError_t su3k_launch_set_counter(uint64_t* counter, uint64_t n, cudaStream_t 
 cudaError_t su3k_launch_init(const InitArgs& a, bool hot, cudaStream_t s);
 int su3k_plaquette_blocks(const su3dev::Geometry& g);
 cudaError_t su3k_launch_plaquette(const PlaqArgs& a, int precision, double* out, cudaStream_t s);
+// The same for a handle's FP64 store (far: SweepState's flag); partials:
+// su3k_plaquette_f64_blocks of them.
+int su3k_plaquette_f64_blocks(const su3dev::Geometry& g);
+cudaError_t su3k_launch_plaquette_f64(const PlaqArgs& a, const int* far, double* out, cudaStream_t s);
 cudaError_t su3k_launch_conv(const ConvArgs& a, bool to_store, cudaStream_t s);
 
 // Record a failure for su3_last_error() (thread-local); returns code.

@@ -14,6 +14,7 @@
 #include "su3_kernels.h"
 
 #include "su3_device.cuh"
+#include "su3_plaquette.cuh"
 #include "su3_reduce.cuh"
 #include "su3_sweepq.cuh"
 #include "su3_update.cuh"
@@ -109,6 +110,14 @@ __global__ void SU3_F64_BOUNDS k_half_sweep_f64_lanes(HalfSweepArgs args, int mu
   if (stats) count_stats<true>(c, args.stats);
 }
 
+__global__ void __launch_bounds__(kPlaqFxThreads) k_plaquette_fx(PlaqArgs args, const int* far) {
+  plaq_block_fx(args.geom, args.links, far, (int)blockIdx.x, args.partials + blockIdx.x);
+}
+
+__global__ void __launch_bounds__(1024) k_plaquette_fx_final(const double* partials, int n, double scale, double* out) {
+  sum_partials(partials, n, scale, out);
+}
+
 // ---------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------
@@ -188,6 +197,17 @@ cudaError_t su3k_launch_sweep_f64(const HalfSweepArgs& a, const SweepQueue& q, b
   if (layers == 0 || a.meas || a.split) return cudaErrorInvalidValue;
   return a.max_tries > 1 ? launch_sweep_f64<true>(a, q, tpl, layers, stats, threads, chained, s)
                          : launch_sweep_f64<false>(a, q, tpl, layers, stats, threads, chained, s);
+}
+
+int su3k_plaquette_f64_blocks(const Geometry& g) { return plaq_fx_blocks(g); }
+
+cudaError_t su3k_launch_plaquette_f64(const PlaqArgs& a, const int* far, double* out, cudaStream_t s) {
+  const int blocks = plaq_fx_blocks(a.geom);
+  k_plaquette_fx<<<blocks, kPlaqFxThreads, 0, s>>>(a, far);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_plaquette_fx_final<<<1, 1024, 0, s>>>(a.partials, blocks, 1.0 / (3.0 * 6.0 * 2.0 * (double)a.geom.Vh), out);
+  return cudaGetLastError();
 }
 
 // The ring takes up to 100 KB of dynamic shared memory (256 threads).
