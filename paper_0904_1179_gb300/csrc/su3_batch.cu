@@ -458,9 +458,9 @@ int set_config(su3_lattice* h, int threads, int blocks_per_sm, int window) {
 
 int check_status(su3_lattice* h, const char* what) {
   su3_batch* b = h->batch;
+  SU3_CUDA(cudaMemcpyAsync(b->h_status, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream), what);
   const int rc = su3_sync(h, what);
   if (rc != SU3_OK) return rc;
-  SU3_CUDA(cudaMemcpy(b->h_status, b->d_status, sizeof(int), cudaMemcpyDeviceToHost), what);
   if (*b->h_status != 0) {
     SU3_CUDA(cudaMemset(b->d_status, 0, sizeof(int)), what);
     // links that the sweep did not reach keep whatever they held
