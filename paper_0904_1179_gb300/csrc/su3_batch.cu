@@ -194,7 +194,7 @@ cudaError_t launch_mu(const BatchArgs& a, const ParamReplicas* pr, int threads, 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.n_items);
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = std::is_same<T, double>::value ? (size_t)threads * kFxRingBytes : 0;
+  cfg.dynamicSmemBytes = std::is_same<T, double>::value ? (size_t)threads * kFxThreadBytes : 0;
   cfg.stream = s;
   cfg.attrs = attr;
   cfg.numAttrs = MU > 0 ? 1 : 0;
@@ -231,7 +231,7 @@ int max_blocks_per_sm(int precision, int threads) {
   cudaError_t e =
       precision == SU3_FP64
           ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_c<double, false, false, 0>, threads,
-                                                          (size_t)threads * kFxRingBytes)
+                                                          (size_t)threads * kFxThreadBytes)
           : precision == SU3_FP32_EFT
                 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_c<float, true, false, 0>, threads, 0)
                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_batch_sweep_c<float, false, false, 0>, threads, 0);
@@ -248,7 +248,7 @@ cudaError_t su3k_prepare_batch_f64() {
                            (const void*)k_batch_sweep<double, false, false, 0>, (const void*)k_batch_sweep<double, false, true, 0>};
   for (const void* f : k) {
     const cudaError_t e =
-        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SU3_BATCH_LB_THREADS * kFxRingBytes);
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, SU3_BATCH_LB_THREADS * kFxThreadBytes);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -231,11 +231,11 @@ cudaError_t launch_update_form(const DecompArgs& a, int precision, const dim3& g
   if (precision == SU3_FP64 && !MEAS && a.lanes > 1) {
     const dim3 lgrid((unsigned)(((long long)a.lanes * a.g.in.Vh + threads - 1) / threads), grid.y);
     if (a.lanes == 8)
-      k_decomp_half_sweep_f64_lanes<8, REPEAT><<<lgrid, threads, (size_t)threads * kFxRingBytes, s>>>(a, MU);
+      k_decomp_half_sweep_f64_lanes<8, REPEAT><<<lgrid, threads, (size_t)threads * kFxThreadBytes, s>>>(a, MU);
     else
-      k_decomp_half_sweep_f64_lanes<4, REPEAT><<<lgrid, threads, (size_t)threads * kFxRingBytes, s>>>(a, MU);
+      k_decomp_half_sweep_f64_lanes<4, REPEAT><<<lgrid, threads, (size_t)threads * kFxThreadBytes, s>>>(a, MU);
   } else if (precision == SU3_FP64)
-    k_decomp_half_sweep_f64<REPEAT, MEAS><<<grid, threads, (size_t)threads * kFxRingBytes, s>>>(a, MU);
+    k_decomp_half_sweep_f64<REPEAT, MEAS><<<grid, threads, (size_t)threads * kFxThreadBytes, s>>>(a, MU);
   else if (precision == SU3_FP32_EFT)
     k_decomp_half_sweep_f32<MU, true, REPEAT, MEAS><<<grid, threads, 0, s>>>(a);
   else
@@ -495,7 +495,7 @@ cudaError_t su3k_prepare_decomp_f64() {
       (const void*)k_decomp_half_sweep_f64_lanes<8, false>, (const void*)k_decomp_half_sweep_f64_lanes<8, true>};
   for (const void* f : k) {
     const cudaError_t e =
-        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSweepThreads * kFxRingBytes);
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSweepThreads * kFxThreadBytes);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -133,7 +133,7 @@ cudaError_t launch_sweep_f64(const HalfSweepArgs& a, const SweepQueue& q, int tp
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(chained ? tpl * layers : 2 * tpl * layers);
   cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = (size_t)threads * kFxRingBytes;
+  cfg.dynamicSmemBytes = (size_t)threads * kFxThreadBytes;
   cfg.stream = s;
   cfg.attrs = attr;
   for (int mu = 0; mu < 4; ++mu)
@@ -153,7 +153,7 @@ cudaError_t su3k_launch_half_sweep_f64(const HalfSweepArgs& a, int mu, bool stat
   const int blocks = (a.geom.Vh + threads - 1) / threads;
   const bool repeat = a.max_tries > 1;
   const int st = stats ? 1 : 0;
-  const size_t smem = (size_t)threads * kFxRingBytes;
+  const size_t smem = (size_t)threads * kFxThreadBytes;
   if (mu > 0 && a.meas) {  // fused plaquette (statistics are not counted in these phases)
     if (repeat)
       k_half_sweep_f64<true, true><<<blocks, threads, smem, s>>>(a, mu, 0);
@@ -220,7 +220,7 @@ cudaError_t su3k_prepare_f64() {
                            (const void*)k_half_sweep_f64_lanes<8, false>, (const void*)k_half_sweep_f64_lanes<8, true>};
   for (const void* f : k) {
     const cudaError_t e =
-        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSweepThreads * kFxRingBytes);
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSweepThreads * kFxThreadBytes);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -347,10 +347,68 @@ __device__ __forceinline__ void cp_async_wait() {
 // there; the SU(2) steps (su3_fx_kp.cuh) use it too, but for the four FP64
 // operations that make delta from 1/alpha, whose range beta leaves open.
 // ---------------------------------------------------------------------------
+// Two rows' entries side by side: their FP32 parts go through the paired FMA
+// (one instruction for both), each half rounded like fx_mac's.
+struct fx2 {
+  int h[2];
+  float2 l, f;
+};
+struct cfx2 {
+  fx2 re, im;
+};
+struct facc2 {
+  long long hh[2];
+  float2 c;
+};
+struct cfacc2 {
+  facc2 re, im;
+};
+__device__ __forceinline__ fx2 fx2_of(const fx& a, const fx& b) {
+  return fx2{{a.h, b.h}, make_float2(a.l, b.l), make_float2(a.f, b.f)};
+}
+__device__ __forceinline__ cfx2 cfx2_of(const cfx& a, const cfx& b) { return cfx2{fx2_of(a.re, b.re), fx2_of(a.im, b.im)}; }
+__device__ __forceinline__ fx fx2_row(const fx2& a, int i) {
+  return i ? fx{a.h[1], a.l.y, a.f.y} : fx{a.h[0], a.l.x, a.f.x};
+}
+__device__ __forceinline__ cfx cfx2_row(const cfx2& a, int i) { return cfx{fx2_row(a.re, i), fx2_row(a.im, i)}; }
+__device__ __forceinline__ void fx2_set(fx2& a, int i, const fx& b) {
+  a.h[i] = b.h;
+  (i ? a.l.y : a.l.x) = b.l;
+  (i ? a.f.y : a.f.x) = b.f;
+}
+__device__ __forceinline__ void cfx2_set(cfx2& a, int i, const fx& re, const fx& im) {
+  fx2_set(a.re, i, re);
+  fx2_set(a.im, i, im);
+}
+__device__ __forceinline__ cfacc2 cfx2_zero() {
+  const facc2 z{{1LL << 29, 1LL << 29}, make_float2(0.0f, 0.0f)};
+  return cfacc2{z, z};
+}
+__device__ __forceinline__ void fx2_mac(facc2& s, const fx2& a, const fx& b) {
+  s.hh[0] += (long long)a.h[0] * b.h;
+  s.hh[1] += (long long)a.h[1] * b.h;
+  s.c = fma2(a.f, bc2(b.l), s.c);
+  s.c = fma2(a.l, bc2(b.f), s.c);
+}
+__device__ __forceinline__ void fx2_msub(facc2& s, const fx2& a, const fx& b) {
+  const int n = -b.h;
+  s.hh[0] += (long long)a.h[0] * n;
+  s.hh[1] += (long long)a.h[1] * n;
+  s.c = fma2(a.f, bc2(-b.l), s.c);
+  s.c = fma2(a.l, bc2(-b.f), s.c);
+}
+__device__ __forceinline__ void cfx2_mac(cfacc2& s, const cfx2& a, const cfx& b) {
+  fx2_mac(s.re, a.re, b.re);
+  fx2_msub(s.re, a.im, b.im);
+  fx2_mac(s.im, a.re, b.im);
+  fx2_mac(s.im, a.im, b.re);
+}
+
 // A link entry of the store, split.  Real parts on the integer pipe (14
 // instructions), imaginary parts by a conversion on the FP64 pipe (5, but 16 SM
-// cycles of a pipe that is otherwise nearly idle): 32^4 3.90 ms per sweep,
-// against 4.17 with both on the integer pipe and 4.26 with both converted.
+// cycles of a pipe that is otherwise nearly idle): 32^4 3.20 ms per sweep, against
+// 3.74 with both converted (and, on an earlier kernel, 3.90 against 4.17 with
+// both on the integer pipe).
 __device__ __forceinline__ cfx fx_entry(double2 v, uint32_t flip) {
   return cfx{fx_from_double(v.x), fx_from_double_cvt(v.y, flip)};
 }
@@ -374,8 +432,11 @@ struct FxLink {
 // behind the arithmetic (the code of a path is rolled up for the instruction
 // caches and loads nothing ahead by itself).  Strides of 7 and 9 double2: eight
 // lanes' 16-byte reads touch every bank once.  Dynamic shared memory,
-// kFxRingBytes per thread.
-constexpr int kFxRingBytes = (7 + 9 + 9) * 16;
+// kFxThreadBytes per thread.
+// After the slots: the thread's half-index steps along the eight directions
+// (FxSteps).
+constexpr int kFxSlotBytes = (7 + 9 + 9) * 16;
+constexpr int kFxThreadBytes = kFxSlotBytes + 8 * 4;
 
 struct FxRing {
   double2 *x, *yz;  // this thread's slot of X, and of Y; Z is `step` further
@@ -397,6 +458,28 @@ struct FxRing {
   }
 };
 
+// Changes of a site's half index for a step up and down along each direction:
+// half indices are separable, so x + mu - nu adds two of them.  Looked up by
+// direction at run time.
+struct FxSteps {
+  int* d;
+  int n;
+  __device__ __forceinline__ FxSteps() {
+    extern __shared__ double2 fx_ring[];
+    n = blockDim.x;
+    d = (int*)((char*)fx_ring + (size_t)n * kFxSlotBytes) + threadIdx.x;
+  }
+  template <typename G, typename S>
+  __device__ __forceinline__ void set(const G& g, const S& st, int h) const {
+#pragma unroll
+    for (int nu = 0; nu < 4; ++nu) {
+      d[nu * n] = nb_half(g, st, nu, +1) - h;
+      d[(4 + nu) * n] = nb_half(g, st, nu, -1) - h;
+    }
+  }
+  __device__ __forceinline__ int at(int nu, bool down) const { return d[(nu + (down ? 4 : 0)) * n]; }
+};
+
 // The two paths of direction nu (forward_path, backward_path above) have one
 // form, X Y^+ Z:
 //   forward:  U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+,  backward: U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu),
@@ -404,12 +487,12 @@ struct FxRing {
 struct FxPath {
   int nu, hx, hy, hz;
   bool backward;
-  template <typename G, typename S>
-  __device__ __forceinline__ FxPath(const G& g, const S& st, int h, int mu, int path) {
+  __device__ __forceinline__ FxPath(const FxSteps& steps, int h, int mu, int path) {
     backward = path & 1;
     nu = (path >> 1) + ((path >> 1) >= mu ? 1 : 0);
-    hy = nb_half_rt(g, st, nu, backward ? -1 : +1);
-    hx = backward ? nb_half2_rt(g, st, mu, nu) : nb_half_rt(g, st, mu, +1);
+    const int o = steps.at(nu, backward);
+    hy = h + o;
+    hx = h + steps.at(mu, false) + (backward ? o : 0);
     hz = backward ? hy : h;
   }
   __device__ __forceinline__ FxLink X(const void* U, int p, int Vh) const {
@@ -432,8 +515,10 @@ template <typename G, typename S>
 __device__ __forceinline__ void staple_paths_fx(fx_staple& A, const G& g, const void* U, const S& st, int h, int p,
                                                 int mu, int first, int last, const FxRing& ring, const FxLink* own,
                                                 fx_mat* Apart = nullptr) {
+  const FxSteps steps;
+  steps.set(g, st, h);
   {
-    const FxPath t(g, st, h, mu, first);
+    const FxPath t(steps, h, mu, first);
     ring.fetch_rows01(t.X(U, p, g.Vh));
     cp_async_commit();
     ring.fetch(0, t.Yd(U, p, mu, g.Vh));
@@ -444,11 +529,14 @@ __device__ __forceinline__ void staple_paths_fx(fx_staple& A, const G& g, const 
 #pragma unroll 1
   for (int path = first; path < last; ++path) {
     const bool backward = path & 1, more = path + 1 < last;
-    const FxPath t(g, st, h, mu, more ? path + 1 : path);
-    fx_rows01 f;
+    const FxPath t(steps, h, mu, more ? path + 1 : path);
+    cfx2 f[3];  // rows 0,1
     cp_async_wait<2>();
 #pragma unroll
-    for (int e = 0; e < 6; ++e) f.e[e / 3][e % 3] = fx_entry(ring.x[e], backward ? 0x80000000u : 0u);
+    for (int k = 0; k < 3; ++k) {
+      const uint32_t flip = backward ? 0x80000000u : 0u;
+      f[k] = cfx2_of(fx_entry(ring.x[k], flip), fx_entry(ring.x[3 + k], flip));
+    }
     if (more) ring.fetch_rows01(t.X(U, p, g.Vh));
     cp_async_commit();
     // the two products in one piece of code
@@ -456,36 +544,37 @@ __device__ __forceinline__ void staple_paths_fx(fx_staple& A, const G& g, const 
     for (int n = 0; n < 2; ++n) {
       const double2* z = ring.yz + n * ring.step;
       const uint32_t flip = n == 0 || !backward ? 0x80000000u : 0u;
-      cfx q[2][3];
+      cfx2 q[3];
       cp_async_wait<2>();
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        cfacc s[2] = {cfx_zero(), cfx_zero()};
+        cfacc2 s = cfx2_zero();
 #pragma unroll
-        for (int j = 0; j < 3; ++j) {
-          const cfx y = fx_entry(z[3 * j + k], flip);
-          cfx_mac(s[0], f.e[0][j], y);
-          cfx_mac(s[1], f.e[1][j], y);
-        }
+        for (int j = 0; j < 3; ++j) cfx2_mac(s, f[j], fx_entry(z[3 * j + k], flip));
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
-          const long long re = fx_merge(s[i].re), im = fx_merge(s[i].im);
-          q[i][k] = cfx{fx_norm_merged(re), fx_norm_merged(im)};
+          const long long re = fx_merge(facc{s.re.hh[i], i ? s.re.c.y : s.re.c.x}),
+                          im = fx_merge(facc{s.im.hh[i], i ? s.im.c.y : s.im.c.x});
+          cfx2_set(q[k], i, fx_norm_merged(re), fx_norm_merged(im));
           A.r[i][k][0] += n ? re : 0;  // the path's rows 0,1
           A.r[i][k][1] += n ? im : 0;
         }
       }
 #pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) f.e[i][k] = q[i][k];
+      for (int k = 0; k < 3; ++k) f[k] = q[k];
       if (more)
         ring.fetch(n, n == 0 ? t.Yd(U, p, mu, g.Vh) : t.Z(U, p, g.Vh));
       else if (own && n == 0)
         ring.fetch(0, *own);
       cp_async_commit();
     }
-    fx_staple_add_row2(A, f);
+    fx_rows01 F;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      F.e[0][k] = cfx2_row(f[k], 0);
+      F.e[1][k] = cfx2_row(f[k], 1);
+    }
+    fx_staple_add_row2(A, F);
     if (Apart && backward && (path >> 1) == mu - 1) *Apart = fx_staple_mat(A, path + 1);
   }
 }
@@ -525,15 +614,12 @@ __device__ __forceinline__ void fx_projection_column(const cfx& ui, const cfx& u
 // Entries of one column of the two rows that R turns (R10 = -conj(R01), R11 =
 // conj(R00)).
 __device__ __forceinline__ void fx_rotate_column(const cfx& R00, const cfx& R01, cfx& ui, cfx& uj) {
-  const cfx R10{fx_neg(R01.re), R01.im}, R11 = cfx_conj(R00);
-  cfacc z = cfx_zero();
-  cfx_mac(z, R00, ui);
-  cfx_mac(z, R01, uj);
-  cfacc w = cfx_zero();
-  cfx_mac(w, R10, ui);
-  cfx_mac(w, R11, uj);
-  ui = cfx_norm(z);
-  uj = cfx_norm(w);
+  const cfx2 Ri = cfx2_of(R00, cfx{fx_neg(R01.re), R01.im}), Rj = cfx2_of(R01, cfx_conj(R00));
+  cfacc2 z = cfx2_zero();
+  cfx2_mac(z, Ri, ui);
+  cfx2_mac(z, Rj, uj);
+  ui = cfx{fx_norm(facc{z.re.hh[0], z.re.c.x}), fx_norm(facc{z.im.hh[0], z.im.c.x})};
+  uj = cfx{fx_norm(facc{z.re.hh[1], z.re.c.y}), fx_norm(facc{z.im.hh[1], z.im.c.y})};
 }
 
 // The uniforms of proposal tr of subgroup sub.
