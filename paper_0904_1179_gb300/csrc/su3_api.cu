@@ -90,6 +90,18 @@ bool use_split(int Vh, int precision) {
   return sms > 0 && 4LL * Vh <= 32LL * warps_per_sm * sms;
 }
 
+// Whether the one-hit half-sweeps of a site-paired FP32 store run one thread per
+// link (k_half_sweep_f32_single) instead of one per pair: up to 2.5 warps of
+// links per scheduler, where twice the threads, each half as long, still fill
+// the GPU less than once.  GB300, ms per sweep, per pair / per link (mixed; EFT):
+// 12^4 (0.5 warps) 0.078 / 0.056; 0.066 / 0.051, 16^4 (1.7) 0.078 / 0.074; 0.068 /
+// 0.064, 16^3 x 20 (2.1) 0.105 / 0.095; 0.084 / 0.080, 20^3 x 16 (3.3) 0.107 /
+// 0.121; 0.088 / 0.105, 24^3 x 16 (5.7) 0.135 / 0.173; 0.119 / 0.146.
+bool pairs_single(int Vh) {
+  const int sms = sm_count();
+  return sms > 0 && 2LL * Vh <= 5LL * 32 * 4 * sms;
+}
+
 // Lanes per link of an FP64 half-sweep launched by itself
 // (k_half_sweep_f64_lanes), by the warps per SM they make.  GB300, ms per sweep
 // with 1 / 4 / 8 lanes: 4^4 0.234 / 0.103 / 0.082, 8^4 (3.4 warps per SM at 8
@@ -182,6 +194,7 @@ HalfSweepArgs half_sweep_args(const su3_lattice* h, int parity) {
   a.split = h->split;
   a.lanes = h->precision == SU3_FP64 ? su3_f64_lanes(h) : 1;
   a.pairs = h->pairs;
+  a.single = h->pairs && pairs_single(h->geom.Vh);
   a.pgeom = h->pgeom;
   a.tile2 = h->pairs ? su3k_pair_tile2(h->pgeom, h->threads) : 0;
   a.geom = h->geom;

@@ -20,14 +20,17 @@
 
 using namespace su3dev;
 
-// Register budget of the FP32-mixed half-sweep: __launch_bounds__(threads,
-// min blocks per SM).  The defaults keep every block size up to
-// kMaxSweepThreads legal.
+// Register budget of the FP32 half-sweep: __launch_bounds__(threads, min blocks
+// per SM), every block size up to kMaxSweepThreads legal.  Two blocks of 256
+// (126 registers, no spills) instead of four (64 registers): GB300, ms per sweep,
+// mixed and EFT: 18 x 10 x 14 x 22 0.0698 -> 0.0596 and 0.0593 -> 0.0475 (few
+// warps: more loads in flight each), 30^4 0.403 -> 0.402 and 0.385 -> 0.356, 42^4
+// 1.368 -> 1.370 and 1.324 -> 1.244.
 #ifndef SU3_F32_LB_THREADS
 #define SU3_F32_LB_THREADS kMaxSweepThreads
 #endif
 #ifndef SU3_F32_MINBLOCKS
-#define SU3_F32_MINBLOCKS 4
+#define SU3_F32_MINBLOCKS 2
 #endif
 
 namespace {
@@ -37,8 +40,8 @@ namespace {
 // ---------------------------------------------------------------------------
 // The same four-lane split for FP32 storage: rows 0,1 of the staple paths on
 // row pairs (12 floats each) are gathered into lane 0 and added in the
-// single-thread order; no register cap (small lattices leave the SMs nearly
-// empty).
+// single-thread order, and the random numbers of the three subgroups are drawn
+// side by side; no register cap (small lattices leave the SMs nearly empty).
 __device__ __forceinline__ pm3 shfl_pm3_rows01(const pm3& m, int src) {
   pm3 r;
 #pragma unroll
@@ -49,6 +52,12 @@ __device__ __forceinline__ pm3 shfl_pm3_rows01(const pm3& m, int src) {
     r.im[k].y = __shfl_sync(0xffffffffu, m.im[k].y, src);
   }
   return r;
+}
+
+__device__ __forceinline__ DrawF32 shfl_draw(const DrawF32& d, int src) {
+  return DrawF32{__shfl_sync(0xffffffffu, d.L, src),    __shfl_sync(0xffffffffu, d.u3, src),
+                 __shfl_sync(0xffffffffu, d.ct, src),   __shfl_sync(0xffffffffu, d.sn, src),
+                 __shfl_sync(0xffffffffu, d.sphi, src), __shfl_sync(0xffffffffu, d.cphi, src)};
 }
 
 template <int MU, bool STATS, bool EFT, bool PAIRS>
@@ -69,6 +78,12 @@ __global__ void __launch_bounds__(kMaxSweepThreads) k_half_sweep_f32_split(HalfS
     B = backward_path_p<false, PAIRS>(g, U, p, MU, nu, nb_half_rt(g, st, nu, -1), nb_half2_rt(g, st, MU, nu));
   }
   const int lane0 = (threadIdx.x & 31) & ~3;
+  // lane n < 3 draws subgroup n's numbers; lane 0 uses them all
+  const uint32_t s = (uint32_t)canon(g, st);
+  const DrawF32 mine = draw_f32<MU>(s, part < 3 ? part : 0, 0, *args.sweep, args.key);
+  DrawF32 draws[3];
+#pragma unroll
+  for (int n = 0; n < 3; ++n) draws[n] = shfl_draw(mine, lane0 + n);
   pm3 A;
   init_completed_p(A, F);
   acc_completed_p(A, B);
@@ -80,8 +95,26 @@ __global__ void __launch_bounds__(kMaxSweepThreads) k_half_sweep_f32_split(HalfS
   UpdateCount c{0, 0};
   if (part == 0 && active) {
     const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, 1, sweep_far(args.sweep)};
-    c = heatbath_f32_on<MU, EFT, false, false, PAIRS>(g, U, h, p, *args.sweep, (uint32_t)canon(g, st), args.key, uc, A,
-                                                       A, nullptr, load_pm3_l<false, PAIRS>(U, MU, p, h, g.Vh), true);
+    c = heatbath_f32_on<MU, EFT, false, false, PAIRS, true>(g, U, h, p, *args.sweep, s, args.key, uc, A, A, nullptr,
+                                                             load_pm3_l<false, PAIRS>(U, MU, p, h, g.Vh), true, draws);
+  }
+  count_stats<STATS>(c, args.stats);
+}
+
+// One thread per link of a site-paired store (small lattices).
+template <int MU, bool STATS, bool EFT>
+__global__ void __launch_bounds__(SU3_F32_LB_THREADS, SU3_F32_MINBLOCKS) k_half_sweep_f32_single(HalfSweepArgs args) {
+  const int h = blockIdx.x * blockDim.x + threadIdx.x;
+  UpdateCount c{0, 0};
+  if (h < args.geom.Vh) {
+    const Geometry& g = args.geom;
+    const UpdateConsts uc{args.three_over_beta_f64, args.three_over_beta, 1, nullptr};
+    float4* U = (float4*)args.links;
+    const Site st = site_of(g, h, args.parity);
+    const pm3 A = staple_p<MU, false, true>(g, U, st, h, args.parity);
+    c = heatbath_f32_on<MU, EFT, false, false, true>(g, U, h, args.parity, *args.sweep, (uint32_t)canon(g, st), args.key,
+                                                     uc, A, A, nullptr,
+                                                     load_pm3_l<false, true>(U, MU, args.parity, h, g.Vh), true);
   }
   count_stats<STATS>(c, args.stats);
 }
@@ -325,6 +358,20 @@ static cudaError_t launch_half_sweep_mu(const HalfSweepArgs& a, int precision, b
   const bool repeat = a.max_tries > 1;
   // FP32 in the site-paired layout: the paired kernel, except for the
   // four-lane form of small lattices
+  if (precision != 0 && a.pairs && a.single && !a.split && !repeat && !(MU > 0 && a.meas)) {
+    if (precision == 2) {
+      if (stats)
+        k_half_sweep_f32_single<MU, true, true><<<blocks, threads, 0, s>>>(a);
+      else
+        k_half_sweep_f32_single<MU, false, true><<<blocks, threads, 0, s>>>(a);
+    } else {
+      if (stats)
+        k_half_sweep_f32_single<MU, true, false><<<blocks, threads, 0, s>>>(a);
+      else
+        k_half_sweep_f32_single<MU, false, false><<<blocks, threads, 0, s>>>(a);
+    }
+    return cudaGetLastError();
+  }
   if (precision != 0 && a.pairs && !(a.split && !repeat && !(MU > 0 && a.meas)))
     return su3k_launch_half_sweep_pair(a, MU, precision == 2, stats, threads, s);
   if (MU > 0 && a.meas) {  // fused plaquette (statistics are not counted in these phases)

@@ -26,6 +26,7 @@ struct HalfSweepArgs {
   int lanes;                  // FP64 store: lanes per link (1, 4 or 8; k_half_sweep_f64_lanes)
   int chained;                // FP64 store, lanes > 1: programmatic dependent of the half-sweep launched before
   int pairs;                  // FP32 store in the site-paired layout (L3 a multiple of 4; su3_sitepair.cuh)
+  int single;                 // pairs only: one thread per link (small lattices; k_half_sweep_f32_single)
   su3dev::Geometry pgeom;     // the pair lattice L0 x L1 x L2 x L3/2 (pairs only)
   int tile2;                  // paired kernel: > 0 runs its blocks in tiles of tile2 x2-lines (su3_kernels_pair.cu)
 };

@@ -131,3 +131,64 @@ def test_near_identity_and_zero_entries():
         with su3.Lattice(L, beta, 3, start=su3.SU3_COLD) as lat:
             lat.sweep(2)
             assert np.abs(lat.get_links() - ref).max() <= 1e-12
+
+
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (4, 4, 4, 4), (6, 4, 10, 8), (8, 8, 8, 16), (10, 14, 6, 12)])
+@pytest.mark.parametrize("tries", [1, 6])
+def test_lanes_share_an_update_bit_for_bit(L, tries):
+    # One, four and the automatic number of lanes per link (eight up to 8^4), and
+    # batches (one lane, other launches): integer sums, so the same bits; the
+    # same acceptance counts.
+    got = []
+    for lanes in (1, 4, 0):
+        with su3.Lattice(L, BETA, 17, start=su3.SU3_HOT) as lat:
+            lat.set_lanes(lanes)
+            lat.set_heatbath(tries)
+            lat.set_stats(True)
+            lat.sweep(2)
+            lat.half_sweep(3, 1)
+            got.append((lat.get_links(), lat.stats()))
+    for links, stats in got[1:]:
+        assert np.array_equal(links, got[0][0])
+        assert stats == got[0][1]
+    with su3.Lattice(L, BETA, 17, start=su3.SU3_HOT) as lat, \
+            su3.Batch([L, (4, 4, 4, 4)], [BETA, 6.0], [17, 5], start=su3.SU3_HOT, precision=su3.SU3_FP64) as bt:
+        lat.set_heatbath(tries)
+        bt.set_heatbath(tries)
+        lat.sweep(2)
+        bt.sweep(2)
+        assert np.array_equal(lat.get_links(), bt.get_links(0))
+        assert lat.plaquette() == bt.plaquettes()[0]
+
+
+@pytest.mark.parametrize("L", [(2, 2, 2, 2), (6, 4, 10, 8), (2, 6, 2, 10), (16, 16, 16, 16)])
+def test_plaquette_of_proper_and_far_configurations(L):
+    # 1e-14: a sum of 6 V terms of at most 1e-15 each over 6 V (the parity tests' bound is 1e-13)
+    ref = oracle.hot_start(L, 8)
+    far = ref.copy()
+    far[0, 0, 0, 0, 1] *= 3.0
+    lost = ref.copy()
+    lost[0, 0, 0, 0, 1] = np.nan
+    with su3.Lattice(L, BETA, 3, start=su3.SU3_COLD) as lat:
+        assert lat.plaquette() == 1.0
+        lat.set_links(ref)
+        assert abs(lat.plaquette() - oracle.plaquette(L, ref)) <= 1e-14
+        lat.set_links(far)
+        assert abs(lat.plaquette() - oracle.plaquette(L, far)) <= 1e-14
+        lat.set_links(lost)
+        assert np.isnan(su3.load_library().su3_plaquette(lat.handle))
+        lat.set_links(ref)
+        assert abs(lat.plaquette() - oracle.plaquette(L, ref)) <= 1e-14
+
+
+@pytest.mark.parametrize("L", [(6, 6, 6, 4), (14, 14, 14, 8), (16, 16, 16, 16)])
+@pytest.mark.parametrize("prec", [su3.SU3_FP32_MIXED, su3.SU3_FP32_EFT])
+def test_fp32_one_thread_per_link_of_a_paired_store(L, prec):
+    # Small site-paired lattices run one thread per link; measuring sweeps run one
+    # thread per pair: the same chain, bit for bit.
+    with su3.Lattice(L, BETA, 23, precision=prec) as a, su3.Lattice(L, BETA, 23, precision=prec) as b:
+        a.set_lanes(1)
+        b.set_lanes(1)
+        a.sweep(2)
+        b.sweep_measured(2)
+        assert np.array_equal(a.get_links(), b.get_links())
