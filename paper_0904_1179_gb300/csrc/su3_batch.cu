@@ -456,9 +456,9 @@ int set_config(su3_lattice* h, int threads, int blocks_per_sm, int window) {
   return resched ? build_schedule(h) : SU3_OK;
 }
 
-int check_status(su3_lattice* h, const char* what) {
+// Waits for the stream, on which a copy of the status word to h_status is enqueued, and checks it.
+int check_copied_status(su3_lattice* h, const char* what) {
   su3_batch* b = h->batch;
-  SU3_CUDA(cudaMemcpyAsync(b->h_status, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream), what);
   const int rc = su3_sync(h, what);
   if (rc != SU3_OK) return rc;
   if (*b->h_status != 0) {
@@ -471,6 +471,12 @@ int check_status(su3_lattice* h, const char* what) {
                     what, (double)b->wait_ns * 1e-9);
   }
   return SU3_OK;
+}
+
+int check_status(su3_lattice* h, const char* what) {
+  su3_batch* b = h->batch;
+  SU3_CUDA(cudaMemcpyAsync(b->h_status, b->d_status, sizeof(int), cudaMemcpyDeviceToHost, h->stream), what);
+  return check_copied_status(h, what);
 }
 
 std::string tune_key_of(const su3_lattice* h) {
@@ -659,9 +665,9 @@ static int batch_links(su3_handle h, int replica, double* host, size_t n_doubles
   const long long V = 2LL * g.Vh;
   if (n_doubles != (size_t)V * 72) return su3_fail(SU3_ESIZE, "%s: n = %zu, expected %lld", what, n_doubles, V * 72);
   void* base = (char*)h->links + b->offsets[replica] * b->elem_bytes;
-  const int rc = su3_transfer(h, g, base, false, host, get, what);
+  const int rc = su3_transfer(h, g, base, false, host, get, what, b->d_status, b->h_status);
   if (rc != SU3_OK) return rc;
-  return check_status(h, what);
+  return check_copied_status(h, what);
 }
 
 int su3_batch_links_get(su3_handle h, int replica, double* host, size_t n_doubles) {

@@ -50,10 +50,12 @@ struct ConvArgs {
   su3dev::Geometry geom;
   int precision;
   long long s_begin, n_sites;
-  double* canon;  // device staging buffer, canonical layout of the chunk
+  double* canon;  // canonical layout of the chunk: the device staging buffer, or (from the store) page-locked memory
   void* links;
   int pairs;  // FP32 store in the site-paired layout
   int* far;   // SweepState's flag, set where the FP64 store takes a link far from SU(3)
+  const int* status = nullptr;  // a batch's status word (device) and where the conversion from the store
+  int* status_host = nullptr;   // copies it (page-locked); null: not copied
 };
 
 // Whether an FP32 store of an L0 x L1 x L2 x L3 lattice uses the site-paired

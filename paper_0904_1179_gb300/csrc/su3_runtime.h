@@ -71,12 +71,13 @@ int su3_fail(int code, const char* fmt, ...);
 int su3_cuda_fail(cudaError_t e, const char* what);
 int su3_sync(su3_lattice* h, const char* what);
 // Copy a configuration (geometry g, device store at `links`) to or from a host
-// buffer in the canonical layout, chunk by chunk: host<->device copies on a
+// buffer in the canonical layout: to page-locked memory by the conversion
+// kernel's own stores, else chunk by chunk, where host<->device copies on a
 // second stream overlap the layout conversions on the handle's stream (one
 // chunk: on that stream alone).  Synchronises, except for batches: their caller
-// does, reading the sweep status with it.
+// does, reading their status word, which is copied to status_host, with it.
 int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pairs, double* host, bool get,
-                 const char* what);
+                 const char* what, const int* status = nullptr, int* status_host = nullptr);
 // Lanes per link of an FP64 half-sweep of this lattice (1, 4 or 8).
 int su3_f64_lanes(const su3_lattice* h);
 // Free a handle and everything it owns (batch part included).
