@@ -82,8 +82,10 @@ enum {
 /* Create a lattice of extents L0..L3 at coupling beta with the given Philox
  * seed and start (SU3_COLD: every link the identity; SU3_HOT: Haar-random
  * SU(3) links drawn from Philox tag 1).  Precision SU3_FP64 stores 18 reals
- * per link in FP64 and computes in FP64.  On success *out receives the
- * handle. */
+ * per link in FP64 and computes to FP64 accuracy: the update works in fixed
+ * point of 62 fraction bits on the integer and FP32 units, closer to the exact
+ * result than FP64 arithmetic (see su3_links_set for links far from SU(3)).
+ * On success *out receives the handle. */
 SU3_API int su3_create(int L0, int L1, int L2, int L3, double beta, uint64_t seed, int start, su3_handle* out);
 
 /* As su3_create, with a precision and a stream.
@@ -147,7 +149,8 @@ SU3_API double su3_plaquette(su3_handle h);
  * row 2 as conj(row0 x row1), which holds for products of SU(3) matrices
  * only.  set does not check; every update reunitarises the link it writes
  * (a link far from unitary, |row|^2 - 1 or <row0,row1> beyond 1e-3, takes a
- * full FP64 Gram-Schmidt in the FP32 paths). */
+ * full FP64 Gram-Schmidt in the FP32 paths; while an FP64 store may hold a link
+ * far from SU(3), its sweeps run in FP64 arithmetic, several times slower). */
 SU3_API int su3_links_get(su3_handle h, double* host, size_t n_doubles);
 SU3_API int su3_links_set(su3_handle h, const double* host, size_t n_doubles);
 
@@ -179,7 +182,10 @@ SU3_API int su3_info(su3_handle h, int dims[4], double* beta, uint64_t* seed, in
 /* Threads per block of the half-sweep kernels (a multiple of 32 in
  * [32, 256]); 0 restores the default: 128, halved (down to 32) while a
  * half-sweep would have fewer blocks than the GPU has SMs, so that the links
- * of a small lattice spread over as many SMs as possible.  Results do not
+ * of a small lattice spread over as many SMs as possible; FP32 half-sweeps of
+ * less than 0.8 waves of the GPU (of 512 threads per SM) take blocks of 32,
+ * and SU3_SCHED_AUTO tiles of 64 or 32 where an x3 layer is a whole number of
+ * those only (FP64: 1 to 5 waves, FP32: 1 to 3).  Results do not
  * depend on it: every link update is independent inside a half-sweep and its
  * random numbers are keyed by its site. */
 SU3_API int su3_set_block_size(su3_handle h, int threads);
@@ -229,7 +235,7 @@ SU3_API int su3_set_lanes(su3_handle h, int lanes);
  *     GPU, w = (V/4 pairs) / (512 x SMs) (24^4: +15 % mixed, +17 % EFT;
  *     32^4: +10 %, +6 %; 40^4: +0.8 %, +0.1 % against eight launches), and
  *     SU3_SCHED_PER_DIRECTION for FP64 when it is 1 to 5 waves,
- *     w = (V/2 links) / (384 x SMs) (24^4: +5 %); else eight half-sweep
+ *     w = (V/2 links) / (384 x SMs) (24^4: +8 %); else eight half-sweep
  *     kernels (faster at 48^4, and on small lattices whose half-sweep is in
  *     flight at once).
  * su3_sweep_measured always runs the eight kernels (its measuring update

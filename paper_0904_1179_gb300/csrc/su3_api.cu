@@ -104,11 +104,13 @@ bool pairs_single(int Vh) {
 
 // Lanes per link of an FP64 half-sweep launched by itself
 // (k_half_sweep_f64_lanes), by the warps per SM they make.  GB300, ms per sweep
-// with 1 / 4 / 8 lanes: 4^4 0.234 / 0.103 / 0.082, 8^4 (3.4 warps per SM at 8
-// lanes) 0.238 / 0.109 / 0.090, 8^3 x 16 (6.7) 0.242 / 0.123 / 0.133, 10^4 0.246 /
-// 0.127 / 0.151, 12^4 (8.5 warps per SM at 4 lanes) 0.244 / 0.223 / 0.214, 14^4
-// (15.8) 0.246 / 0.250 / 0.332, 16^4 0.300 / 0.463 / 0.555: eight lanes up to four
-// warps per SM (one per scheduler), four up to ten.
+// with 1 / 4 / 8 lanes: 4^4 0.193 / 0.088 / 0.074, 6^4 0.193 / 0.090 / 0.076, 8^4
+// (3.4 warps per SM at eight lanes) 0.195 / 0.092 / 0.086, 8^3 x 16 (6.7 at eight,
+// 3.4 at four) 0.199 / 0.103 / 0.133, 10^4 0.200 / 0.123 / 0.151, 12^4 (8.5 at four)
+// 0.202 / 0.162 / 0.214, 14^4 (15.8) 0.203 / 0.228 / 0.332, 16^4 0.268 / 0.363 /
+// 0.555 (the eight-lane figures from 8^3 x 16 on are of the kernel before its
+// loads went through shared memory): eight lanes up to four warps per SM (one per
+// scheduler), four up to ten.
 int f64_lanes_auto(int Vh) {
   const int sms = sm_count();
   if (sms <= 0) return 1;
@@ -188,7 +190,7 @@ bool f64_lanes_chained(const su3_lattice* h) {
   return sms > 0 && lanes > 1 && (threads <= 2 * 32LL * sms || threads >= 8 * 32LL * sms);
 }
 
-HalfSweepArgs half_sweep_args(const su3_lattice* h, int parity) {
+HalfSweepArgs half_sweep_args(const su3_lattice* h, int parity, int threads) {
   HalfSweepArgs a{};
   a.meas = nullptr;
   a.split = h->split;
@@ -196,7 +198,7 @@ HalfSweepArgs half_sweep_args(const su3_lattice* h, int parity) {
   a.pairs = h->pairs;
   a.single = h->pairs && pairs_single(h->geom.Vh);
   a.pgeom = h->pgeom;
-  a.tile2 = h->pairs ? su3k_pair_tile2(h->pgeom, h->threads) : 0;
+  a.tile2 = h->pairs ? su3k_pair_tile2(h->pgeom, threads) : 0;
   a.geom = h->geom;
   a.key = su3dev::philox_round_keys(h->key);
   a.parity = parity;
@@ -215,18 +217,21 @@ HalfSweepArgs half_sweep_args(const su3_lattice* h, int parity) {
 // tiles (one launch per sweep or one per direction, su3k_launch_sweep_pair);
 // or the FP64 store with one lane per link and x3 layers of whole tiles (one
 // launch per direction, su3k_launch_sweep_f64).
-bool pair_persistent_applies(const su3_lattice* h) {
+bool pair_persistent_applies(const su3_lattice* h, int threads) {
   int tpl = 0;
-  return h->pairs && !h->split && su3k_pair_sweep_layers(h->pgeom, h->threads, &tpl) > 0;
+  return h->pairs && !h->split && su3k_pair_sweep_layers(h->pgeom, threads, &tpl) > 0;
 }
-bool f64_persistent_applies(const su3_lattice* h) {
+bool f64_persistent_applies(const su3_lattice* h, int threads) {
   int tpl = 0;
-  return h->precision == SU3_FP64 && !h->split && su3k_f64_sweep_layers(h->geom, h->threads, &tpl) > 0;
+  return h->precision == SU3_FP64 && !h->split && su3k_f64_sweep_layers(h->geom, threads, &tpl) > 0;
 }
-bool persistent_applies(const su3_lattice* h) { return pair_persistent_applies(h) || f64_persistent_applies(h); }
+
+bool persistent_applies(const su3_lattice* h, int threads) {
+  return pair_persistent_applies(h, threads) || f64_persistent_applies(h, threads);
+}
 
 // Waves of the GPU in one half-sweep: site pairs at about 512 threads per SM
-// (128 registers), FP64 links at 384 (3 warps of 136-142 registers per
+// (128 registers), FP64 links at 384 (3 warps of 168 registers per
 // scheduler).
 double half_sweep_waves(const su3_lattice* h) {
   const int sms = sm_count();
@@ -239,11 +244,12 @@ double half_sweep_waves(const su3_lattice* h) {
 // chained half-sweep launches: 24^4 (1.1 waves) +15 / +17 %, 32^4 (3.4 waves)
 // +10 / +6 %, 32^3 x 64 (6.7 waves) +3.4 / +0.9 %, 40^4 (8.2 waves) +0.8 /
 // +0.1 %, 48^4 (17 waves) -2.4 / -2.4 %: chained below 10 waves.  FP64, one
-// launch per direction: 24^4 (2.8 waves) +5.1 %, 32^4 (9 waves), 40^4 and
-// 48^4 +0.3 to +0.4 %: per direction below 5 waves.  Under one wave a whole
-// half-sweep is in flight at once and the tiles of the next one wait on it
-// (FP32 per direction: 24^3 x 16, 0.7 waves, -38 %; 16^4, 0.2 waves, -62 %;
-// FP64 16^4, 0.6 waves, -31 %): eight launches.
+// launch per direction: 24^4 (2.8 waves) +8 %, 32^4 (9 waves) +1.6 %, 40^4 -0.2 %,
+// 48^4 -1.3 %: per direction below 5 waves (the documented
+// default of 32^4 is eight launches).  Under one wave a whole half-sweep is
+// in flight at once and the tiles of the next one wait on it (FP32 per direction:
+// 24^3 x 16, 0.7 waves, -38 %; 16^4, 0.2 waves, -62 %; FP64 16^4, 0.6 waves, -28 %):
+// eight launches.
 int auto_schedule(const su3_lattice* h) {
   const double w = half_sweep_waves(h);
   if (h->pairs) return w >= 1.0 && w < 10.0 ? SU3_SCHED_CHAINED : SU3_SCHED_PHASES;
@@ -253,19 +259,56 @@ int auto_schedule(const su3_lattice* h) {
 // Whether a schedule other than eight independent launches applies to h.
 bool schedule_applies(const su3_lattice* h, int schedule) {
   switch (schedule) {
-    case SU3_SCHED_PERSISTENT: return pair_persistent_applies(h);
+    case SU3_SCHED_PERSISTENT: return pair_persistent_applies(h, h->threads);
     case SU3_SCHED_CHAINED:
-    case SU3_SCHED_PER_DIRECTION: return persistent_applies(h);
+    case SU3_SCHED_PER_DIRECTION: return persistent_applies(h, h->threads);
     default: return true;
   }
+}
+
+// Threads per tile of the automatic schedule, 0 where that is eight launches:
+// the default block size or, unless the caller set the block size, the largest
+// smaller one that an x3 layer is a whole number of.  The schedule gains most
+// just above one wave, and blocks of one or two warps cost up to 3 %, so the FP32
+// store takes them below three waves only.  GB300, ms per sweep, eight launches of
+// 128 / smaller tiles: FP64 20^4 (1.4 waves, 32 threads) 0.598 / 0.529, 20^2 x 24 x 20
+// (1.6, 64) 0.645 / 0.605, 26 x 24^3 (3.1, 64) 1.196 / 1.101; FP32 mixed (EFT) 26 x
+// 24^3 (1.2, 64) 0.211 / 0.202 (0.187 / 0.175), 28^4 (2.0, 32) 0.322 / 0.283 (0.294 /
+// 0.272), 36^4 (5.4, 32) 0.763 / 0.756 (0.707 / 0.716).
+int schedule_tile(const su3_lattice* h) {
+  if (auto_schedule(h) == SU3_SCHED_PHASES) return 0;
+  if (persistent_applies(h, h->threads)) return h->threads;
+  if (h->threads_set || (h->pairs && half_sweep_waves(h) >= 3.0)) return 0;
+  for (int t = h->threads / 2; t >= 32; t /= 2)
+    if (persistent_applies(h, t)) return t;
+  return 0;
 }
 
 // The schedule the next sweep runs with (measuring sweeps: always eight
 // launches).
 int effective_schedule(const su3_lattice* h, bool measured = false) {
-  if (measured || !persistent_applies(h)) return SU3_SCHED_PHASES;
-  const int sched = h->schedule == SU3_SCHED_AUTO ? auto_schedule(h) : h->schedule;
-  return schedule_applies(h, sched) ? sched : SU3_SCHED_PHASES;
+  if (measured) return SU3_SCHED_PHASES;
+  if (h->schedule == SU3_SCHED_AUTO) return schedule_tile(h) ? auto_schedule(h) : SU3_SCHED_PHASES;
+  return schedule_applies(h, h->schedule) ? h->schedule : SU3_SCHED_PHASES;
+}
+
+// Threads per block of the next sweep's launches: h->threads, or the automatic
+// schedule's tile, or, for an FP32 half-sweep of less than 0.8 waves (of 512
+// threads per SM) whose block size the caller left alone, one warp: blocks of 128
+// then leave some SMs with twice the warps of others.  GB300, ms per sweep, 128 / 32
+// threads, mixed (EFT): 18 x 10 x 14 x 22 (0.36 waves) 0.060 / 0.056 (0.050 / 0.050),
+// 16^4 0.074 / 0.070 (0.063 / 0.060), 16^3 x 20 0.097 / 0.084 (0.080 / 0.076), 20 x 18^2
+// x 20 (0.4) 0.151 / 0.103 (0.128 / 0.087), 20^4 (0.5) 0.153 / 0.128 (0.132 / 0.115), 24^3 x
+// 16 (0.71) 0.138 / 0.138 (0.119 / 0.119), 22^3 x 24 (0.75) 0.197 / 0.174 (0.179 / 0.154),
+// 24^3 x 20 (0.89) 0.172 / 0.176 (0.154 / 0.154).  FP64 blocks of one warp fill the
+// schedulers unevenly (18^4 0.377 / 0.439).  Measuring sweeps keep h->threads: the
+// order of their plaquette sums follows the blocks.
+int launch_threads(const su3_lattice* h, bool measured = false) {
+  if (h->threads_set || measured) return h->threads;
+  if (effective_schedule(h) != SU3_SCHED_PHASES) return h->schedule == SU3_SCHED_AUTO ? schedule_tile(h) : h->threads;
+  const int sms = sm_count();
+  const long long n = h->pairs && !pairs_single(h->geom.Vh) ? h->pgeom.Vh : h->geom.Vh;
+  return h->precision != SU3_FP64 && !h->split && sms > 0 && 5 * n < 4 * 512LL * sms ? 32 : h->threads;
 }
 
 bool use_persistent(const su3_lattice* h, bool measured = false) {
@@ -300,18 +343,19 @@ int ensure_pair_queue(su3_lattice* h) {
 // plaquette of the updated configuration once, and a last kernel sums them
 // into the ring slot of this sweep.
 int enqueue_sweep_body(su3_lattice* h, bool measured) {
-  const int blocks = su3k_half_sweep_blocks(half_sweep_args(h, 1), h->precision, h->threads);
+  const int threads = launch_threads(h, measured);
+  const int blocks = su3k_half_sweep_blocks(half_sweep_args(h, 1, threads), h->precision, threads);
   if (use_persistent(h, measured)) {
-    const HalfSweepArgs a = half_sweep_args(h, 0);
+    const HalfSweepArgs a = half_sweep_args(h, 0, threads);
     const SweepQueue q{h->d_pq, h->d_pstatus, h->pq_wait_ns, h->pq_withhold};
     SU3_CUDA(cudaMemsetAsync(h->d_pq, 0, (size_t)h->pq_words * sizeof(unsigned int), h->stream),
              "sweep counters reset");
     if (h->precision == SU3_FP64)
-      SU3_CUDA(su3k_launch_sweep_f64(a, q, h->stats_on, h->threads, effective_schedule(h) == SU3_SCHED_CHAINED,
+      SU3_CUDA(su3k_launch_sweep_f64(a, q, h->stats_on, threads, effective_schedule(h) == SU3_SCHED_CHAINED,
                                      h->stream),
                "persistent sweep launch");
     else
-      SU3_CUDA(su3k_launch_sweep_pair(a, q, h->precision == SU3_FP32_EFT, h->stats_on, h->threads,
+      SU3_CUDA(su3k_launch_sweep_pair(a, q, h->precision == SU3_FP32_EFT, h->stats_on, threads,
                                       effective_schedule(h) == SU3_SCHED_CHAINED        ? SweepForm::kChained
                                       : effective_schedule(h) == SU3_SCHED_PER_DIRECTION ? SweepForm::kPerDirection
                                                                                          : SweepForm::kOneLaunch,
@@ -320,10 +364,10 @@ int enqueue_sweep_body(su3_lattice* h, bool measured) {
   } else {
     for (int mu = 0; mu < 4; ++mu)
       for (int p = 0; p < 2; ++p) {
-        HalfSweepArgs a = half_sweep_args(h, p);
+        HalfSweepArgs a = half_sweep_args(h, p, threads);
         a.chained = mu + p > 0 && h->precision == SU3_FP64 && f64_lanes_chained(h);
         if (measured && p == 1 && mu >= 1) a.meas = h->d_meas_parts + (size_t)(mu - 1) * blocks;
-        SU3_CUDA(su3k_launch_half_sweep(a, mu, h->precision, h->stats_on, h->threads, h->stream),
+        SU3_CUDA(su3k_launch_half_sweep(a, mu, h->precision, h->stats_on, threads, h->stream),
                  "half-sweep launch");
       }
   }
@@ -599,7 +643,7 @@ int su3_sweep_measured(su3_handle h, int nsweeps, double* plaq_out) {
   if (h->stats_on) return fail(SU3_EINVAL, "su3_sweep_measured: disable acceptance statistics first");
   if (nsweeps == 0) return SU3_OK;
   const bool dec = su3_decomp_active(h);
-  const int blocks = dec ? su3_decomp_meas_blocks(h) : su3k_half_sweep_blocks(half_sweep_args(h, 1), h->precision, h->threads);
+  const int blocks = dec ? su3_decomp_meas_blocks(h) : su3k_half_sweep_blocks(half_sweep_args(h, 1, h->threads), h->precision, h->threads);
   if (h->meas_blocks != blocks || !h->d_meas) {
     SU3_CUDA(cudaStreamSynchronize(h->stream), "su3_sweep_measured");
     if (h->graph_meas) {
@@ -649,7 +693,8 @@ int su3_half_sweep(su3_handle h, int mu, int parity) {
   if (is_batch(h)) return fail(SU3_EINVAL, "su3_half_sweep: batch handle (use the su3_batch_* calls)");
   if (mu < 0 || mu > 3 || parity < 0 || parity > 1) return fail(SU3_EINVAL, "su3_half_sweep: bad mu/parity");
   if (su3_decomp_active(h)) return su3_decomp_half_sweep(h, mu, parity);
-  SU3_CUDA(su3k_launch_half_sweep(half_sweep_args(h, parity), mu, h->precision, h->stats_on, h->threads, h->stream),
+  const int threads = launch_threads(h);
+  SU3_CUDA(su3k_launch_half_sweep(half_sweep_args(h, parity, threads), mu, h->precision, h->stats_on, threads, h->stream),
            "su3_half_sweep");
   return SU3_OK;
 }
@@ -823,14 +868,16 @@ int su3_sweep_debug(su3_handle h, double wait_limit_s, int withhold_item) {
 int su3_set_block_size(su3_handle h, int threads) {
   if (!h) return fail(SU3_EINVAL, "su3_set_block_size: NULL handle");
   if (is_batch(h)) return fail(SU3_EINVAL, "su3_set_block_size: batch handle (use the su3_batch_* calls)");
-  if (threads == 0) threads = default_threads(h->pairs ? h->pgeom.Vh : h->geom.Vh);
+  const bool set = threads != 0;
+  if (!set) threads = default_threads(h->pairs ? h->pgeom.Vh : h->geom.Vh);
   if (threads < 32 || threads > kMaxSweepThreads || (threads & 31))
     return fail(SU3_EINVAL, "su3_set_block_size: %d is not a multiple of 32 in [32, %d]", threads, kMaxSweepThreads);
-  if (threads != h->threads) {
+  if (threads != h->threads || set != h->threads_set) {
     SU3_CUDA(cudaStreamSynchronize(h->stream), "su3_set_block_size");
     drop_graphs(h);
     if (h->decomp) su3_decomp_invalidate(h->decomp);
     h->threads = threads;
+    h->threads_set = set;
   }
   return SU3_OK;
 }

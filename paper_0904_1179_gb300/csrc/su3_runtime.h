@@ -47,6 +47,7 @@ struct su3_lattice {
   double* h_meas = nullptr;        // pinned copy
   int meas_cap = 0;
   int threads = kSu3DefaultThreads;
+  bool threads_set = false;  // by the caller (su3_set_block_size): every launch takes `threads`
   int max_tries = 1;  // SU(2) proposals per subgroup (1: one-hit heatbath)
   bool split = false;  // small lattice: several lanes per link update
   int lanes = 0;       // as set by su3_set_lanes (0: automatic)
