@@ -51,18 +51,6 @@ PAPER_TABLE1_SECONDS = [48.2, 48.3, 48.7, 48.9]
 # of the other directions are read once, the V/2 updated links written once:
 # 9 links moved per update.
 BYTES_PER_UPDATE = {"fp64": 9 * 18 * 8, "fp32_mixed": 9 * 12 * 4}
-# FP64 floating-point operations per link update of the FP64 kernel as written
-# (an FMA counts 2; transcendental calls, square roots and divisions are not
-# counted):
-#   staple 2070: 6 paths x 2 products of rows 0,1 (or columns 0,1) = 12 x 144,
-#     first path's row completion 42, 5 accumulations with the row completion
-#     fused in, 60 each;
-#   three SU(2) steps 254 + 254 + 212 = 720: projection 100, |r|^2 and
-#     1/alpha 8, uniforms 6, Kennedy-Pendleton proposal and test 8, a0 and the
-#     direction 8, quaternions 8, SU(2) matrix 32, rotation of rows (i, j) 84
-#     (42 in the last step, whose row 2 is rebuilt by Gram-Schmidt);
-#   Gram-Schmidt 84 and row completion 42.
-FP64_FLOP_PER_UPDATE = 2070 + 720 + 126
 
 
 def peaks():
@@ -82,7 +70,7 @@ def peaks():
 # units that define and launch the kernel and every csrc/*.cuh, comments
 # stripped).  A line reports the figure only while that code still hashes the
 # same; otherwise its traffic is null and the line says why.
-_U_F64, _U_F32, _U_BATCH = ("su3_kernels.cu",), ("su3_kernels.cu", "su3_kernels_pair.cu"), ("su3_batch.cu",)
+_U_F64, _U_F32, _U_BATCH = ("su3_kernels_f64.cu",), ("su3_kernels.cu", "su3_kernels_pair.cu"), ("su3_batch.cu",)
 _SHA_F64 = "885129abed2f07dcf526279300c7e616b6ab6d05d7f194316ac183375be7f880"
 _SHA_F32 = "b69b3efb95b8c7b71cd98f8e15af6aec0aaf08bce33ea207b3a093f079754790"
 _SHA_BATCH = "d9029b824bda46a252b5670089d82c5b7d10b27581aefd95730e21efa98e8ad2"
@@ -160,13 +148,6 @@ def traffic_of(variant):
         return None, "kernel sources changed since the ncu capture (%s)" % rec["capture"]
     return rec["bytes"], "ncu capture: %s; code sha256 of %s and csrc/*.cuh: %s" % (
         rec["capture"], ", ".join(rec["units"]), rec["sources_sha256"][:16])
-
-# FP64 peak of GB300 from unit counts and clock: 152 SMs x 2 FP64 FMA per
-# clock (1/64 of the 128 FP32 lanes) x 2 flop x 2.070 GHz = 1.2586 TFLOP/s
-# (the nominal 1.25).  An FMA-loop probe reached 1.006 TFLOP/s (0.80 of it);
-# both are reported.
-FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.070e9 / 1e12
-FP64_PROBE_TFLOPS = 1.006
 
 
 class ClockSampler:
@@ -1012,8 +993,8 @@ def main():
     secs, all_units = reduce_max_sum(world, total_ms * 1e-3, units, device)
     value = all_units / secs
     kernel_ms = statistics.mean(sweep_ms) / 8
-    flop_per_launch = FP64_FLOP_PER_UPDATE * (V // 2)
-    achieved_tf = flop_per_launch / (kernel_ms * 1e-3) / 1e12
+    bytes_per_launch = BYTES_PER_UPDATE["fp64"] * (V // 2)
+    achieved = bytes_per_launch / (kernel_ms * 1e-3) / 1e9
 
     if rank != 0:
         barrier(world)
@@ -1050,14 +1031,12 @@ def main():
         "e2e": e2e,
         "gpu_launches": args.steps * SWEEPS_PER_STEP * 9,
         "gpu_launches_note": "headline timed region: per sweep 8 half-sweep kernels + 1 sweep-counter kernel",
-        "roofline": {"bound": "alu", "achieved": achieved_tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                     "frac": achieved_tf / FP64_PEAK_TFLOPS, "traffic": traffic_of("fp64")[0],
-                     "traffic_source": traffic_of("fp64")[1],
-                     "peak_kind": "derived: 152 SMs x 2 FP64 FMA/clock x 2 flop x 2.070 GHz",
-                     "probe_peak": FP64_PROBE_TFLOPS, "frac_of_probe": achieved_tf / FP64_PROBE_TFLOPS,
-                     "kernel": "k_half_sweep_f64", "flop_per_launch": flop_per_launch, "kernel_ms": kernel_ms,
-                     "hbm_frac": BYTES_PER_UPDATE["fp64"] * (V // 2) / (kernel_ms * 1e-3) / 1e9 / hbm_peak,
-                     "hbm_peak": hbm_peak, "hbm_peak_kind": peak_kind},
+        # the kernel works on the integer and FP32 pipes, in fixed point; what limits it is instruction issue
+        "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
+                     "frac": achieved / hbm_peak, "peak_kind": peak_kind,
+                     "traffic": traffic_of("fp64")[0], "traffic_source": traffic_of("fp64")[1],
+                     "kernel": "k_half_sweep_f64", "bytes_per_launch": bytes_per_launch, "kernel_ms": kernel_ms,
+                     "limited_by": "instruction issue (integer and FP32 pipes), not DRAM"},
         "cpu_baseline": cpu,
         "variants": variants,
     }

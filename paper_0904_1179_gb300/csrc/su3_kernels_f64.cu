@@ -4,13 +4,17 @@
 // argument, so that one copy of its code serves the four directions.
 //
 // The same update in FP64 arithmetic kept the FP64 pipe (two lanes per SM) busy
-// for 93 % of 13.2 ms per 32^4 sweep.  With the matrix products of the staple,
-// the rotations and the reunitarisation on the integer multiplier and FP32 (1.76
-// SM cycles per multiply-add and warp instead of 16) a sweep took 5.15 ms; with
-// the scalars of the proposals there too (su3_fx_kp.cuh) and the subgroups in
-// one loop (instruction fetch had become the largest stall: 2.4 of 6.6 cycles
-// per instruction) 3.90 ms.  Now 20,000 instructions per warp at 0.51 issued
-// per cycle and scheduler; waits for instructions are still the first stall.
+// for 93 % of 13.2 ms per 32^4 sweep.  What changed it, ms per sweep: the matrix
+// products of the staple, the rotations and the reunitarisation on the integer
+// multiplier and FP32 (1.76 SM cycles per multiply-add and warp instead of 16)
+// 5.15; the scalars of the proposals there too (su3_fx_kp.cuh) and the subgroups
+// in one loop (instruction fetch had become the largest stall) 3.90; the staple's
+// links copied ahead into shared memory and no spills 3.35; neighbour steps
+// looked up and row pairs on the paired FMA 3.20.  Now 17,100 instructions per
+// warp at 0.57 issued per cycle and scheduler; what holds the rest are
+// fixed-latency dependencies (1.2 of 5.1 cycles per instruction) and the shared
+// integer pipe (0.7) at three warps per scheduler, which 168 registers allow.
+// DRAM moves at a quarter of its rate.
 #include "su3_kernels.h"
 
 #include "su3_device.cuh"
@@ -21,9 +25,9 @@
 
 using namespace su3dev;
 
-// Registers per thread.  GB300, 32^4, ms per sweep: 128 registers 4.52, 144: 4.44,
-// 168: 4.18, 200: 4.61.  168 is the most that keeps 12 warps on an SM; blocks of
-// 256 threads stay legal.
+// Registers per thread.  GB300, ms per sweep of 32^4 / 24^4 in eight launches: 128
+// registers 3.61 / 1.267, 136: 3.32 / 1.149, 144: 3.45 / 1.171, 168: 3.20 / 1.120.
+// 168 is the most that keeps 12 warps on an SM; blocks of 256 threads stay legal.
 #ifndef SU3_F64_REGS
 #define SU3_F64_REGS 168
 #endif
