@@ -159,11 +159,9 @@ void release(su3_lattice* h) {
   cudaFree(h->d_sweep);
   cudaFree(h->d_stats);
   cudaFree(h->d_partials);
-  cudaFree(h->d_plaq);
   cudaFree(h->d_stage);
   cudaFree(h->d_stage2);
   cudaFree(h->d_meas_parts);
-  cudaFree(h->d_meas);
   cudaFreeHost(h->h_meas);
   for (int b = 0; b < 2; ++b) {
     if (h->ev_copied[b]) cudaEventDestroy(h->ev_copied[b]);
@@ -372,7 +370,7 @@ int enqueue_sweep_body(su3_lattice* h, bool measured) {
       }
   }
   if (measured)
-    SU3_CUDA(su3k_launch_meas_final(h->d_meas_parts, 3 * blocks, 1.0 / (6.0 * (double)h->V), h->d_sweep, h->d_meas,
+    SU3_CUDA(su3k_launch_meas_final(h->d_meas_parts, 3 * blocks, 1.0 / (6.0 * (double)h->V), h->d_sweep, h->h_meas,
                                     h->meas_cap, h->stream),
              "plaquette reduction launch");
   SU3_CUDA(su3k_launch_increment(h->d_sweep, 1, h->stream), "sweep counter launch");
@@ -585,7 +583,6 @@ int su3_create_ex(int L0, int L1, int L2, int L3, double beta, uint64_t seed, in
       (e = cudaMalloc(&h->d_sweep, sizeof(su3dev::SweepState))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_stats, 2 * sizeof(unsigned long long))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_partials, (size_t)nparts * sizeof(double))) != cudaSuccess ||
-      (e = cudaMalloc(&h->d_plaq, sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_stage, (size_t)chunk * 4 * 18 * sizeof(double))) != cudaSuccess ||
       (e = cudaMallocHost(&h->h_plaq, sizeof(double))) != cudaSuccess ||
       (e = cudaMallocHost(&h->h_stats, 2 * sizeof(unsigned long long))) != cudaSuccess) {
@@ -644,7 +641,7 @@ int su3_sweep_measured(su3_handle h, int nsweeps, double* plaq_out) {
   if (nsweeps == 0) return SU3_OK;
   const bool dec = su3_decomp_active(h);
   const int blocks = dec ? su3_decomp_meas_blocks(h) : su3k_half_sweep_blocks(half_sweep_args(h, 1, h->threads), h->precision, h->threads);
-  if (h->meas_blocks != blocks || !h->d_meas) {
+  if (h->meas_blocks != blocks || !h->h_meas) {
     SU3_CUDA(cudaStreamSynchronize(h->stream), "su3_sweep_measured");
     if (h->graph_meas) {
       cudaGraphExecDestroy(h->graph_meas);
@@ -655,9 +652,8 @@ int su3_sweep_measured(su3_handle h, int nsweeps, double* plaq_out) {
     h->d_meas_parts = nullptr;
     SU3_CUDA(cudaMalloc(&h->d_meas_parts, (size_t)3 * blocks * sizeof(double)), "su3_sweep_measured: partials");
     h->meas_blocks = blocks;
-    if (!h->d_meas) {
+    if (!h->h_meas) {
       h->meas_cap = 4096;
-      SU3_CUDA(cudaMalloc(&h->d_meas, (size_t)h->meas_cap * sizeof(double)), "su3_sweep_measured: ring");
       SU3_CUDA(cudaMallocHost(&h->h_meas, (size_t)h->meas_cap * sizeof(double)), "su3_sweep_measured: ring");
     }
   }
@@ -670,16 +666,6 @@ int su3_sweep_measured(su3_handle h, int nsweeps, double* plaq_out) {
     const uint64_t t0 = h->sweep_host;
     for (int i = 0; i < n; ++i) SU3_CUDA(cudaGraphLaunch(exec, h->stream), "su3_sweep_measured: graph launch");
     h->sweep_host += (uint64_t)n;
-    // copy back only the n slots just written (two pieces where they wrap)
-    const int first = (int)(t0 % (uint64_t)h->meas_cap);
-    const int n1 = n < h->meas_cap - first ? n : h->meas_cap - first;
-    SU3_CUDA(cudaMemcpyAsync(h->h_meas + first, h->d_meas + first, (size_t)n1 * sizeof(double),
-                             cudaMemcpyDeviceToHost, h->stream),
-             "su3_sweep_measured: copy");
-    if (n > n1)
-      SU3_CUDA(cudaMemcpyAsync(h->h_meas, h->d_meas, (size_t)(n - n1) * sizeof(double), cudaMemcpyDeviceToHost,
-                               h->stream),
-               "su3_sweep_measured: copy");
     rc = sync(h, "su3_sweep_measured");
     if (rc != SU3_OK) return rc;
     for (int i = 0; i < n; ++i) plaq_out[done + i] = h->h_meas[(t0 + (uint64_t)i) % (uint64_t)h->meas_cap];
@@ -707,9 +693,8 @@ double su3_plaquette(su3_handle h) {
   if (su3_decomp_sync_global(h) != SU3_OK) return NAN;
   PlaqArgs a{h->geom, h->links, h->d_partials, h->pairs ? 1 : 0};
   cudaError_t e = h->precision == SU3_FP64
-                      ? su3k_launch_plaquette_f64(a, su3dev::sweep_far(h->d_sweep), h->d_plaq, h->stream)
-                      : su3k_launch_plaquette(a, h->precision, h->d_plaq, h->stream);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(h->h_plaq, h->d_plaq, sizeof(double), cudaMemcpyDeviceToHost, h->stream);
+                      ? su3k_launch_plaquette_f64(a, su3dev::sweep_far(h->d_sweep), h->h_plaq, h->stream)
+                      : su3k_launch_plaquette(a, h->precision, h->h_plaq, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) {
     cuda_fail(e, "su3_plaquette");

@@ -273,8 +273,7 @@ struct su3_batch {
   int2* d_plaq_items = nullptr;  // k_batch_plaquette: (replica, block)
   int* d_plaq_starts = nullptr;  // first item of each replica, n + 1 entries
   int n_plaq = 0;
-  double* d_plaq_n = nullptr;
-  double* h_plaq_n = nullptr;  // pinned
+  double* h_plaq_n = nullptr;  // page-locked; the kernel writes it
   int threads = 128;
   int blocks_per_sm = 0;  // as given to su3_batch_config; no effect (one block per work item)
   int window = 0;         // replicas per window, 0: all
@@ -301,7 +300,6 @@ void su3_batch_release(su3_batch* b) {
   cudaFree(b->d_status);
   cudaFree(b->d_plaq_items);
   cudaFree(b->d_plaq_starts);
-  cudaFree(b->d_plaq_n);
   cudaFreeHost(b->h_status);
   cudaFreeHost(b->h_plaq_n);
   delete b;
@@ -323,8 +321,10 @@ __global__ void __launch_bounds__(F64 ? kPlaqFxThreads : kPlaqThreads)
     plaq_block<float>(rd.g, (const float4*)links + rd.offset, false, it.y, partials + blockIdx.x);
 }
 __global__ void __launch_bounds__(1024) k_batch_plaquette_final(const ReplicaDesc* reps, const int* starts,
-                                                                const double* partials, double* out) {
+                                                                const double* partials, double* out, const int* status,
+                                                                int* status_host) {
   const int r = blockIdx.x;
+  if (r == 0 && threadIdx.x == 0) *status_host = *status;
   sum_partials(partials + starts[r], starts[r + 1] - starts[r], 1.0 / (3.0 * 6.0 * 2.0 * (double)reps[r].g.Vh), out + r);
 }
 
@@ -582,7 +582,6 @@ int su3_batch_create(int n, const int (*dims)[4], const double* betas, const uin
       (e = cudaMalloc(&b->d_reps, (size_t)n * sizeof(ReplicaDesc))) != cudaSuccess ||
       (e = cudaMalloc(&b->d_sync, (4 + 8 * (size_t)n) * sizeof(unsigned))) != cudaSuccess ||
       (e = cudaMalloc(&b->d_status, sizeof(int))) != cudaSuccess ||
-      (e = cudaMalloc(&b->d_plaq_n, (size_t)n * sizeof(double))) != cudaSuccess ||
       (e = cudaMallocHost(&b->h_status, sizeof(int))) != cudaSuccess ||
       (e = cudaMallocHost(&b->h_plaq_n, (size_t)n * sizeof(double))) != cudaSuccess) {
     const int rc = su3_cuda_fail(e, "su3_batch_create: allocation");
@@ -646,11 +645,10 @@ int su3_batch_plaquettes(su3_handle h, double* out_n) {
   else
     k_batch_plaquette<false><<<b->n_plaq, kPlaqThreads, 0, h->stream>>>(b->d_reps, b->d_plaq_items, h->links, far, h->d_partials);
   SU3_CUDA(cudaGetLastError(), "su3_batch_plaquettes");
-  k_batch_plaquette_final<<<b->n, 1024, 0, h->stream>>>(b->d_reps, b->d_plaq_starts, h->d_partials, b->d_plaq_n);
+  k_batch_plaquette_final<<<b->n, 1024, 0, h->stream>>>(b->d_reps, b->d_plaq_starts, h->d_partials, b->h_plaq_n,
+                                                      b->d_status, b->h_status);
   SU3_CUDA(cudaGetLastError(), "su3_batch_plaquettes");
-  SU3_CUDA(cudaMemcpyAsync(b->h_plaq_n, b->d_plaq_n, (size_t)b->n * sizeof(double), cudaMemcpyDeviceToHost, h->stream),
-           "su3_batch_plaquettes");
-  const int rc = check_status(h, "su3_batch_plaquettes");
+  const int rc = check_copied_status(h, "su3_batch_plaquettes");
   if (rc != SU3_OK) return rc;
   memcpy(out_n, b->h_plaq_n, (size_t)b->n * sizeof(double));
   return SU3_OK;

@@ -376,7 +376,7 @@ int ensure_decomp_graph(su3_lattice* h, bool measured = false) {
       rc = enqueue_phase(h, mu, p, measured && p == 1 && mu >= 1 ? h->d_meas_parts + (size_t)(mu - 1) * blocks : nullptr);
   if (rc == SU3_OK && measured) {
     const cudaError_t e = su3k_launch_meas_final(h->d_meas_parts, 3 * blocks, 1.0 / (6.0 * (double)h->V), h->d_sweep,
-                                                 h->d_meas, h->meas_cap, h->stream);
+                                                 h->h_meas, h->meas_cap, h->stream);
     if (e != cudaSuccess) rc = su3_cuda_fail(e, "plaquette reduction launch");
   }
   if (rc == SU3_OK) {

@@ -31,8 +31,7 @@ struct su3_lattice {
   unsigned long long* d_stats = nullptr;
   bool stats_on = false;
   double* d_partials = nullptr;
-  double* d_plaq = nullptr;
-  double* h_plaq = nullptr;               // pinned
+  double* h_plaq = nullptr;               // page-locked; the kernel writes it (a copy costs 4 us more)
   unsigned long long* h_stats = nullptr;  // pinned, 2 words
   double* d_stage = nullptr;   // canonical-layout staging buffers (two, for the
   double* d_stage2 = nullptr;  // copy/convert pipeline of links_get/set)
@@ -43,8 +42,7 @@ struct su3_lattice {
   cudaGraphExec_t graph_meas = nullptr;           // sweep with the fused plaquette
   double* d_meas_parts = nullptr;  // fused plaquette: block partials of the 3 measuring phases
   int meas_blocks = 0;             // blocks per phase the partials were sized for
-  double* d_meas = nullptr;        // plaquette per sweep, ring of meas_cap entries
-  double* h_meas = nullptr;        // pinned copy
+  double* h_meas = nullptr;        // plaquette per sweep, ring of meas_cap entries, page-locked: the kernel writes it
   int meas_cap = 0;
   int threads = kSu3DefaultThreads;
   bool threads_set = false;  // by the caller (su3_set_block_size): every launch takes `threads`
@@ -96,7 +94,7 @@ int su3_decomp_sweep(su3_lattice* h, int nsweeps);
 int su3_decomp_half_sweep(su3_lattice* h, int mu, int parity);
 // Partials per phase of the decomposed sweep's fused plaquette, and the graph
 // of one measured decomposed sweep (built on first use; it writes the
-// handle's d_meas_parts and d_meas ring).
+// handle's d_meas_parts and h_meas ring).
 int su3_decomp_meas_blocks(su3_lattice* h);
 int su3_decomp_sweep_measured_graph(su3_lattice* h, cudaGraphExec_t* out);
 int su3_decomp_sync_global(su3_lattice* h);   // before reading the global store
