@@ -71,31 +71,31 @@ def peaks():
 # stripped).  A line reports the figure only while that code still hashes the
 # same; otherwise its traffic is null and the line says why.
 _U_F64, _U_F32, _U_BATCH = ("su3_kernels_f64.cu",), ("su3_kernels.cu", "su3_kernels_pair.cu"), ("su3_batch.cu",)
-_SHA_F64 = "885129abed2f07dcf526279300c7e616b6ab6d05d7f194316ac183375be7f880"
-_SHA_F32 = "b69b3efb95b8c7b71cd98f8e15af6aec0aaf08bce33ea207b3a093f079754790"
-_SHA_BATCH = "d9029b824bda46a252b5670089d82c5b7d10b27581aefd95730e21efa98e8ad2"
+_SHA_F64 = "421c9b9264f9a448f02aad59cfa8d8ec77a989a86c13919d60855e554299e33e"
+_SHA_F32 = "0be1cf889a757d08dd8fd6f17162339f48bf1848e1adc616c5e1822dbba4e714"
+_SHA_BATCH = "1c7404eb60c41a3b311221e380604ebf20a4b945b17eaaca301da3ba42eb332a"
 _NCU_METRICS = "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control none"
 NCU_TRAFFIC = {
     # one launch of the default 32^4 FP32 sweep = one chained half-sweep; the mean of the eight launches of
     # the second sweep
-    "fp32_mixed": {"bytes": 208961760 + 12656192, "units": _U_F32, "sources_sha256": _SHA_F32,
+    "fp32_mixed": {"bytes": 209017952 + 13074368, "units": _U_F32, "sources_sha256": _SHA_F32,
                    "capture": _NCU_METRICS + " -k regex:k_half_sweep_f32_chain -s 8 -c 8 python bench.py --profile "
                                              "fp32_mixed"},
-    "fp32_eft": {"bytes": 208966496 + 13336640, "units": _U_F32, "sources_sha256": _SHA_F32,
+    "fp32_eft": {"bytes": 208964224 + 13374976, "units": _U_F32, "sources_sha256": _SHA_F32,
                  "capture": _NCU_METRICS + " -k regex:k_half_sweep_f32_chain -s 8 -c 8 python bench.py --profile "
                                            "fp32_eft"},
-    "fp32_mixed_phases": {"bytes": 207816192 + 15345664, "units": _U_F32, "sources_sha256": _SHA_F32,
+    "fp32_mixed_phases": {"bytes": 207773440 + 15260928, "units": _U_F32, "sources_sha256": _SHA_F32,
                           "capture": _NCU_METRICS + " -k regex:k_half_sweep -s 8 -c 1 python bench.py --profile "
                                                     "fp32_mixed_phases"},
-    "fp32_eft_phases": {"bytes": 207962880 + 15926528, "units": _U_F32, "sources_sha256": _SHA_F32,
+    "fp32_eft_phases": {"bytes": 207864064 + 15980800, "units": _U_F32, "sources_sha256": _SHA_F32,
                         "capture": _NCU_METRICS + " -k regex:k_half_sweep -s 8 -c 1 python bench.py --profile "
                                                   "fp32_eft_phases"},
-    "fp64": {"bytes": 624059904 + 64907520, "units": _U_F64, "sources_sha256": _SHA_F64,
+    "fp64": {"bytes": 626610176 + 70885120, "units": _U_F64, "sources_sha256": _SHA_F64,
              "capture": _NCU_METRICS + " -k regex:k_half_sweep -s 8 -c 1 python bench.py --profile fp64"},
-    "batched": {"bytes": 2830772736 + 442051584, "units": _U_BATCH, "sources_sha256": _SHA_BATCH,
+    "batched": {"bytes": 2834974976 + 442795776, "units": _U_BATCH, "sources_sha256": _SHA_BATCH,
                 "capture": _NCU_METRICS + " -k regex:k_batch_sweep -s 4 -c 4 python bench.py --profile batched "
                                           "(the four launches of the second sweep, summed)"},
-    "batched_eft": {"bytes": 2829066240 + 442415616, "units": _U_BATCH, "sources_sha256": _SHA_BATCH,
+    "batched_eft": {"bytes": 2828132608 + 442020352, "units": _U_BATCH, "sources_sha256": _SHA_BATCH,
                     "capture": _NCU_METRICS + " -k regex:k_batch_sweep -s 4 -c 4 python bench.py --profile batched_eft "
                                               "(the four launches of the second sweep, summed)"},
 }
