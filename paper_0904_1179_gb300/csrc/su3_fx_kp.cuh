@@ -207,14 +207,17 @@ SU3_HD bool fx_direction(const long long rI[4], fx v[4], double* ik) {
 #pragma unroll
   for (int c = 0; c < 4; ++c) fx_mac(a, x[c], x[c]);
   long long k60 = fx_merge(a);  // [1/16, 1)
-  const bool small = k60 < (1LL << 58) + (1LL << 48);
-  if (small) {
-    k60 *= 4;
-    ++n;
+  // |x| doubled where it is below 1/2, and twice where it is next to 1/4 (a power of
+  // two along one axis): 1/|x| stays below 2, the end of a real of unit 2^-30
+  if (k60 < (1LL << 58) + (1LL << 48)) {
+    const int e = k60 < (1LL << 56) + (1LL << 36) ? 2 : 1;
+    k60 <<= 2 * e;
+    n += e;
+    const float f = e == 2 ? 4.0f : 2.0f;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) x[c] = fx{2 * x[c].h, 2.0f * x[c].l, 2.0f * x[c].f};
+    for (int c = 0; c < 4; ++c) x[c] = fx{x[c].h * (1 << e), f * x[c].l, f * x[c].f};
   }
-  const fx k = fx_from_i62(4 * k60);  // (1/4, 1 + 2^-9)
+  const fx k = fx_from_i62(4 * k60);  // (1/4 + 2^-22, 1 + 2^-9)
   const float g2 = fx_rsqrt_approx(fx_mul(k.f, 0x1p-30f));
   const fx g = fx_make(fx_f2i(fx_mul(g2, 0x1p29f)), 0.0f);
   const fx w = fx_mulv(k, g);
@@ -223,7 +226,7 @@ SU3_HD bool fx_direction(const long long rI[4], fx v[4], double* ik) {
   const fx z = fx_root_series(4 * fx_merge(e));
   facc s{0, 0.0f};
   fx_mac(s, g, z);
-  const long long y62 = 2 * (((long long)g.h << 32) + 4 * fx_merge(s));  // 1/|x|, (0.998, 1.9996)
+  const long long y62 = 2 * (((long long)g.h << 32) + 4 * fx_merge(s));  // 1/|x|, (0.998, 2 - 2^-21)
   const fx y = fx_from_i62(y62);
 #pragma unroll
   for (int c = 0; c < 4; ++c) v[c] = fx_mulv(x[c], y);
