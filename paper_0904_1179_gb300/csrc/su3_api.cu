@@ -373,7 +373,7 @@ int enqueue_sweep_body(su3_lattice* h, bool measured) {
     SU3_CUDA(su3k_launch_meas_final(h->d_meas_parts, 3 * blocks, 1.0 / (6.0 * (double)h->V), h->d_sweep, h->h_meas,
                                     h->meas_cap, h->stream),
              "plaquette reduction launch");
-  SU3_CUDA(su3k_launch_increment(h->d_sweep, 1, h->stream), "sweep counter launch");
+  SU3_CUDA(su3k_launch_increment(h->d_sweep, 1, su3dev::sweep_far(h->d_sweep), 1, h->stream), "sweep counter launch");
   return SU3_OK;
 }
 
@@ -454,14 +454,14 @@ static double* host_direct(double* host, size_t bytes) {
   return (first | last) & cudaHostRegisterReadOnly ? nullptr : (double*)d;
 }
 
-int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pairs, double* host, bool get,
+int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pairs, int* far, double* host, bool get,
                  const char* what, const int* status, int* status_host) {
   const long long V = 2LL * g.Vh;
   // Page-locked memory: the conversion writes the caller's buffer itself, one launch of any size.  GB300, get through
   // the staging buffer / directly: 4^4 18 / 14 us, 8^4 30 / 26 us (FP32 38 / 28), 16^4 222 / 210 us (FP32 246 / 215),
   // 32^4 3.18 / 3.14 ms, 48^4 15.98 / 15.82 ms (the host link's 193 GB/s: 3.13 and 15.8 ms).
   if (double* direct = get ? host_direct(host, (size_t)V * 72 * sizeof(double)) : nullptr) {
-    ConvArgs a{g, h->precision, 0, V, direct, links, pairs ? 1 : 0, su3dev::sweep_far(h->d_sweep)};
+    ConvArgs a{g, h->precision, 0, V, direct, links, pairs ? 1 : 0, far};
     a.status = status;
     a.status_host = status_host;
     SU3_CUDA(su3k_launch_conv(a, false, h->stream), what);
@@ -472,14 +472,13 @@ int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pa
   if (V <= kChunkSites) {
     // one chunk has nothing to overlap: conversion and copy follow each other on
     // the handle's stream, without the events and the second wait (one 8^4 replica of a batch: 52.6 -> 40.0 us)
-    ConvArgs a{g, h->precision, 0, V, h->d_stage, links, pairs ? 1 : 0, su3dev::sweep_far(h->d_sweep)};
+    ConvArgs a{g, h->precision, 0, V, h->d_stage, links, pairs ? 1 : 0, far};
     const size_t bytes = (size_t)V * 72 * sizeof(double);
     if (get) {
       SU3_CUDA(su3k_launch_conv(a, false, h->stream), what);
       SU3_CUDA(cudaMemcpyAsync(host, h->d_stage, bytes, cudaMemcpyDeviceToHost, h->stream), what);
     } else {
-      if (!h->batch)
-        SU3_CUDA(cudaMemsetAsync(su3dev::sweep_far(h->d_sweep), 0, 2 * sizeof(int), h->stream), what);
+      if (far) SU3_CUDA(cudaMemsetAsync(far, 0, 2 * sizeof(int), h->stream), what);
       SU3_CUDA(cudaMemcpyAsync(h->d_stage, host, bytes, cudaMemcpyHostToDevice, h->stream), what);
       SU3_CUDA(su3k_launch_conv(a, true, h->stream), what);
     }
@@ -488,16 +487,15 @@ int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pa
   int rc = ensure_transfer(h, what);
   if (rc != SU3_OK) return rc;
   double* stage[2] = {h->d_stage, h->d_stage2};
-  // the conversion into the store flags links far from SU(3); a batch's other replicas keep theirs
-  if (!get && !h->batch)
-    SU3_CUDA(cudaMemsetAsync(su3dev::sweep_far(h->d_sweep), 0, 2 * sizeof(int), h->stream), what);
+  // the conversion into the store flags links far from SU(3)
+  if (!get && far) SU3_CUDA(cudaMemsetAsync(far, 0, 2 * sizeof(int), h->stream), what);
   int i = 0;
   for (long long s0 = 0; s0 < V; s0 += kChunkSites, ++i) {
     const long long n = (V - s0) < kChunkSites ? (V - s0) : kChunkSites;
     const int b = i & 1;
     cudaStream_t cs = h->copy_stream;
     const size_t bytes = (size_t)n * 72 * sizeof(double);
-    ConvArgs a{g, h->precision, s0, n, stage[b], links, pairs ? 1 : 0, su3dev::sweep_far(h->d_sweep)};
+    ConvArgs a{g, h->precision, s0, n, stage[b], links, pairs ? 1 : 0, far};
     if (get) {
       // stage[b] is free once the copy-out of chunk i-2 has finished
       if (i >= 2) SU3_CUDA(cudaStreamWaitEvent(h->stream, h->ev_copied[b], 0), what);
@@ -709,14 +707,15 @@ int su3_links_get(su3_handle h, double* host, size_t n_doubles) {
   if (n_doubles != (size_t)h->V * 72) return fail(SU3_ESIZE, "su3_links_get: n = %zu, expected %lld", n_doubles, h->V * 72);
   const int rc = su3_decomp_sync_global(h);
   if (rc != SU3_OK) return rc;
-  return su3_transfer(h, h->geom, h->links, h->pairs, host, true, "su3_links_get");
+  return su3_transfer(h, h->geom, h->links, h->pairs, su3dev::sweep_far(h->d_sweep), host, true, "su3_links_get");
 }
 
 int su3_links_set(su3_handle h, const double* host, size_t n_doubles) {
   if (!h || !host) return fail(SU3_EINVAL, "su3_links_set: NULL argument");
   if (is_batch(h)) return fail(SU3_EINVAL, "su3_links_set: batch handle (use the su3_batch_* calls)");
   if (n_doubles != (size_t)h->V * 72) return fail(SU3_ESIZE, "su3_links_set: n = %zu, expected %lld", n_doubles, h->V * 72);
-  const int rc = su3_transfer(h, h->geom, h->links, h->pairs, const_cast<double*>(host), false, "su3_links_set");
+  const int rc = su3_transfer(h, h->geom, h->links, h->pairs, su3dev::sweep_far(h->d_sweep),
+                              const_cast<double*>(host), false, "su3_links_set");
   if (rc == SU3_OK) su3_decomp_global_written(h);
   return rc;
 }

@@ -69,6 +69,7 @@ struct BatchArgs {
   unsigned int* done;    // [replica * 8 + phase]: tiles completed in this sweep
   int* status;           // 0 or kStatusTimeout
   const uint64_t* sweep;
+  int* far;  // FP64: [2 r], [2 r + 1] the flags of replica r (far and far_next of SweepState)
   void* links;
   long long wait_ns;
   int withhold_item;  // fault-injection hook: this item never signals completion (-1: none)
@@ -163,7 +164,7 @@ __device__ __forceinline__ void batch_item(const BatchArgs& a, const ReplicaDesc
   if (s_stop) return;
   const ReplicaDesc& rd = PARAM ? reps[it.x] : s_rep;
   const int h = it.z * (int)blockDim.x + (int)threadIdx.x;
-  if (h < rd.g.Vh) update_item<T, EFT, REPEAT, MU>(rd, a.links, h, it.y & 1, a.mu, t, a.max_tries, sweep_far(a.sweep));
+  if (h < rd.g.Vh) update_item<T, EFT, REPEAT, MU>(rd, a.links, h, it.y & 1, a.mu, t, a.max_tries, a.far + 2 * it.x);
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -268,6 +269,7 @@ struct su3_batch {
   int4* d_schedule = nullptr;  // the work items of directions 0..3, one after another
   int n_items_mu[4] = {0, 0, 0, 0};
   unsigned* d_sync = nullptr;  // [mu] queue of direction mu's launch, [4 + 8r + k] arrival counters
+  int* d_far = nullptr;  // flags of each replica (BatchArgs::far): one far from SU(3) slows no other
   int* d_status = nullptr;
   int* h_status = nullptr;  // pinned
   int2* d_plaq_items = nullptr;  // k_batch_plaquette: (replica, block)
@@ -297,6 +299,7 @@ void su3_batch_release(su3_batch* b) {
   cudaFree(b->d_reps);
   cudaFree(b->d_schedule);
   cudaFree(b->d_sync);
+  cudaFree(b->d_far);
   cudaFree(b->d_status);
   cudaFree(b->d_plaq_items);
   cudaFree(b->d_plaq_starts);
@@ -316,7 +319,7 @@ __global__ void __launch_bounds__(F64 ? kPlaqFxThreads : kPlaqThreads)
   const int2 it = items[blockIdx.x];
   const ReplicaDesc& rd = reps[it.x];
   if constexpr (F64)
-    plaq_block_fx(rd.g, (const double2*)links + rd.offset, far, it.y, partials + blockIdx.x);
+    plaq_block_fx(rd.g, (const double2*)links + rd.offset, far + 2 * it.x, it.y, partials + blockIdx.x);
   else
     plaq_block<float>(rd.g, (const float4*)links + rd.offset, false, it.y, partials + blockIdx.x);
 }
@@ -408,6 +411,7 @@ int enqueue_batch_sweep(su3_lattice* h) {
     a[mu].done = b->d_sync + 4;
     a[mu].status = b->d_status;
     a[mu].sweep = h->d_sweep;
+    a[mu].far = b->d_far;
     a[mu].links = h->links;
     a[mu].wait_ns = b->wait_ns;
     a[mu].withhold_item = b->withhold_item;
@@ -415,7 +419,8 @@ int enqueue_batch_sweep(su3_lattice* h) {
     first += b->n_items_mu[mu];
   }
   SU3_CUDA(launch_batch(a, b->param_reps.get(), h->precision, b->threads, h->stream), "batch sweep launch");
-  SU3_CUDA(su3k_launch_increment(h->d_sweep, 1, h->stream), "sweep counter launch");
+  SU3_CUDA(su3k_launch_increment(h->d_sweep, 1, b->d_far, h->precision == SU3_FP64 ? b->n : 0, h->stream),
+           "sweep counter launch");
   return SU3_OK;
 }
 
@@ -464,7 +469,7 @@ int check_copied_status(su3_lattice* h, const char* what) {
   if (*b->h_status != 0) {
     SU3_CUDA(cudaMemset(b->d_status, 0, sizeof(int)), what);
     // links that the sweep did not reach keep whatever they held
-    SU3_CUDA(cudaMemset(sweep_far(h->d_sweep), 1, sizeof(int)), what);
+    SU3_CUDA(cudaMemset2DAsync(b->d_far, 2 * sizeof(int), 1, sizeof(int), b->n, h->stream), what);
     return su3_fail(SU3_ETIMEOUT,
                     "%s: a batched sweep gave up waiting for a phase to complete (bounded wait of %.3f s); the "
                     "configuration of that sweep is incomplete",
@@ -581,6 +586,7 @@ int su3_batch_create(int n, const int (*dims)[4], const double* betas, const uin
       (e = cudaMalloc(&h->d_stage, (size_t)chunk * 72 * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&b->d_reps, (size_t)n * sizeof(ReplicaDesc))) != cudaSuccess ||
       (e = cudaMalloc(&b->d_sync, (4 + 8 * (size_t)n) * sizeof(unsigned))) != cudaSuccess ||
+      (e = cudaMalloc(&b->d_far, (size_t)n * 2 * sizeof(int))) != cudaSuccess ||
       (e = cudaMalloc(&b->d_status, sizeof(int))) != cudaSuccess ||
       (e = cudaMallocHost(&b->h_status, sizeof(int))) != cudaSuccess ||
       (e = cudaMallocHost(&b->h_plaq_n, (size_t)n * sizeof(double))) != cudaSuccess) {
@@ -591,6 +597,7 @@ int su3_batch_create(int n, const int (*dims)[4], const double* betas, const uin
   }
   int rc = SU3_OK;
   if ((e = cudaMemsetAsync(h->d_sweep, 0, sizeof(SweepState), h->stream)) != cudaSuccess ||
+      (e = cudaMemsetAsync(b->d_far, 0, (size_t)n * 2 * sizeof(int), h->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(b->d_status, 0, sizeof(int), h->stream)) != cudaSuccess)
     rc = su3_cuda_fail(e, "su3_batch_create: memset");
   for (int r = 0; r < n && rc == SU3_OK; ++r) {
@@ -639,7 +646,7 @@ int su3_batch_sweep(su3_handle h, int nsweeps) {
 int su3_batch_plaquettes(su3_handle h, double* out_n) {
   su3_batch* b = batch_of(h);
   if (!b || !out_n) return fail(SU3_EINVAL, "su3_batch_plaquettes: not a batch handle or NULL output");
-  const int* far = sweep_far(h->d_sweep);
+  const int* far = b->d_far;
   if (h->precision == SU3_FP64)
     k_batch_plaquette<true><<<b->n_plaq, kPlaqFxThreads, 0, h->stream>>>(b->d_reps, b->d_plaq_items, h->links, far, h->d_partials);
   else
@@ -663,7 +670,8 @@ static int batch_links(su3_handle h, int replica, double* host, size_t n_doubles
   const long long V = 2LL * g.Vh;
   if (n_doubles != (size_t)V * 72) return su3_fail(SU3_ESIZE, "%s: n = %zu, expected %lld", what, n_doubles, V * 72);
   void* base = (char*)h->links + b->offsets[replica] * b->elem_bytes;
-  const int rc = su3_transfer(h, g, base, false, host, get, what, b->d_status, b->h_status);
+  int* far = h->precision == SU3_FP64 ? b->d_far + 2 * replica : nullptr;
+  const int rc = su3_transfer(h, g, base, false, far, host, get, what, b->d_status, b->h_status);
   if (rc != SU3_OK) return rc;
   return check_copied_status(h, what);
 }
@@ -700,8 +708,9 @@ int su3_batch_autotune(su3_handle h, int* threads, int* blocks_per_sm, int* wind
   SU3_CUDA(cudaMalloc(&saved, h->link_bytes), "su3_batch_autotune: save buffer");
   cudaError_t e = cudaMemcpyAsync(saved, h->links, h->link_bytes, cudaMemcpyDeviceToDevice, h->stream);
   const uint64_t count = h->sweep_host;
-  int far[2] = {0, 0};
-  if (e == cudaSuccess) e = cudaMemcpyAsync(far, sweep_far(h->d_sweep), sizeof far, cudaMemcpyDeviceToHost, h->stream);
+  std::vector<int> far(2 * (size_t)b->n);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(far.data(), b->d_far, far.size() * sizeof(int), cudaMemcpyDeviceToHost, h->stream);
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
@@ -750,7 +759,8 @@ int su3_batch_autotune(su3_handle h, int* threads, int* blocks_per_sm, int* wind
   if (rc == SU3_OK) {
     e = cudaMemcpyAsync(h->links, saved, h->link_bytes, cudaMemcpyDeviceToDevice, h->stream);
     if (e == cudaSuccess) e = su3k_launch_set_counter(h->d_sweep, count, h->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sweep_far(h->d_sweep), far, sizeof far, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(b->d_far, far.data(), far.size() * sizeof(int), cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) rc = su3_cuda_fail(e, "su3_batch_autotune: restore");
     h->sweep_host = count;

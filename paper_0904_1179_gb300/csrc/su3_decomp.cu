@@ -380,7 +380,7 @@ int ensure_decomp_graph(su3_lattice* h, bool measured = false) {
     if (e != cudaSuccess) rc = su3_cuda_fail(e, "plaquette reduction launch");
   }
   if (rc == SU3_OK) {
-    const cudaError_t e = su3k_launch_increment(h->d_sweep, 1, h->stream);
+    const cudaError_t e = su3k_launch_increment(h->d_sweep, 1, sweep_far(h->d_sweep), 1, h->stream);
     if (e != cudaSuccess) rc = su3_cuda_fail(e, "sweep counter launch");
   }
   const cudaError_t e = cudaStreamEndCapture(h->stream, &graph);

@@ -690,6 +690,7 @@ __device__ __forceinline__ void gram_schmidt_rows01(cx<double> r0[3], cx<double>
 // whose range and reunitarisation assume near-unitary links.  far_next: an
 // FP64 update of this sweep left such a link.  Every link has been rewritten
 // by the end of a sweep, so the counter's increment moves far_next to far.
+// (The replicas of a batch have a pair of flags each, in an array of their own.)
 struct SweepState {
   uint64_t t;
   int far, far_next;

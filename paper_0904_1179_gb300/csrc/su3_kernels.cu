@@ -133,11 +133,13 @@ __global__ void __launch_bounds__(SU3_F32_LB_THREADS, SU3_F32_MINBLOCKS) k_half_
   if (MEAS) block_partial(m, args.meas);
 }
 
-__global__ void k_increment(uint64_t* counter, uint64_t n) {
-  *counter += n;
-  int* far = sweep_far(counter);
-  far[0] = far[1];
-  far[1] = 0;
+// far: nfar pairs of flags (far and far_next of SweepState).
+__global__ void k_increment(uint64_t* counter, uint64_t n, int* far, int nfar) {
+  if (threadIdx.x == 0) *counter += n;
+  for (int i = threadIdx.x; i < nfar; i += blockDim.x) {
+    far[2 * i] = far[2 * i + 1];
+    far[2 * i + 1] = 0;
+  }
 }
 
 __global__ void __launch_bounds__(1024) k_meas_final(const double* parts, int n, double scale, const uint64_t* sweep,
@@ -416,8 +418,8 @@ int su3k_half_sweep_blocks(const HalfSweepArgs& a, int precision, int threads) {
   return (n + threads - 1) / threads;
 }
 
-cudaError_t su3k_launch_increment(uint64_t* counter, uint64_t n, cudaStream_t s) {
-  k_increment<<<1, 1, 0, s>>>(counter, n);
+cudaError_t su3k_launch_increment(uint64_t* counter, uint64_t n, int* far, int nfar, cudaStream_t s) {
+  k_increment<<<1, nfar > 1 ? 128 : 1, 0, s>>>(counter, n, far, nfar);
   return cudaGetLastError();
 }
 

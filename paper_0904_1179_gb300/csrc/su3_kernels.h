@@ -132,7 +132,7 @@ cudaError_t su3k_bounds_status_f64(unsigned int* v, bool clear);
 cudaError_t su3k_bounds_status_pair(unsigned int* v, bool clear);
 cudaError_t su3k_bounds_status_batch(unsigned int* v, bool clear);
 cudaError_t su3k_bounds_status_decomp(unsigned int* v, bool clear);
-cudaError_t su3k_launch_increment(uint64_t* counter, uint64_t n, cudaStream_t s);
+cudaError_t su3k_launch_increment(uint64_t* counter, uint64_t n, int* far, int nfar, cudaStream_t s);
 // Sum the nparts fused-plaquette partials of one sweep (fixed order) into
 // out[*sweep % cap] * scale.
 cudaError_t su3k_launch_meas_final(const double* parts, int nparts, double scale, const uint64_t* sweep, double* out,

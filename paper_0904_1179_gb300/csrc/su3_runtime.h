@@ -75,7 +75,9 @@ int su3_sync(su3_lattice* h, const char* what);
 // second stream overlap the layout conversions on the handle's stream (one
 // chunk: on that stream alone).  Synchronises, except for batches: their caller
 // does, reading their status word, which is copied to status_host, with it.
-int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pairs, double* host, bool get,
+// far: the flags of this configuration (far and far_next of SweepState), which a
+// configuration that comes in sets anew; null: an FP32 store of a batch.
+int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pairs, int* far, double* host, bool get,
                  const char* what, const int* status = nullptr, int* status_host = nullptr);
 // Lanes per link of an FP64 half-sweep of this lattice (1, 4 or 8).
 int su3_f64_lanes(const su3_lattice* h);

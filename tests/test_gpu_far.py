@@ -1,0 +1,51 @@
+"""FP64 configurations with a link far from SU(3), which take the update in FP64 arithmetic: what that is limited to,
+and every kernel that holds it."""
+import contextlib
+
+import numpy as np
+import pytest
+
+import oracle
+import paper_0904_1179_gb300 as su3
+
+pytestmark = pytest.mark.gpu
+
+MIX = [(4, 4, 4, 4), (6, 4, 10, 8), (8, 8, 8, 8)]
+BETAS = [5.7, 5.5, 6.0]
+SEEDS = [11, 12, 13]
+
+
+def with_far_link(L, seed, kind):
+    u = oracle.hot_start(L, seed)
+    if kind == "nan":
+        u[0, 1, 1, 0, 2] = np.nan
+    else:
+        u[0, 1, 1, 0, 2] *= 1.5
+    return u
+
+
+@pytest.mark.parametrize("kind", ["stretched", "nan"])
+@pytest.mark.parametrize("tries", [1, 4])
+def test_replicas_of_a_batch_are_independent(kind, tries):
+    # The far link of one replica changes no bit of another, which equals the lattice alone; its own replica equals
+    # its lattice too.  A proper configuration, or a sweep, brings the replica back.
+    far = with_far_link(MIX[1], 7, kind)
+    with su3.Batch(MIX, BETAS, SEEDS, start=su3.SU3_HOT, precision=su3.SU3_FP64) as b, contextlib.ExitStack() as stack:
+        alone = [stack.enter_context(su3.Lattice(L, BETAS[r], SEEDS[r], start=su3.SU3_HOT)) for r, L in enumerate(MIX)]
+        b.set_heatbath(tries)
+        for lat in alone:
+            lat.set_heatbath(tries)
+        b.set_links(1, far)
+        alone[1].set_links(far)
+        for step in range(3):
+            if step == 2:
+                proper = oracle.hot_start(MIX[1], 8)
+                b.set_links(1, proper)
+                alone[1].set_links(proper)
+            plaq = b.plaquettes()
+            for r, lat in enumerate(alone):
+                assert np.array_equal(b.get_links(r), lat.get_links(), equal_nan=True), (step, r)
+                assert np.array_equal(plaq[r], su3.load_library().su3_plaquette(lat.handle), equal_nan=True), (step, r)
+            b.sweep(1)
+            for lat in alone:
+                lat.sweep(1)
