@@ -39,9 +39,10 @@ int su3_sync(su3_lattice* h, const char* what) {
   SU3_CUDA(cudaGetLastError(), what);
   if (h->d_pstatus) {
     if (*h->h_pstatus != 0) {
-      SU3_CUDA(cudaMemset(h->d_pstatus, 0, sizeof(int)), what);
+      // (on the handle's stream: the next sweep reads both words)
+      SU3_CUDA(cudaMemsetAsync(h->d_pstatus, 0, sizeof(int), h->stream), what);
       // links that the sweep did not reach keep whatever they held
-      SU3_CUDA(cudaMemset(su3dev::sweep_far(h->d_sweep), 1, sizeof(int)), what);
+      SU3_CUDA(cudaMemsetAsync(su3dev::sweep_far(h->d_sweep), 1, sizeof(int), h->stream), what);
       return su3_fail(SU3_ETIMEOUT,
                       "%s: a sweep gave up waiting for tiles of the previous half-sweep (bounded wait of %.3f s); "
                       "the configuration is incomplete",

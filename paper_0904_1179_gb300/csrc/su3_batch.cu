@@ -379,9 +379,12 @@ int build_schedule(su3_lattice* h) {
   cudaFree(b->d_schedule);
   b->d_schedule = nullptr;
   SU3_CUDA(cudaMalloc(&b->d_schedule, items.size() * sizeof(int4)), "batch schedule");
-  SU3_CUDA(cudaMemcpy(b->d_schedule, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice), "batch schedule");
-  SU3_CUDA(cudaMemcpy(b->d_reps, reps.data(), reps.size() * sizeof(ReplicaDesc), cudaMemcpyHostToDevice),
+  // (on the stream whose kernels read them; waited for while the vectors live)
+  SU3_CUDA(cudaMemcpyAsync(b->d_schedule, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream),
+           "batch schedule");
+  SU3_CUDA(cudaMemcpyAsync(b->d_reps, reps.data(), reps.size() * sizeof(ReplicaDesc), cudaMemcpyHostToDevice, h->stream),
            "batch descriptors");
+  SU3_CUDA(cudaStreamSynchronize(h->stream), "batch schedule");
   if (b->n <= kParamReplicas) {
     if (!b->param_reps) b->param_reps.reset(new (std::nothrow) ParamReplicas());
     if (!b->param_reps) return fail(SU3_ENOMEM, "batch descriptors: host allocation failed");
@@ -467,7 +470,8 @@ int check_copied_status(su3_lattice* h, const char* what) {
   const int rc = su3_sync(h, what);
   if (rc != SU3_OK) return rc;
   if (*b->h_status != 0) {
-    SU3_CUDA(cudaMemset(b->d_status, 0, sizeof(int)), what);
+    // (on the handle's stream: the next sweep reads these words)
+    SU3_CUDA(cudaMemsetAsync(b->d_status, 0, sizeof(int), h->stream), what);
     // links that the sweep did not reach keep whatever they held
     SU3_CUDA(cudaMemset2DAsync(b->d_far, 2 * sizeof(int), 1, sizeof(int), b->n, h->stream), what);
     return su3_fail(SU3_ETIMEOUT,
@@ -581,8 +585,10 @@ int su3_batch_create(int n, const int (*dims)[4], const double* betas, const uin
       (e = cudaMalloc(&h->d_partials, items.size() * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&b->d_plaq_items, items.size() * sizeof(int2))) != cudaSuccess ||
       (e = cudaMalloc(&b->d_plaq_starts, starts.size() * sizeof(int))) != cudaSuccess ||
-      (e = cudaMemcpy(b->d_plaq_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice)) != cudaSuccess ||
-      (e = cudaMemcpy(b->d_plaq_starts, starts.data(), starts.size() * sizeof(int), cudaMemcpyHostToDevice)) != cudaSuccess ||
+      (e = cudaMemcpyAsync(b->d_plaq_items, items.data(), items.size() * sizeof(int2), cudaMemcpyHostToDevice, h->stream)) !=
+          cudaSuccess ||
+      (e = cudaMemcpyAsync(b->d_plaq_starts, starts.data(), starts.size() * sizeof(int), cudaMemcpyHostToDevice,
+                           h->stream)) != cudaSuccess ||
       (e = cudaMalloc(&h->d_stage, (size_t)chunk * 72 * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&b->d_reps, (size_t)n * sizeof(ReplicaDesc))) != cudaSuccess ||
       (e = cudaMalloc(&b->d_sync, (4 + 8 * (size_t)n) * sizeof(unsigned))) != cudaSuccess ||

@@ -621,8 +621,9 @@ int su3_decomp_create(int L0, int L1, int L2, int L3, double beta, uint64_t seed
     if (d->nghost[p] == 0) continue;
     e = cudaMalloc(&d->d_ghost[p], lists[p].size() * sizeof(int4));
     if (e == cudaSuccess)
-      e = cudaMemcpy(d->d_ghost[p], lists[p].data(), lists[p].size() * sizeof(int4), cudaMemcpyHostToDevice);
+      e = cudaMemcpyAsync(d->d_ghost[p], lists[p].data(), lists[p].size() * sizeof(int4), cudaMemcpyHostToDevice, h->stream);
   }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);  // the lists end with this call
   if (e != cudaSuccess) {
     rc = su3_cuda_fail(e, "su3_decomp_create: allocation");
     cudaGetLastError();
