@@ -42,6 +42,8 @@ int su3_sync(su3_lattice* h, const char* what) {
       // (on the handle's stream: the next sweep reads both words)
       SU3_CUDA(cudaMemsetAsync(h->d_pstatus, 0, sizeof(int), h->stream), what);
       // links that the sweep did not reach keep whatever they held
+      h->far_possible = h->precision == SU3_FP64;
+      h->half_sweeps = 0;
       SU3_CUDA(cudaMemsetAsync(su3dev::sweep_far(h->d_sweep), 1, sizeof(int), h->stream), what);
       return su3_fail(SU3_ETIMEOUT,
                       "%s: a sweep gave up waiting for tiles of the previous half-sweep (bounded wait of %.3f s); "
@@ -171,6 +173,7 @@ void release(su3_lattice* h) {
   if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
   cudaFreeHost(h->h_plaq);
   cudaFreeHost(h->h_stats);
+  cudaFreeHost(h->h_far);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }
@@ -408,6 +411,19 @@ int sync(su3_lattice* h, const char* what) { return su3_sync(h, what); }
 // Single-lattice calls reject batch handles and vice versa.
 bool is_batch(const su3_lattice* h) { return h && h->batch; }
 
+// After a half-sweep called by itself: once all eight have run since the flags were
+// last set or moved (links_set, a timeout, a sweep, this function), every link has been rewritten and the flags move
+// on as at the end of a sweep (nothing else would end the FP64 arithmetic of a chain
+// driven by half-sweeps).
+int note_half_sweep(su3_lattice* h, int mu, int parity) {
+  if (!h->far_possible) return SU3_OK;
+  h->half_sweeps |= 1u << (2 * mu + parity);
+  if (h->half_sweeps != 0xffu) return SU3_OK;
+  h->half_sweeps = 0;
+  SU3_CUDA(su3k_launch_increment(h->d_sweep, 0, su3dev::sweep_far(h->d_sweep), 1, h->stream), "su3_half_sweep");
+  return SU3_OK;
+}
+
 }  // namespace
 
 void su3_release_handle(su3_lattice* h) { release(h); }
@@ -474,6 +490,7 @@ int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pa
     // one chunk has nothing to overlap: conversion and copy follow each other on
     // the handle's stream, without the events and the second wait (one 8^4 replica of a batch: 52.6 -> 40.0 us)
     ConvArgs a{g, h->precision, 0, V, h->d_stage, links, pairs ? 1 : 0, far};
+    a.far_host = h->h_far;
     const size_t bytes = (size_t)V * 72 * sizeof(double);
     if (get) {
       SU3_CUDA(su3k_launch_conv(a, false, h->stream), what);
@@ -497,6 +514,7 @@ int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pa
     cudaStream_t cs = h->copy_stream;
     const size_t bytes = (size_t)n * 72 * sizeof(double);
     ConvArgs a{g, h->precision, s0, n, stage[b], links, pairs ? 1 : 0, far};
+    a.far_host = h->h_far;
     if (get) {
       // stage[b] is free once the copy-out of chunk i-2 has finished
       if (i >= 2) SU3_CUDA(cudaStreamWaitEvent(h->stream, h->ev_copied[b], 0), what);
@@ -584,7 +602,8 @@ int su3_create_ex(int L0, int L1, int L2, int L3, double beta, uint64_t seed, in
       (e = cudaMalloc(&h->d_partials, (size_t)nparts * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_stage, (size_t)chunk * 4 * 18 * sizeof(double))) != cudaSuccess ||
       (e = cudaMallocHost(&h->h_plaq, sizeof(double))) != cudaSuccess ||
-      (e = cudaMallocHost(&h->h_stats, 2 * sizeof(unsigned long long))) != cudaSuccess) {
+      (e = cudaMallocHost(&h->h_stats, 2 * sizeof(unsigned long long))) != cudaSuccess ||
+      (e = cudaMallocHost(&h->h_far, sizeof(int))) != cudaSuccess) {
     const int rc = cuda_fail(e, "su3_create: allocation");
     cudaGetLastError();
     release(h);
@@ -623,6 +642,7 @@ int su3_sweep(su3_handle h, int nsweeps) {
   if (is_batch(h)) return fail(SU3_EINVAL, "su3_sweep: batch handle (use the su3_batch_* calls)");
   if (nsweeps < 0) return fail(SU3_EINVAL, "su3_sweep: nsweeps < 0");
   if (nsweeps == 0) return SU3_OK;
+  h->half_sweeps = 0;  // the sweep moves the flags itself
   if (su3_decomp_active(h)) return su3_decomp_sweep(h, nsweeps);
   int rc = ensure_graph(h);
   if (rc != SU3_OK) return rc;
@@ -638,6 +658,7 @@ int su3_sweep_measured(su3_handle h, int nsweeps, double* plaq_out) {
   if (nsweeps < 0 || (nsweeps > 0 && !plaq_out)) return fail(SU3_EINVAL, "su3_sweep_measured: bad nsweeps or NULL out");
   if (h->stats_on) return fail(SU3_EINVAL, "su3_sweep_measured: disable acceptance statistics first");
   if (nsweeps == 0) return SU3_OK;
+  h->half_sweeps = 0;
   const bool dec = su3_decomp_active(h);
   const int blocks = dec ? su3_decomp_meas_blocks(h) : su3k_half_sweep_blocks(half_sweep_args(h, 1, h->threads), h->precision, h->threads);
   if (h->meas_blocks != blocks || !h->h_meas) {
@@ -677,11 +698,14 @@ int su3_half_sweep(su3_handle h, int mu, int parity) {
   if (!h) return fail(SU3_EINVAL, "su3_half_sweep: NULL handle");
   if (is_batch(h)) return fail(SU3_EINVAL, "su3_half_sweep: batch handle (use the su3_batch_* calls)");
   if (mu < 0 || mu > 3 || parity < 0 || parity > 1) return fail(SU3_EINVAL, "su3_half_sweep: bad mu/parity");
-  if (su3_decomp_active(h)) return su3_decomp_half_sweep(h, mu, parity);
+  if (su3_decomp_active(h)) {
+    const int rc = su3_decomp_half_sweep(h, mu, parity);
+    return rc == SU3_OK ? note_half_sweep(h, mu, parity) : rc;
+  }
   const int threads = launch_threads(h);
   SU3_CUDA(su3k_launch_half_sweep(half_sweep_args(h, parity, threads), mu, h->precision, h->stats_on, threads, h->stream),
            "su3_half_sweep");
-  return SU3_OK;
+  return note_half_sweep(h, mu, parity);
 }
 
 double su3_plaquette(su3_handle h) {
@@ -715,8 +739,11 @@ int su3_links_set(su3_handle h, const double* host, size_t n_doubles) {
   if (!h || !host) return fail(SU3_EINVAL, "su3_links_set: NULL argument");
   if (is_batch(h)) return fail(SU3_EINVAL, "su3_links_set: batch handle (use the su3_batch_* calls)");
   if (n_doubles != (size_t)h->V * 72) return fail(SU3_ESIZE, "su3_links_set: n = %zu, expected %lld", n_doubles, h->V * 72);
+  *h->h_far = 0;  // (only the conversion below writes it)
   const int rc = su3_transfer(h, h->geom, h->links, h->pairs, su3dev::sweep_far(h->d_sweep),
                               const_cast<double*>(host), false, "su3_links_set");
+  h->far_possible = *h->h_far != 0 || (rc != SU3_OK && h->precision == SU3_FP64);
+  h->half_sweeps = 0;
   if (rc == SU3_OK) su3_decomp_global_written(h);
   return rc;
 }

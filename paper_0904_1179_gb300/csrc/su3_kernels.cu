@@ -269,7 +269,10 @@ __global__ void k_canon_to_store(ConvArgs args) {
     mat3<double> m;
 #pragma unroll
     for (int c = 0; c < 9; ++c) m.e[c / 3][c % 3] = mk(src[2 * c], src[2 * c + 1]);
-    if (far_from_su3(m)) *(volatile int*)args.far = 1;
+    if (far_from_su3(m)) {
+      *(volatile int*)args.far = 1;
+      if (args.far_host) *(volatile int*)args.far_host = 1;
+    }
     store_f64((double2*)args.links, mu, p, h, g.Vh, m);
   } else {
     float o[12];

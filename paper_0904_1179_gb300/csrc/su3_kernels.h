@@ -54,6 +54,7 @@ struct ConvArgs {
   void* links;
   int pairs;  // FP32 store in the site-paired layout
   int* far;   // SweepState's flag, set where the FP64 store takes a link far from SU(3)
+  int* far_host = nullptr;      // the same word for the host (page-locked)
   const int* status = nullptr;  // a batch's status word (device) and where the conversion from the store
   int* status_host = nullptr;   // copies it (page-locked); null: not copied
 };

@@ -33,6 +33,11 @@ struct su3_lattice {
   double* d_partials = nullptr;
   double* h_plaq = nullptr;               // page-locked; the kernel writes it (a copy costs 4 us more)
   unsigned long long* h_stats = nullptr;  // pinned, 2 words
+  // FP64 store, half-sweeps called one by one: whether its flags (SweepState) may be set -- links_set found a link far
+  // from SU(3) or a sweep timed out --, and the (mu, parity) run since they were last set or moved
+  int* h_far = nullptr;  // page-locked; written by the conversion of links_set
+  bool far_possible = false;
+  unsigned half_sweeps = 0;
   double* d_stage = nullptr;   // canonical-layout staging buffers (two, for the
   double* d_stage2 = nullptr;  // copy/convert pipeline of links_get/set)
   cudaStream_t copy_stream = nullptr;

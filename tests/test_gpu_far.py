@@ -49,3 +49,44 @@ def test_replicas_of_a_batch_are_independent(kind, tries):
             b.sweep(1)
             for lat in alone:
                 lat.sweep(1)
+
+
+PHASES = [(mu, parity) for mu in range(4) for parity in range(2)]
+
+
+@pytest.mark.parametrize("L,decomp", [((8, 4, 6, 4), None), ((16, 16, 16, 16), None), ((8, 4, 8, 4), (2, 2, 1))])
+def test_eight_half_sweeps_end_the_fp64_arithmetic(L, decomp):
+    # A chain driven by half-sweeps is the chain of sweeps, bit for bit: once all eight have rewritten the far link
+    # and its neighbours, it is back in the arithmetic of proper configurations.
+    far = with_far_link(L, 3, "stretched")
+    with su3.Lattice(L, 5.7, 5, decomp=decomp) as a, su3.Lattice(L, 5.7, 5, decomp=decomp) as b:
+        a.set_links(far)
+        b.set_links(far)
+        for t in range(3):
+            a.sweep(1)
+            for mu, parity in PHASES:
+                b.half_sweep(mu, parity)
+            b.sweep_count = t + 1
+            assert np.array_equal(a.get_links(), b.get_links()), t
+            assert a.plaquette() == b.plaquette()
+
+
+@pytest.mark.parametrize("decomp", [None, (2, 2, 1)])
+def test_half_sweeps_around_a_sweep_do_not_end_it(decomp):
+    # Four half-sweeps, a sweep, the other four: not all links were rewritten since the sweep found its NaN, which
+    # stays the only one.
+    L = (8, 4, 8, 4)
+    ref = oracle.hot_start(L, 3)
+    bad = with_far_link(L, 3, "nan")
+    with su3.Lattice(L, 5.7, 5, decomp=decomp) as lat:
+        lat.set_links(bad)
+        for mu, parity in PHASES[:4]:
+            lat.half_sweep(mu, parity)
+        lat.sweep(1)
+        for mu, parity in PHASES[4:] + PHASES:
+            lat.half_sweep(mu, parity)
+        u = lat.get_links()
+    lost = np.isnan(u).any(axis=(-1, -2, -3))
+    assert lost.sum() == 1 and lost[0, 1, 1, 0, 2]
+    # the plaquettes of the lost link hold links whose staples were no numbers: they have never changed
+    assert np.abs(u - ref)[0, 1, 1, 0, 0].max() <= 1e-12
