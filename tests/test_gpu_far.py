@@ -90,3 +90,39 @@ def test_half_sweeps_around_a_sweep_do_not_end_it(decomp):
     assert lost.sum() == 1 and lost[0, 1, 1, 0, 2]
     # the plaquettes of the lost link hold links whose staples were no numbers: they have never changed
     assert np.abs(u - ref)[0, 1, 1, 0, 0].max() <= 1e-12
+
+
+@pytest.mark.parametrize("kind", ["stretched", "nan"])
+@pytest.mark.parametrize("tries", [1, 4])
+@pytest.mark.parametrize("L,threads", [((8, 8, 4, 4), 32), ((16, 16, 16, 8), 128)])
+def test_every_kernel_holds_the_same_update(kind, tries, L, threads):
+    # One thread per link in eight launches, against four and the automatic number of lanes, the per-direction and the
+    # chained launches and the measuring sweep: the same links, bit for bit, and the plaquettes of each sweep.
+    far = with_far_link(L, 6, kind)
+
+    def lattice():
+        lat = su3.Lattice(L, 5.7, 5)
+        lat.set_heatbath(tries)
+        lat.set_links(far)
+        return lat
+
+    with lattice() as lat:
+        lat.set_lanes(1)
+        lat.set_schedule(su3.SU3_SCHED_PHASES)
+        plaquettes = []
+        for _ in range(2):
+            lat.sweep(1)
+            plaquettes.append(su3.load_library().su3_plaquette(lat.handle))
+        want = lat.get_links()
+    for lanes, schedule in ((4, None), (0, None), (1, su3.SU3_SCHED_PER_DIRECTION), (1, su3.SU3_SCHED_CHAINED)):
+        with lattice() as lat:
+            lat.set_lanes(lanes)
+            if schedule is not None:
+                lat.set_block_size(threads)
+                lat.set_schedule(schedule)
+            lat.sweep(2)
+            assert np.array_equal(lat.get_links(), want, equal_nan=True), (lanes, schedule)
+    with lattice() as lat:
+        measured = lat.sweep_measured(2)
+        assert np.array_equal(lat.get_links(), want, equal_nan=True)
+    np.testing.assert_allclose(measured, plaquettes, rtol=0, atol=1e-13)  # the bound of the parity tests
