@@ -204,12 +204,6 @@ SU3_HD void cfx_mac(cfacc& s, const cfx& a, const cfx& b) {
   fx_mac(s.im, a.re, b.im);
   fx_mac(s.im, a.im, b.re);
 }
-SU3_HD void cfx_msub(cfacc& s, const cfx& a, const cfx& b) {
-  fx_msub(s.re, a.re, b.re);
-  fx_mac(s.re, a.im, b.im);
-  fx_msub(s.im, a.re, b.im);
-  fx_msub(s.im, a.im, b.re);
-}
 SU3_HD void cfx_mac_cb(cfacc& s, const cfx& a, const cfx& b) {
   fx_mac(s.re, a.re, b.re);
   fx_mac(s.re, a.im, b.im);

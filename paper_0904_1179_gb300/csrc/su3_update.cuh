@@ -32,27 +32,6 @@ __device__ __forceinline__ mat3<T> zero3() {
   return m;
 }
 
-// Link loader for the two storage forms.  CG = true reads through L2 only
-// (ld.global.cg): required where other thread blocks of the same launch have
-// written the links (the persistent batched sweep); otherwise the read-only
-// path (ld.global.nc) is used.
-template <typename T, bool CG>
-struct Store;
-
-template <bool CG>
-struct Store<double, CG> {
-  __device__ __forceinline__ static mat3<double> load(const void* U, int mu, int p, int h, int Vh) {
-    return load_f64<CG>((const double2*)U, mu, p, h, Vh);
-  }
-};
-
-template <bool CG>
-struct Store<float, CG> {
-  __device__ __forceinline__ static mat3<float> load(const void* U, int mu, int p, int h, int Vh) {
-    return load_f32<CG>((const float4*)U, mu, p, h, Vh);
-  }
-};
-
 // The FP32 stores come in two layouts: one site per float4 column group (the
 // single-site layout) and the site-paired layout of su3_sitepair.cuh, which
 // stores the sites x and x + (L3/2) e3 of a lattice whose L3 is a multiple of
@@ -117,38 +96,40 @@ __device__ __forceinline__ void store_pair_site(float4* U, int mu, int p, int h,
 // Each three-link path is an SU(3) matrix, so only its rows 0 and 1 are
 // multiplied out; its row 2, conj(row0 x row1), is formed inside the
 // accumulation of A's row 2 (acc_completed).  The paths are added in the
-// order forward, backward for nu ascending; every kernel that forms a staple
-// keeps this order, so their results agree bit for bit.
-// The two three-link paths of direction nu (nu != mu), rows 0,1:
+// order forward, backward for nu ascending; every floating-point kernel that
+// forms a staple keeps this order, so their results agree bit for bit.
+// The two three-link paths of direction nu (nu != mu), rows 0,1, in FP64
+// arithmetic (update_link_f64_far; links through L2, as other blocks of the
+// same launch may have written them):
 //   forward  F = U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+,
 //   backward B = U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu).
 // h_pmu is the half index of x + mu-hat.
-template <typename T, bool CG, typename G, typename S>
-__device__ __forceinline__ mat3<T> forward_path(const G& g, const void* U, const S& st, int h, int p, int mu, int nu,
-                                                int h_pmu, int h_pnu) {
+template <typename G>
+__device__ __forceinline__ mat3<double> forward_path(const G& g, const double2* U, int h, int p, int mu, int nu, int h_pmu,
+                                                     int h_pnu) {
   const int q = p ^ 1;
-  const mat3<T> a = Store<T, CG>::load(U, nu, q, h_pmu, g.Vh);  // U_nu(x+mu)
-  const mat3<T> b = Store<T, CG>::load(U, mu, q, h_pnu, g.Vh);  // U_mu(x+nu)
-  mat3<T> t;
+  const mat3<double> a = load_f64<true>(U, nu, q, h_pmu, g.Vh);  // U_nu(x+mu)
+  const mat3<double> b = load_f64<true>(U, mu, q, h_pnu, g.Vh);  // U_mu(x+nu)
+  mat3<double> t;
   mul_nd_rows01(a, b, t);
-  const mat3<T> c = Store<T, CG>::load(U, nu, p, h, g.Vh);  // U_nu(x)
-  mat3<T> f;
+  const mat3<double> c = load_f64<true>(U, nu, p, h, g.Vh);  // U_nu(x)
+  mat3<double> f;
   mul_nd_rows01(t, c, f);
   return f;
 }
 
-template <typename T, bool CG, typename G>
-__device__ __forceinline__ mat3<T> backward_path(const G& g, const void* U, int p, int mu, int nu, int h_mnu,
-                                                 int h_pmu_mnu) {
+template <typename G>
+__device__ __forceinline__ mat3<double> backward_path(const G& g, const double2* U, int p, int mu, int nu, int h_mnu,
+                                                      int h_pmu_mnu) {
   const int q = p ^ 1;
-  const mat3<T> d = Store<T, CG>::load(U, nu, p, h_pmu_mnu, g.Vh);  // U_nu(x+mu-nu)
-  const mat3<T> e = Store<T, CG>::load(U, mu, q, h_mnu, g.Vh);      // U_mu(x-nu)
+  const mat3<double> d = load_f64<true>(U, nu, p, h_pmu_mnu, g.Vh);  // U_nu(x+mu-nu)
+  const mat3<double> e = load_f64<true>(U, mu, q, h_mnu, g.Vh);      // U_mu(x-nu)
   // Rows 0,1 of d^+ e^+ = (e d)^+ are the conjugated columns 0,1 of e d, which
   // need all three rows of e (stored in full here) but no row-2 completion.
-  mat3<T> hm;
+  mat3<double> hm;
   mul_nn_cols01(e, d, hm);
-  const mat3<T> f = Store<T, CG>::load(U, nu, q, h_mnu, g.Vh);  // U_nu(x-nu)
-  mat3<T> b;
+  const mat3<double> f = load_f64<true>(U, nu, q, h_mnu, g.Vh);  // U_nu(x-nu)
+  mat3<double> b;
   mul_dn_rows01(hm, f, b);
   return b;
 }
@@ -271,8 +252,8 @@ __device__ __noinline__ UpdateCount update_link_f64_far(const G& g, double2* U, 
 #pragma unroll 1
   for (int nu = 0; nu < 4; ++nu) {
     if (nu == mu) continue;
-    acc_completed(A, forward_path<double, true>(g, U, st, h, p, mu, nu, h_pmu, nb_half_rt(g, st, nu, +1)));
-    acc_completed(A, backward_path<double, true>(g, U, p, mu, nu, nb_half_rt(g, st, nu, -1), nb_half2_rt(g, st, mu, nu)));
+    acc_completed(A, forward_path(g, U, h, p, mu, nu, h_pmu, nb_half_rt(g, st, nu, +1)));
+    acc_completed(A, backward_path(g, U, p, mu, nu, nb_half_rt(g, st, nu, -1), nb_half2_rt(g, st, mu, nu)));
     if (nu == mu - 1) Apart = A;
   }
   UpdateCount cnt{0, 0};
