@@ -69,10 +69,6 @@ int cuda_fail(cudaError_t e, const char* what) { return su3_cuda_fail(e, what); 
 
 constexpr int kDefaultThreads = kSu3DefaultThreads;
 
-// Default block size for a half-sweep of Vh links: 128 threads, fewer (down
-// to one warp) when that would leave SMs idle, so that a small lattice's
-// links spread over as many SMs as there are warps (each link's update is a
-// long serial chain, and on the FP64 pipe a few warps saturate an SM).
 int sm_count() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -107,13 +103,11 @@ bool pairs_single(int Vh) {
 
 // Lanes per link of an FP64 half-sweep launched by itself
 // (k_half_sweep_f64_lanes), by the warps per SM they make.  GB300, ms per sweep
-// with 1 / 4 / 8 lanes: 4^4 0.193 / 0.088 / 0.074, 6^4 0.193 / 0.090 / 0.076, 8^4
+// with 1 / 4 / 8 lanes: 4^4 0.191 / 0.088 / 0.074, 6^4 0.191 / 0.090 / 0.076, 8^4
 // (3.4 warps per SM at eight lanes) 0.195 / 0.092 / 0.086, 8^3 x 16 (6.7 at eight,
-// 3.4 at four) 0.199 / 0.103 / 0.133, 10^4 0.200 / 0.123 / 0.151, 12^4 (8.5 at four)
-// 0.202 / 0.162 / 0.214, 14^4 (15.8) 0.203 / 0.228 / 0.332, 16^4 0.268 / 0.363 /
-// 0.555 (the eight-lane figures from 8^3 x 16 on are of the kernel before its
-// loads went through shared memory): eight lanes up to four warps per SM (one per
-// scheduler), four up to ten.
+// 3.4 at four) 0.199 / 0.102 / 0.109, 10^4 0.201 / 0.123 / 0.135, 12^4 (8.5 at four)
+// 0.201 / 0.162 / 0.214, 14^4 (15.8) 0.201 / 0.228 / 0.328, 16^4 0.266 / 0.364 /
+// 0.570: eight lanes up to four warps per SM (one per scheduler), four up to ten.
 int f64_lanes_auto(int Vh) {
   const int sms = sm_count();
   if (sms <= 0) return 1;
@@ -121,6 +115,10 @@ int f64_lanes_auto(int Vh) {
   return 4LL * Vh <= 10 * 32LL * sms ? 4 : 1;
 }
 
+// Default block size for a half-sweep of Vh links: 128 threads, fewer (down
+// to one warp) when that would leave SMs idle, so that a small lattice's
+// links spread over as many SMs as there are warps (each link's update is a
+// long serial chain).
 int default_threads(int Vh) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -173,7 +171,6 @@ void release(su3_lattice* h) {
   if (h->copy_stream) cudaStreamDestroy(h->copy_stream);
   cudaFreeHost(h->h_plaq);
   cudaFreeHost(h->h_stats);
-  cudaFreeHost(h->h_far);
   if (h->own_stream && h->stream) cudaStreamDestroy(h->stream);
   delete h;
 }
@@ -602,13 +599,14 @@ int su3_create_ex(int L0, int L1, int L2, int L3, double beta, uint64_t seed, in
       (e = cudaMalloc(&h->d_partials, (size_t)nparts * sizeof(double))) != cudaSuccess ||
       (e = cudaMalloc(&h->d_stage, (size_t)chunk * 4 * 18 * sizeof(double))) != cudaSuccess ||
       (e = cudaMallocHost(&h->h_plaq, sizeof(double))) != cudaSuccess ||
-      (e = cudaMallocHost(&h->h_stats, 2 * sizeof(unsigned long long))) != cudaSuccess ||
-      (e = cudaMallocHost(&h->h_far, sizeof(int))) != cudaSuccess) {
+      (e = cudaMallocHost(&h->h_stats, 3 * sizeof(unsigned long long))) != cudaSuccess) {
     const int rc = cuda_fail(e, "su3_create: allocation");
     cudaGetLastError();
     release(h);
     return rc;
   }
+  h->h_far = (int*)(h->h_stats + 2);
+  *h->h_far = 0;
   int rc = SU3_OK;
   if ((e = cudaMemsetAsync(h->d_sweep, 0, sizeof(su3dev::SweepState), h->stream)) != cudaSuccess ||
       (e = cudaMemsetAsync(h->d_stats, 0, 2 * sizeof(unsigned long long), h->stream)) != cudaSuccess) {

@@ -32,7 +32,7 @@ struct su3_lattice {
   bool stats_on = false;
   double* d_partials = nullptr;
   double* h_plaq = nullptr;               // page-locked; the kernel writes it (a copy costs 4 us more)
-  unsigned long long* h_stats = nullptr;  // pinned, 2 words
+  unsigned long long* h_stats = nullptr;  // pinned, 2 words; h_far's after them
   // FP64 store, half-sweeps called one by one: whether its flags (SweepState) may be set -- links_set found a link far
   // from SU(3) or a sweep timed out --, and the (mu, parity) run since they were last set or moved
   int* h_far = nullptr;  // page-locked; written by the conversion of links_set
