@@ -82,9 +82,11 @@ enum {
 /* Create a lattice of extents L0..L3 at coupling beta with the given Philox
  * seed and start (SU3_COLD: every link the identity; SU3_HOT: Haar-random
  * SU(3) links drawn from Philox tag 1).  Precision SU3_FP64 stores 18 reals
- * per link in FP64 and computes to FP64 accuracy: the update works in fixed
- * point of 62 fraction bits on the integer and FP32 units, closer to the exact
- * result than FP64 arithmetic (see su3_links_set for links far from SU(3)).
+ * per link in FP64 and computes to FP64 accuracy: the update works on the
+ * integer and FP32 units with numbers held to 2^-56 (absolute, not of
+ * themselves); the links it leaves are on average 0.4 to 0.8 units of 2^-53
+ * from the exact update for beta up to 5000 (3 at 1e6), where FP64 arithmetic
+ * left 1 to 25 (360).  See su3_links_set for links far from SU(3).
  * On success *out receives the handle. */
 SU3_API int su3_create(int L0, int L1, int L2, int L3, double beta, uint64_t seed, int start, su3_handle* out);
 
@@ -149,8 +151,10 @@ SU3_API double su3_plaquette(su3_handle h);
  * row 2 as conj(row0 x row1), which holds for products of SU(3) matrices
  * only.  set does not check; every update reunitarises the link it writes
  * (a link far from unitary, |row|^2 - 1 or <row0,row1> beyond 1e-3, takes a
- * full FP64 Gram-Schmidt in the FP32 paths; while an FP64 store may hold a link
- * far from SU(3), its sweeps run in FP64 arithmetic, several times slower). */
+ * full FP64 Gram-Schmidt in the FP32 paths; while an FP64 store, or a replica of
+ * an FP64 batch, may hold a link far from SU(3), it is swept in FP64 arithmetic,
+ * several times slower: until a sweep, or all eight half-sweeps, have rewritten
+ * every link and left none that is, NaN for example). */
 SU3_API int su3_links_get(su3_handle h, double* host, size_t n_doubles);
 SU3_API int su3_links_set(su3_handle h, const double* host, size_t n_doubles);
 
@@ -248,7 +252,9 @@ SU3_API int su3_set_schedule(su3_handle h, int schedule);
 
 /* The schedule the next sweep runs with (SU3_SCHED_PHASES,
  * SU3_SCHED_PERSISTENT, SU3_SCHED_PER_DIRECTION or SU3_SCHED_CHAINED) into
- * *schedule. */
+ * *schedule.  Under SU3_SCHED_AUTO this may be a schedule in tiles smaller than
+ * the block size (su3_set_block_size), which su3_set_schedule does not take at
+ * the default block size: to go back to it, set SU3_SCHED_AUTO. */
 SU3_API int su3_get_schedule(su3_handle h, int* schedule);
 
 /* Fault-detection hook of the persistent sweep (single lattices), as

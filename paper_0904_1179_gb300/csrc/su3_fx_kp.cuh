@@ -10,8 +10,10 @@
 // look up 1/2048 of an octave or 1/4096 of a turn, and need three terms of a
 // series on what is left, of which only the first two exceed FP32.  Square
 // roots start from the hardware's FP32 reciprocal root and take one step of
-// third order.  Errors are absolute and below 2^-54 of numbers up to 1 (tests:
-// against long double, next to the FP64 form).
+// third order.  Errors are absolute; the largest measured against long double over
+// 200,000 draws, in units of 2^-53 of numbers up to 1: logarithm 1.13 (of up to 37),
+// cosine and sine 1.49, root 1.23; root mean squares here / in FP64: direction
+// 0.27 / 0.37, a0 0.27 / 0.42, a1 to a3 0.24 / 1.33.
 //
 // 64-bit integers named x62 hold x in units of 2^-62.
 #pragma once

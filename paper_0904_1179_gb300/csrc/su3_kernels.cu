@@ -3,7 +3,7 @@
 // One thread updates one link U_mu(x) of the half-sweep (mu, parity): it
 // gathers the six-staple sum from the 18 neighbouring links, runs the one-hit
 // Kennedy-Pendleton heatbath in the SU(2) subgroups (0,1), (0,2), (1,2)
-// (Cabibbo-Marinari), reunitarises in FP64 and stores the link.  Links of one
+// (Cabibbo-Marinari), reunitarises and stores the link.  Links of one
 // (mu, parity) never enter each other's staples (checkerboard updating,
 // Abstract and Sec. 1 of Berg & Wu, arXiv:0904.1179), so threads are
 // independent; the counter-based Philox stream makes the result independent of
@@ -24,8 +24,11 @@ using namespace su3dev;
 // per SM), every block size up to kMaxSweepThreads legal.  Two blocks of 256
 // (126 registers, no spills) instead of four (64 registers): GB300, ms per sweep,
 // mixed and EFT: 18 x 10 x 14 x 22 0.0698 -> 0.0596 and 0.0593 -> 0.0475 (few
-// warps: more loads in flight each), 30^4 0.403 -> 0.402 and 0.385 -> 0.356, 42^4
-// 1.368 -> 1.370 and 1.324 -> 1.244.
+// warps: more loads in flight each), 30^4 0.4019 -> 0.4026 and 0.385 -> 0.356, 42^4
+// 1.3681 -> 1.3694 and 1.324 -> 1.244; mixed 26^4 0.242 -> 0.229, 36^3 x 30 0.653 ->
+// 0.648, 50^4 2.703 -> 2.692, but 42 x 30 x 44 x 22 0.5744 -> 0.5758: EFT gains
+// throughout, mixed up to about 0.25 % less on large lattices of some shapes and up
+// to 5 % more on others, which no rule on the size tells apart.
 #ifndef SU3_F32_LB_THREADS
 #define SU3_F32_LB_THREADS kMaxSweepThreads
 #endif
@@ -38,9 +41,9 @@ namespace {
 // ---------------------------------------------------------------------------
 // Single-lattice half-sweeps: one thread per link of (mu, parity).
 // ---------------------------------------------------------------------------
-// The same four-lane split for FP32 storage: rows 0,1 of the staple paths on
-// row pairs (12 floats each) are gathered into lane 0 and added in the
-// single-thread order, and the random numbers of the three subgroups are drawn
+// Four lanes per link for FP32 storage (small lattices): lanes 0-2 form the two
+// paths of one direction each; rows 0,1 of the paths on row pairs (12 floats
+// each) are gathered into lane 0 and added in the single-thread order, and the random numbers of the three subgroups are drawn
 // side by side; no register cap (small lattices leave the SMs nearly empty).
 __device__ __forceinline__ pm3 shfl_pm3_rows01(const pm3& m, int src) {
   pm3 r;

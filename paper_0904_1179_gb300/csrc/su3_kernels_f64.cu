@@ -10,10 +10,11 @@
 // 5.15; the scalars of the proposals there too (su3_fx_kp.cuh) and the subgroups
 // in one loop (instruction fetch had become the largest stall) 3.90; the staple's
 // links copied ahead into shared memory and no spills 3.35; neighbour steps
-// looked up and row pairs on the paired FMA 3.20.  Now 17,100 instructions per
-// warp at 0.57 issued per cycle and scheduler; what holds the rest are
-// fixed-latency dependencies (1.2 of 5.1 cycles per instruction) and the shared
-// integer pipe (0.7) at three warps per scheduler, which 168 registers allow.
+// looked up and row pairs on the paired FMA 3.20.  Now 16,700 instructions per
+// warp at 0.56 issued per cycle and scheduler; what holds the rest are
+// fixed-latency dependencies (1.1 of 5.2 cycles per instruction), the shared
+// integer pipe (0.7), dispatch (0.6) and instruction fetch (0.5) at three warps
+// per scheduler, which 168 registers allow.
 // DRAM moves at a quarter of its rate.
 #include "su3_kernels.h"
 
@@ -28,6 +29,9 @@ using namespace su3dev;
 // Registers per thread.  GB300, ms per sweep of 32^4 / 24^4 in eight launches: 128
 // registers 3.61 / 1.267, 136: 3.32 / 1.149, 144: 3.45 / 1.171, 168: 3.20 / 1.120.
 // 168 is the most that keeps 12 warps on an SM; blocks of 256 threads stay legal.
+// Spilled at 168, bytes stored: nothing in the one-hit forms of one, four and eight lanes and
+// of the per-direction launches, 16 in the chained one; 40, 52 and 36 in the repeat forms of
+// one lane, per direction and chained; 156 and 224 in the measuring forms.
 #ifndef SU3_F64_REGS
 #define SU3_F64_REGS 168
 #endif
@@ -214,7 +218,7 @@ cudaError_t su3k_launch_plaquette_f64(const PlaqArgs& a, const int* far, double*
   return cudaGetLastError();
 }
 
-// The ring takes up to 100 KB of dynamic shared memory (256 threads).
+// The ring takes up to 108 KiB of dynamic shared memory (256 threads of 432 B).
 cudaError_t su3k_prepare_f64() {
   const void* const k[] = {(const void*)k_half_sweep_f64<false, false>, (const void*)k_half_sweep_f64<true, false>,
                            (const void*)k_half_sweep_f64<false, true>,  (const void*)k_half_sweep_f64<true, true>,

@@ -8,8 +8,11 @@
 // partial sum per thread block -- lives in a fixed file-scope device array
 // instead of a handle's cudaMalloc'd buffer.
 // Every GPU that loads libsu3 holds this array (512 KiB) until the process
-// exits.  The kernels are the library's plaquette kernels (su3_kernels.cu),
-// launched with that array as their partial-sum buffer.
+// exits.  The kernels are those of su3_kernels.cu, launched with that array as
+// their partial-sum buffer: for FP32 stores su3_plaquette's own; for FP64 stores one
+// thread per site in FP64 arithmetic (a store that no handle owns has no flag of
+// links far from SU(3)), where su3_plaquette uses k_plaquette_fx: the two agree to
+// rounding, not bit for bit.
 #include <cuda.h>
 
 #include <cstdio>
