@@ -5,6 +5,8 @@
 // conversion and the instantiated CUDA graphs of one sweep.  The timing
 // programs of Berg & Wu (Sec. 2) run `nequi` sweeps with nothing else in the
 // loop; su3_sweep replays a graph of the eight half-sweeps for each of them.
+#include <cuda.h>
+
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -447,25 +449,44 @@ int ensure_transfer(su3_lattice* h, const char* what) {
 
 }  // namespace
 
-// The GPU's address of a host buffer that a kernel may write, or null: both ends
-// in page-locked memory, not registered read-only, on a GPU that shares the
-// host's page tables (so that no address between them can fault), 16-byte aligned.
-static double* host_direct(double* host, size_t bytes) {
-  int dev = 0, shared_tables = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&shared_tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev) != cudaSuccess) {
+// The GPU's address of a host buffer that a kernel may write, or null: all of it in
+// one page-locked allocation or registration (between two lie pages that the GPU may
+// not write or that nobody mapped), not registered read-only, on a GPU that shares
+// the host's page tables, 16-byte aligned.  (The driver call is resolved through the
+// runtime, so that libsu3 does not link the driver library.)
+static double* host_direct(su3_lattice* h, double* host, size_t bytes) {
+  typedef CUresult (*AttributesFn)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+  static const AttributesFn attributes = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool found = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) ==
+                           cudaSuccess &&
+                       q == cudaDriverEntryPointSuccess;
+    return found ? (AttributesFn)f : (AttributesFn) nullptr;
+  }();
+  if (h->shared_tables < 0) {  // of the handle's GPU: asked once
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&h->shared_tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+  }
+  unsigned flags = 0;
+  if (!attributes || !h->shared_tables || ((uintptr_t)host & 15)) return nullptr;
+  if (cudaHostGetFlags(&flags, host) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;
   }
-  if (!shared_tables || ((uintptr_t)host & 15)) return nullptr;
-  void* d = nullptr;
-  unsigned first = 0, last = 0;
-  if (cudaHostGetFlags(&first, host) != cudaSuccess || cudaHostGetFlags(&last, (char*)host + bytes - 1) != cudaSuccess ||
-      cudaHostGetDevicePointer(&d, host, 0) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  return (first | last) & cudaHostRegisterReadOnly ? nullptr : (double*)d;
+  if (flags & cudaHostRegisterReadOnly) return nullptr;
+  CUpointer_attribute what[3] = {CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE,
+                                 CU_POINTER_ATTRIBUTE_DEVICE_POINTER};
+  CUdeviceptr start = 0, device = 0;
+  size_t size = 0;
+  void* data[3] = {&start, &size, &device};
+  if (attributes(3, what, data, (CUdeviceptr)host) != CUDA_SUCCESS || start == 0 || (CUdeviceptr)host < start) return nullptr;
+  const size_t before = (size_t)((CUdeviceptr)host - start);
+  return before <= size && bytes <= size - before ? (double*)device : nullptr;
 }
 
 int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pairs, int* far, double* host, bool get,
@@ -474,7 +495,7 @@ int su3_transfer(su3_lattice* h, const su3dev::Geometry& g, void* links, bool pa
   // Page-locked memory: the conversion writes the caller's buffer itself, one launch of any size.  GB300, get through
   // the staging buffer / directly: 4^4 18 / 14 us, 8^4 30 / 26 us (FP32 38 / 28), 16^4 222 / 210 us (FP32 246 / 215),
   // 32^4 3.18 / 3.14 ms, 48^4 15.98 / 15.82 ms (the host link's 193 GB/s: 3.13 and 15.8 ms).
-  if (double* direct = get ? host_direct(host, (size_t)V * 72 * sizeof(double)) : nullptr) {
+  if (double* direct = get ? host_direct(h, host, (size_t)V * 72 * sizeof(double)) : nullptr) {
     ConvArgs a{g, h->precision, 0, V, direct, links, pairs ? 1 : 0, far};
     a.status = status;
     a.status_host = status_host;

@@ -40,6 +40,7 @@ struct su3_lattice {
   unsigned half_sweeps = 0;
   double* d_stage = nullptr;   // canonical-layout staging buffers (two, for the
   double* d_stage2 = nullptr;  // copy/convert pipeline of links_get/set)
+  int shared_tables = -1;  // whether the GPU uses the host's page tables (links_get; -1: not asked yet)
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t ev_copied[2] = {nullptr, nullptr};
   cudaEvent_t ev_conv[2] = {nullptr, nullptr};
