@@ -71,31 +71,31 @@ def peaks():
 # stripped).  A line reports the figure only while that code still hashes the
 # same; otherwise its traffic is null and the line says why.
 _U_F64, _U_F32, _U_BATCH = ("su3_kernels_f64.cu",), ("su3_kernels.cu", "su3_kernels_pair.cu"), ("su3_batch.cu",)
-_SHA_F64 = "421c9b9264f9a448f02aad59cfa8d8ec77a989a86c13919d60855e554299e33e"
-_SHA_F32 = "0be1cf889a757d08dd8fd6f17162339f48bf1848e1adc616c5e1822dbba4e714"
-_SHA_BATCH = "1c7404eb60c41a3b311221e380604ebf20a4b945b17eaaca301da3ba42eb332a"
+_SHA_F64 = "209273350aa4dd0c1e6dfc66e1b5c6beb87992ef736c6477a67c678743c10e59"
+_SHA_F32 = "303fedb64d018eee27a2765b535ffce16ece8cc03fe4fe9e77ca8db521ab6582"
+_SHA_BATCH = "a3d08c29a8c9a58326c08ae965f86a5d84f0e0c037a90d4e27bf8db68424f7f9"
 _NCU_METRICS = "ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum --clock-control none"
 NCU_TRAFFIC = {
     # one launch of the default 32^4 FP32 sweep = one chained half-sweep; the mean of the eight launches of
     # the second sweep
-    "fp32_mixed": {"bytes": 209017952 + 13074368, "units": _U_F32, "sources_sha256": _SHA_F32,
+    "fp32_mixed": {"bytes": 208923328 + 12901856, "units": _U_F32, "sources_sha256": _SHA_F32,
                    "capture": _NCU_METRICS + " -k regex:k_half_sweep_f32_chain -s 8 -c 8 python bench.py --profile "
                                              "fp32_mixed"},
-    "fp32_eft": {"bytes": 208964224 + 13374976, "units": _U_F32, "sources_sha256": _SHA_F32,
+    "fp32_eft": {"bytes": 208916416 + 13243360, "units": _U_F32, "sources_sha256": _SHA_F32,
                  "capture": _NCU_METRICS + " -k regex:k_half_sweep_f32_chain -s 8 -c 8 python bench.py --profile "
                                            "fp32_eft"},
-    "fp32_mixed_phases": {"bytes": 207773440 + 15260928, "units": _U_F32, "sources_sha256": _SHA_F32,
+    "fp32_mixed_phases": {"bytes": 207800832 + 15122944, "units": _U_F32, "sources_sha256": _SHA_F32,
                           "capture": _NCU_METRICS + " -k regex:k_half_sweep -s 8 -c 1 python bench.py --profile "
                                                     "fp32_mixed_phases"},
-    "fp32_eft_phases": {"bytes": 207864064 + 15980800, "units": _U_F32, "sources_sha256": _SHA_F32,
+    "fp32_eft_phases": {"bytes": 207935488 + 15894784, "units": _U_F32, "sources_sha256": _SHA_F32,
                         "capture": _NCU_METRICS + " -k regex:k_half_sweep -s 8 -c 1 python bench.py --profile "
                                                   "fp32_eft_phases"},
-    "fp64": {"bytes": 626610176 + 70885120, "units": _U_F64, "sources_sha256": _SHA_F64,
+    "fp64": {"bytes": 625988608 + 70800384, "units": _U_F64, "sources_sha256": _SHA_F64,
              "capture": _NCU_METRICS + " -k regex:k_half_sweep -s 8 -c 1 python bench.py --profile fp64"},
-    "batched": {"bytes": 2834974976 + 442795776, "units": _U_BATCH, "sources_sha256": _SHA_BATCH,
+    "batched": {"bytes": 2826466816 + 441094656, "units": _U_BATCH, "sources_sha256": _SHA_BATCH,
                 "capture": _NCU_METRICS + " -k regex:k_batch_sweep -s 4 -c 4 python bench.py --profile batched "
                                           "(the four launches of the second sweep, summed)"},
-    "batched_eft": {"bytes": 2828132608 + 442020352, "units": _U_BATCH, "sources_sha256": _SHA_BATCH,
+    "batched_eft": {"bytes": 2830712576 + 442390528, "units": _U_BATCH, "sources_sha256": _SHA_BATCH,
                     "capture": _NCU_METRICS + " -k regex:k_batch_sweep -s 4 -c 4 python bench.py --profile batched_eft "
                                               "(the four launches of the second sweep, summed)"},
 }
