@@ -1031,12 +1031,12 @@ def main():
         "e2e": e2e,
         "gpu_launches": args.steps * SWEEPS_PER_STEP * 9,
         "gpu_launches_note": "headline timed region: per sweep 8 half-sweep kernels + 1 sweep-counter kernel",
-        # the kernel works on the integer and FP32 pipes, in fixed point; what limits it is instruction issue
+        # the kernel works on the integer and FP32 pipes, in fixed point; dependency latency and the integer pipe limit it
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                      "frac": achieved / hbm_peak, "peak_kind": peak_kind,
                      "traffic": traffic_of("fp64")[0], "traffic_source": traffic_of("fp64")[1],
                      "kernel": "k_half_sweep_f64", "bytes_per_launch": bytes_per_launch, "kernel_ms": kernel_ms,
-                     "limited_by": "instruction issue (integer and FP32 pipes), not DRAM"},
+                     "limited_by": "dependency latency and the integer pipe, not DRAM"},
         "cpu_baseline": cpu,
         "variants": variants,
     }
